@@ -171,6 +171,31 @@ k_relu_bwd_cast(const float* __restrict__ dy, int lddy, int dyoff, const __nv_bf
     }
 }
 
+// The two above in one pass, without the fp32 copy of dz: the masked gradient goes to bf16 and its fp32
+// values into the bias sums (V = 8, c / 8 divides 256, so a thread keeps its channels).  Memory bound: reads
+// 4 + 2 bytes and writes 2 per value, where the two passes read 4 + 2 + 4 and write 4 + 2.
+__global__ void __launch_bounds__(256)
+k_relu_bwd_bias(const float* __restrict__ dy, int lddy, int dyoff, const __nv_bfloat16* __restrict__ y, int ldy, int yoff,
+                int c, long long nvox, __nv_bfloat16* __restrict__ dzb, float* db) {
+    __shared__ float sh[8 * 256];
+    const int nc = c / 8, ch = (int)(threadIdx.x % nc) * 8, per = 256 / nc;
+    float acc[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc[q] = 0.f;
+    for (long long v = blockIdx.x * (long long)per + threadIdx.x / nc; v < nvox; v += (long long)gridDim.x * per) {
+        float g[8], m[8];
+        load_f<8>(dy + v * lddy + dyoff + ch, g);
+        load_bf<8>(y + v * ldy + yoff + ch, m);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            g[q] = m[q] > 0.f ? g[q] : 0.f;
+            acc[q] += g[q];
+        }
+        store_bf<8>(dzb + v * c + ch, g);
+    }
+    block_channel_sums<8>(acc, nc, sh, db);
+}
+
 // [27][Cout][Cin] -> [27][Cin][Cout]
 __global__ void k_wtranspose(const __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wt, int cout, int cin) {
     const long long n = 27LL * cout * cin;
@@ -257,7 +282,7 @@ k_upsample(const __nv_bfloat16* __restrict__ x, int c, __nv_bfloat16* __restrict
 template <int V, typename IX>
 __global__ void __launch_bounds__(256)
 k_upsample_bwd(const float* __restrict__ dy, int lddy, int dyoff, int c, float* __restrict__ dx, long long n, int D, int H,
-               int W) {
+               int W, int overwrite) {
     for (IX q = blockIdx.x * (IX)256 + threadIdx.x; q < (IX)n; q += (IX)gridDim.x * 256) {
         int ch;
         IX cv, fv;
@@ -271,10 +296,12 @@ k_upsample_bwd(const float* __restrict__ dy, int lddy, int dyoff, int c, float* 
 #pragma unroll
             for (int k = 0; k < V; ++k) s[k] += f[k];
         }
-        load_f<V>(dx + (long long)cv * c + ch, f);
+        if (!overwrite) {
+            load_f<V>(dx + (long long)cv * c + ch, f);
 #pragma unroll
-        for (int k = 0; k < V; ++k) f[k] += s[k];
-        store_f<V>(dx + (long long)cv * c + ch, f);
+            for (int k = 0; k < V; ++k) s[k] += f[k];
+        }
+        store_f<V>(dx + (long long)cv * c + ch, s);
     }
 }
 
@@ -517,13 +544,19 @@ pf_status pfnn_upsample(const void* x, int c, void* y, int ldy, int yoff, int n,
     return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
 }
 
-pf_status pfnn_upsample_bwd(const float* dy, int lddy, int dyoff, int c, float* dx, int n, int d, int h, int wd,
-                            void* stream) {
+static pf_status upsample_bwd(const float* dy, int lddy, int dyoff, int c, float* dx, int n, int d, int h, int wd,
+                              int overwrite, void* stream) {
     if (!dy || !dx) return PF_E_INVALID;
     const bool vec = vec_ok(4, {lddy, dyoff, c}, {dy, dx});
     const long long items = (long long)n * d * h * wd * c;
-    LAUNCH_VI(vec, 4, items, 8LL * n * d * h * wd, k_upsample_bwd, dy, lddy, dyoff, c, dx, items / (vec ? 4 : 1), 2 * d, 2 * h, 2 * wd);
+    LAUNCH_VI(vec, 4, items, 8LL * n * d * h * wd, k_upsample_bwd, dy, lddy, dyoff, c, dx, items / (vec ? 4 : 1), 2 * d, 2 * h,
+              2 * wd, overwrite);
     return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
+}
+
+pf_status pfnn_upsample_bwd(const float* dy, int lddy, int dyoff, int c, float* dx, int n, int d, int h, int wd,
+                            void* stream) {
+    return upsample_bwd(dy, lddy, dyoff, c, dx, n, d, h, wd, 0, stream);
 }
 
 pf_status pfnn_head_forward(const void* x, int c, const float* w, const float* b, const float* target, long long nvox,
@@ -573,3 +606,27 @@ pf_status pfnn_adam(float* p, const float* g, float* m, float* v, void* p_bf16, 
 }
 
 }  // extern "C"
+
+namespace pfgb {
+
+pf_status nn_upsample_bwd_set(const float* dy, int lddy, int dyoff, int c, float* dx, int n, int d, int h, int wd,
+                              void* stream) {
+    return upsample_bwd(dy, lddy, dyoff, c, dx, n, d, h, wd, 1, stream);
+}
+
+pf_status nn_relu_bwd_bias(const float* dy, int lddy, int dyoff, const void* y, int ldy, int yoff, int c, long long nvox,
+                           void* dz_bf16, float* db, void* stream) {
+    if (!dy || !y || !dz_bf16 || !db || !vec_ok(8, {lddy, dyoff, ldy, yoff, c}, {dy, y, dz_bf16}) || c > 2048 ||
+        256 % (c / 8))
+        return PF_E_INVALID;
+    // about four voxels per thread, at most eight blocks per SM
+    const long long per = 4LL * 256 / (c / 8);
+    long long b = (nvox + per - 1) / per;
+    if (b > 152 * 8) b = 152 * 8;
+    k_relu_bwd_bias<<<(unsigned)(b < 1 ? 1 : b), 256, 0, (cudaStream_t)stream>>>(dy, lddy, dyoff, (const bf16*)y, ldy, yoff,
+                                                                                c, nvox, (bf16*)dz_bf16, db);
+    count_launch();
+    return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
+}
+
+}  // namespace pfgb

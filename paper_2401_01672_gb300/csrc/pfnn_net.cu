@@ -22,6 +22,14 @@
 #include <string>
 #include <vector>
 
+namespace pfgb {
+// pfnn_conv.cu: dx = (not +=) the sum of the eight children; ReLU backward to bf16 with db[c] += its sums
+pf_status nn_upsample_bwd_set(const float* dy, int lddy, int dyoff, int c, float* dx, int n, int d, int h, int wd,
+                              void* stream);
+pf_status nn_relu_bwd_bias(const float* dy, int lddy, int dyoff, const void* y, int ldy, int yoff, int c, long long nvox,
+                           void* dz_bf16, float* db, void* stream);
+}  // namespace pfgb
+
 namespace {
 
 enum Buf { IN0, E1A, CAT1, P1, E2A, CAT2, P2, E3A, CAT3, P3, E4A, E4B, UP3, D3A, D3B, UP2, D2A, D2B, UP1, D1A, D1B, NBUF };
@@ -62,7 +70,6 @@ constexpr int NFEAT = 2;            // supercooling and surface-tension features
 struct Param {
     long long nw = 0, nb = 0;
     float *w = nullptr, *b = nullptr, *gw = nullptr, *gb = nullptr;
-    float *mw = nullptr, *vw = nullptr, *mb = nullptr, *vb = nullptr;
     void* wb = nullptr;   // bf16 working copy [27][cout][cin]
     void* wt = nullptr;   // bf16 transposed copy [27][cin][cout] (backward data)
 };
@@ -80,21 +87,81 @@ double normal(uint64_t& s) {
     return std::sqrt(-2.0 * std::log(u1)) * std::cos(6.283185307179586 * u2);
 }
 
-__global__ void k_f32_to_bf16(const float* __restrict__ in, __nv_bfloat16* __restrict__ out, long long n) {
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x)
-        out[q] = __float2bfloat16_rn(in[q]);
+// All parameters lie in one arena (and their gradients, moments, bf16 copies in others with the same
+// layout): segment 2q the weights, 2q + 1 the biases of parameter q, each starting on a multiple of SEG
+// elements, so the optimiser step is one launch (one block per SEG elements; 36 launches of a few blocks
+// each took 130 us) and the gradients are zeroed by one memset.
+constexpr int SEG = 1024, NSEG = 2 * NPARAM;
+struct Segments {
+    int block0[NSEG + 1];         // first block of each segment
+    int n[NSEG];                  // elements
+    int cout[NSEG], cin[NSEG];    // convolution weights [27][cout][cin] (0: no bf16 copies)
+};
+
+// segment of this block (uniform)
+__device__ __forceinline__ int segment_of(const Segments& S) {
+    int s = 0;
+    while ((int)blockIdx.x >= S.block0[s + 1]) ++s;
+    return s;
+}
+
+// the bf16 working copy of one weight and its transposed copy [27][cin][cout] (backward data)
+__device__ __forceinline__ void store_copies(const Segments& S, int s, long long base, int e, float p,
+                                             __nv_bfloat16* wb, __nv_bfloat16* wt) {
+    const __nv_bfloat16 b = __float2bfloat16_rn(p);
+    const int ci = e % S.cin[s], r = e / S.cin[s], co = r % S.cout[s], t = r / S.cout[s];
+    wb[base + e] = b;
+    wt[base + ((long long)t * S.cin[s] + ci) * S.cout[s] + co] = b;
+}
+
+// Adam with bias correction on the FP32 master parameters (the arithmetic of pfnn_adam)
+__global__ void __launch_bounds__(256)
+k_adam_all(const __grid_constant__ Segments S, float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
+           float* __restrict__ v, __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ wt, float lr, float b1,
+           float b2, float eps, float c1, float c2) {
+    const int s = segment_of(S);
+    const long long base = (long long)S.block0[s] * SEG;
+    const int e0 = ((int)blockIdx.x - S.block0[s]) * SEG;
+#pragma unroll
+    for (int k = 0; k < SEG / 256; ++k) {
+        const int e = e0 + k * 256 + threadIdx.x;
+        if (e >= S.n[s]) break;
+        const long long q = base + e;
+        const float gq = g[q];
+        const float mq = b1 * m[q] + (1.f - b1) * gq;
+        const float vq = b2 * v[q] + (1.f - b2) * gq * gq;
+        m[q] = mq;
+        v[q] = vq;
+        const float pq = p[q] - lr * (mq * c1) / (sqrtf(vq * c2) + eps);
+        p[q] = pq;
+        if (S.cin[s]) store_copies(S, s, base, e, pq, wb, wt);
+    }
+}
+
+// the bf16 copies of every convolution weight (after the parameters were set)
+__global__ void __launch_bounds__(256)
+k_copies_all(const __grid_constant__ Segments S, const float* __restrict__ p, __nv_bfloat16* __restrict__ wb,
+             __nv_bfloat16* __restrict__ wt) {
+    const int s = segment_of(S);
+    if (!S.cin[s]) return;
+    const long long base = (long long)S.block0[s] * SEG;
+    const int e0 = ((int)blockIdx.x - S.block0[s]) * SEG;
+    for (int e = e0 + threadIdx.x; e < e0 + SEG && e < S.n[s]; e += 256) store_copies(S, s, base, e, p[base + e], wb, wt);
 }
 
 }  // namespace
 
 struct pfnn_net {
     Param p[NPARAM];
+    Segments seg{};
+    float *pw = nullptr, *pg = nullptr, *pm = nullptr, *pv = nullptr;   // arenas: parameters, gradients, moments
+    __nv_bfloat16 *pb = nullptr, *pt = nullptr;                         // bf16 copies, plain and transposed
     cudaStream_t stream = nullptr;
     int step = 0;
     int n = 0, S = 0;                      // batch and side of the allocated activation buffers
     void* act[NBUF] = {};                  // bf16 activations
     float* grad[NBUF] = {};                // fp32 gradients of the activations
-    float *dz_f = nullptr, *logit_grad = nullptr, *prob = nullptr;
+    float *logit_grad = nullptr, *prob = nullptr;
     void* dz_b = nullptr;
     void* wg_work = nullptr;               // scratch of the weight gradients
     long long wg_bytes = 0;
@@ -128,7 +195,7 @@ void free_acts(pfnn_net* net) {
         net->act[b] = nullptr;
         net->grad[b] = nullptr;
     }
-    net->dz_f = net->logit_grad = net->prob = nullptr;
+    net->logit_grad = net->prob = nullptr;
     net->dz_b = nullptr;
     net->wg_work = nullptr;
     net->wg_bytes = 0;
@@ -147,9 +214,16 @@ pf_status ensure_acts(pfnn_net* net, int n, int S) {
         if (cudaMemsetAsync(net->act[b], 0, 2 * cells, net->stream) != cudaSuccess)
             return nfail(net, PF_E_CUDA, "activation buffers");
     }
+    // the input's gradient is never formed: it reads as zero
+    if (cudaMemsetAsync(net->grad[IN0], 0, 4LL * n * S * S * S * kBufC[IN0], net->stream) != cudaSuccess)
+        return nfail(net, PF_E_CUDA, "gradient buffers");
     const long long nvox = (long long)n * S * S * S;
-    net->dz_f = (float*)nalloc(net->act_allocs, 4 * nvox * 128);
-    net->dz_b = nalloc(net->act_allocs, 2 * nvox * 128);
+    long long dz = 0;  // largest layer output
+    for (int q = 0; q < NCONV; ++q) {
+        const long long sd = S >> kLayers[q].lev, b = n * sd * sd * sd * kLayers[q].cout;
+        dz = b > dz ? b : dz;
+    }
+    net->dz_b = nalloc(net->act_allocs, 2 * dz);
     net->logit_grad = (float*)nalloc(net->act_allocs, 4 * nvox);
     net->prob = (float*)nalloc(net->act_allocs, 4 * nvox);
     long long wg = 0;
@@ -160,7 +234,7 @@ pf_status ensure_acts(pfnn_net* net, int n, int S) {
     }
     net->wg_work = nalloc(net->act_allocs, (size_t)wg);
     net->wg_bytes = wg;
-    if (!net->dz_f || !net->dz_b || !net->logit_grad || !net->prob || !net->wg_work)
+    if (!net->dz_b || !net->logit_grad || !net->prob || !net->wg_work)
         return nfail(net, PF_E_OOM, "work buffers");
     net->n = n;
     net->S = S;
@@ -239,43 +313,48 @@ pf_status pfnn_net_create(unsigned long long seed, void* stream, pfnn_net** out)
     pfnn_net* net = new pfnn_net();
     net->stream = (cudaStream_t)stream;
     uint64_t rs = seed;
+    Segments& G = net->seg;
     for (int q = 0; q < NPARAM; ++q) {
         Param& P = net->p[q];
         const int cin = q < NCONV ? kLayers[q].cin : 16, cout = q < NCONV ? kLayers[q].cout : 1;
         P.nw = q < NCONV ? 27LL * cout * cin : 16;
         P.nb = cout;
-        float** f32s[] = {&P.w, &P.gw, &P.mw, &P.vw};
-        for (float** f : f32s) *f = (float*)nalloc(net->allocs, 4 * P.nw);
-        float** f32b[] = {&P.b, &P.gb, &P.mb, &P.vb};
-        for (float** f : f32b) *f = (float*)nalloc(net->allocs, 4 * P.nb);
-        if (q < NCONV) {
-            P.wb = nalloc(net->allocs, 2 * P.nw);
-            P.wt = nalloc(net->allocs, 2 * P.nw);
-        }
-        if (!P.w || !P.gw || !P.mw || !P.vw || !P.b || !P.gb || !P.mb || !P.vb || (q < NCONV && (!P.wb || !P.wt))) {
-            pfnn_net_destroy(net);
-            return PF_E_OOM;
-        }
-        // He-normal weights for the ReLU layers (std sqrt(2 / fan_in)), sqrt(1/16) for the head; zero biases
-        std::vector<float> w(P.nw), z(P.nb, 0.f);
-        const double sd = q < NCONV ? std::sqrt(2.0 / (27.0 * cin)) : std::sqrt(1.0 / 16.0);
-        for (long long k = 0; k < P.nw; ++k) w[k] = (float)(normal(rs) * sd);
-        cudaError_t e = cudaMemcpy(P.w, w.data(), 4 * P.nw, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(P.b, z.data(), 4 * P.nb, cudaMemcpyHostToDevice);
-        for (float* f : {P.gw, P.mw, P.vw})
-            if (e == cudaSuccess) e = cudaMemset(f, 0, 4 * P.nw);
-        for (float* f : {P.gb, P.mb, P.vb})
-            if (e == cudaSuccess) e = cudaMemset(f, 0, 4 * P.nb);
-        if (e == cudaSuccess && P.wb) {
-            k_f32_to_bf16<<<(unsigned)((P.nw + 255) / 256), 256>>>(P.w, (__nv_bfloat16*)P.wb, P.nw);
-            pfgb::count_launch();
-            e = cudaGetLastError();
-        }
-        if (e == cudaSuccess) e = cudaDeviceSynchronize();
-        if (e != cudaSuccess) {
-            pfnn_net_destroy(net);
-            return PF_E_CUDA;
-        }
+        G.n[2 * q] = (int)P.nw;
+        G.n[2 * q + 1] = (int)P.nb;
+        G.cin[2 * q] = q < NCONV ? cin : 0;
+        G.cout[2 * q] = q < NCONV ? cout : 0;
+    }
+    for (int k = 0; k < NSEG; ++k) G.block0[k + 1] = G.block0[k] + (G.n[k] + SEG - 1) / SEG;
+    const size_t total = (size_t)G.block0[NSEG] * SEG;
+    for (float** f : {&net->pw, &net->pg, &net->pm, &net->pv}) *f = (float*)nalloc(net->allocs, 4 * total);
+    for (__nv_bfloat16** f : {&net->pb, &net->pt}) *f = (__nv_bfloat16*)nalloc(net->allocs, 2 * total);
+    if (!net->pw || !net->pg || !net->pm || !net->pv || !net->pb || !net->pt) {
+        pfnn_net_destroy(net);
+        return PF_E_OOM;
+    }
+    // He-normal weights for the ReLU layers (std sqrt(2 / fan_in)), sqrt(1/16) for the head; zero biases
+    std::vector<float> w(total, 0.f);
+    for (int q = 0; q < NPARAM; ++q) {
+        Param& P = net->p[q];
+        const size_t ow = (size_t)G.block0[2 * q] * SEG, ob = (size_t)G.block0[2 * q + 1] * SEG;
+        P.w = net->pw + ow; P.gw = net->pg + ow;
+        P.b = net->pw + ob; P.gb = net->pg + ob;
+        if (q < NCONV) { P.wb = net->pb + ow; P.wt = net->pt + ow; }
+        const double sd = q < NCONV ? std::sqrt(2.0 / (27.0 * kLayers[q].cin)) : std::sqrt(1.0 / 16.0);
+        for (long long k = 0; k < P.nw; ++k) w[ow + k] = (float)(normal(rs) * sd);
+    }
+    cudaError_t e = cudaMemcpy(net->pw, w.data(), 4 * total, cudaMemcpyHostToDevice);
+    for (float* f : {net->pg, net->pm, net->pv})
+        if (e == cudaSuccess) e = cudaMemset(f, 0, 4 * total);
+    if (e == cudaSuccess) {
+        k_copies_all<<<G.block0[NSEG], 256>>>(G, net->pw, net->pb, net->pt);
+        pfgb::count_launch();
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) {
+        pfnn_net_destroy(net);
+        return PF_E_CUDA;
     }
     net->loss = (double*)nalloc(net->allocs, sizeof(double));
     if (!net->loss) {
@@ -294,7 +373,7 @@ pf_status pfnn_net_set_params(pfnn_net* net, int q, const float* w, const float*
         cudaMemcpyAsync(P.b, b, 4 * P.nb, cudaMemcpyHostToDevice, net->stream) != cudaSuccess)
         return nfail(net, PF_E_CUDA, "set_params");
     if (P.wb) {
-        k_f32_to_bf16<<<(unsigned)((P.nw + 255) / 256), 256, 0, net->stream>>>(P.w, (__nv_bfloat16*)P.wb, P.nw);
+        k_copies_all<<<net->seg.block0[NSEG], 256, 0, net->stream>>>(net->seg, net->pw, net->pb, net->pt);
         pfgb::count_launch();
     }
     if (cudaStreamSynchronize(net->stream) != cudaSuccess) return nfail(net, PF_E_CUDA, "set_params");
@@ -374,16 +453,11 @@ pf_status pfnn_net_backward(pfnn_net* net) {
     cudaStream_t s = net->stream;
     const int n = net->n, side = net->S;
     auto dims = [&](int lev, int* d) { const int sd = side >> lev; d[0] = n; d[1] = d[2] = d[3] = sd; };
-    for (int b = 0; b < NBUF; ++b) {
-        const long long sd = side >> kBufL[b];
-        if (cudaMemsetAsync(net->grad[b], 0, 4LL * n * sd * sd * sd * kBufC[b], s) != cudaSuccess)
-            return nfail(net, PF_E_CUDA, "zero gradients");
-    }
-    for (int q = 0; q < NPARAM; ++q) {
-        if (cudaMemsetAsync(net->p[q].gw, 0, 4 * net->p[q].nw, s) != cudaSuccess ||
-            cudaMemsetAsync(net->p[q].gb, 0, 4 * net->p[q].nb, s) != cudaSuccess)
-            return nfail(net, PF_E_CUDA, "zero gradients");
-    }
+    if (cudaMemsetAsync(net->pg, 0, 4 * (size_t)net->seg.block0[NSEG] * SEG, s) != cudaSuccess)
+        return nfail(net, PF_E_CUDA, "zero gradients");
+    // Every activation gradient is first written whole (the head's adjoint, a data gradient over all channels
+    // of the buffer, or an upsampling's adjoint) and only then added to (a pooling's adjoint into the encoder
+    // half of a skip buffer, whose decoder layer comes later in the forward order), so none is zeroed.
     const long long nvox0 = (long long)n * side * side * side;
     const Param& H = net->p[NCONV];
     NN_CK(net, pfnn_head_backward(net->act[D1B], 16, H.w, net->logit_grad, nvox0, net->grad[D1B], H.gw, H.gb, s),
@@ -396,15 +470,13 @@ pf_status pfnn_net_backward(pfnn_net* net) {
         const long long nvox = (long long)d[0] * d[1] * d[2] * d[3];
         const int ldy = kBufC[L.dst];
         // ReLU backward on this layer's output slice, then the three products of the convolution
-        NN_CK(net, pfnn_relu_bwd_cast(net->grad[L.dst], ldy, L.doff, net->act[L.dst], ldy, L.doff, L.cout, nvox,
-                                      net->dz_f, net->dz_b, s), "relu backward");
-        NN_CK(net, pfnn_bias_grad(net->dz_f, L.cout, 0, L.cout, nvox, P.gb, s), "bias gradient");
+        NN_CK(net, pfgb::nn_relu_bwd_bias(net->grad[L.dst], ldy, L.doff, net->act[L.dst], ldy, L.doff, L.cout, nvox,
+                                          net->dz_b, P.gb, s), "relu backward");
         NN_CK(net, pfnn_conv3d_wgrad(net->dz_b, L.cout, 0, L.cout, net->act[L.src], kBufC[L.src], L.soff, L.cin, P.gw,
                                      d[0], d[1], d[2], d[3], net->wg_work, net->wg_bytes, s), "weight gradient");
         if (L.src != IN0) {
-            NN_CK(net, pfnn_weight_transpose(P.wb, P.wt, L.cout, L.cin, s), "weight transpose");
             NN_CK(net, pfnn_conv3d(net->dz_b, L.cout, 0, P.wt, L.cout, L.cin, nullptr, 0, 1, nullptr, net->grad[L.src],
-                                   kBufC[L.src], L.soff, 1, d[0], d[1], d[2], d[3], s), "data gradient");
+                                   kBufC[L.src], L.soff, 0, d[0], d[1], d[2], d[3], s), "data gradient");
         }
         // adjoint of the data movement that produced this layer's input
         if (L.pre == 1) {
@@ -415,8 +487,8 @@ pf_status pfnn_net_backward(pfnn_net* net) {
         } else if (L.pre == 2) {
             int e[4];
             dims(L.pre_lev + 1, e);  // the coarse side
-            NN_CK(net, pfnn_upsample_bwd(net->grad[L.pre_dst], kBufC[L.pre_dst], 0, L.pre_c, net->grad[L.pre_src],
-                                         e[0], e[1], e[2], e[3], s), "upsample backward");
+            NN_CK(net, pfgb::nn_upsample_bwd_set(net->grad[L.pre_dst], kBufC[L.pre_dst], 0, L.pre_c,
+                                                 net->grad[L.pre_src], e[0], e[1], e[2], e[3], s), "upsample backward");
         }
     }
     return PF_OK;
@@ -425,11 +497,12 @@ pf_status pfnn_net_backward(pfnn_net* net) {
 pf_status pfnn_net_adam_step(pfnn_net* net, float lr, float b1, float b2, float eps) {
     if (!net || !(lr > 0.f)) return PF_E_INVALID;
     net->step += 1;
-    for (int q = 0; q < NPARAM; ++q) {
-        Param& P = net->p[q];
-        NN_CK(net, pfnn_adam(P.w, P.gw, P.mw, P.vw, P.wb, P.nw, lr, b1, b2, eps, net->step, net->stream), "adam");
-        NN_CK(net, pfnn_adam(P.b, P.gb, P.mb, P.vb, nullptr, P.nb, lr, b1, b2, eps, net->step, net->stream), "adam");
-    }
+    const float c1 = 1.f / (1.f - powf(b1, (float)net->step));
+    const float c2 = 1.f / (1.f - powf(b2, (float)net->step));
+    k_adam_all<<<net->seg.block0[NSEG], 256, 0, net->stream>>>(net->seg, net->pw, net->pg, net->pm, net->pv, net->pb,
+                                                               net->pt, lr, b1, b2, eps, c1, c2);
+    pfgb::count_launch();
+    if (cudaGetLastError() != cudaSuccess) return nfail(net, PF_E_CUDA, "adam failed");
     return PF_OK;
 }
 
