@@ -54,11 +54,11 @@ pf_status pfnn_status(int* failed);
 pf_status pfnn_test_withhold_stage(int stage, long long tries);
 
 /* Weight gradient: dw[t][co][ci] += sum_v dy[v][co] x[v + off(t)][ci], on the fifth-generation tensor cores:
- * dy and x are packed channel-major over the zero-padded grid (dy three times, shifted by dx = -1, 0, 1) in
- * the caller-owned device scratch `work` (16-byte aligned, at least pfnn_conv3d_wgrad_work_bytes bytes,
- * overwritten), then a GEMM over the packed voxels with rows (tap, co) -- 128 / cout taps per MMA tile --
- * and columns ci accumulates in TMEM; each CTA adds its voxel chunk's partial sums into dw with FP32
- * atomics.  cout in {16, 32, 64, 128}, cin a multiple of 16 up to 256. */
+ * a GEMM whose reduction runs over the voxels of 8 x 16-cell columns, both operands read as they lie in memory
+ * (channels last, by TMA); the tap's offset is a start address in the tile of x.  Each CTA adds the partial sums of
+ * its column into dw with FP32 atomics.  cout in {16, 32, 64, 128}, cin a multiple of 16 up to 256.  `work`: caller-
+ * owned device scratch, 16-byte aligned, at least pfnn_conv3d_wgrad_work_bytes bytes; operands whose rows do not
+ * start on 16 bytes (ld or off not a multiple of 8) are copied there first. */
 long long pfnn_conv3d_wgrad_work_bytes(int cout, int cin, int n, int d, int h, int wd);
 pf_status pfnn_conv3d_wgrad(const void* dy, int lddy, int dyoff, int cout, const void* x, int ldx, int xoff, int cin,
                             float* dw, int n, int d, int h, int wd, void* work, long long work_bytes, void* stream);

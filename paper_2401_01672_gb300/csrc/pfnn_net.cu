@@ -28,6 +28,9 @@ pf_status nn_upsample_bwd_set(const float* dy, int lddy, int dyoff, int c, float
                               void* stream);
 pf_status nn_relu_bwd_bias(const float* dy, int lddy, int dyoff, const void* y, int ldy, int yoff, int c, long long nvox,
                            void* dz_bf16, float* db, void* stream);
+// pfnn_umma.cu: pfnn_conv3d_wgrad of a compact dy and 16-byte aligned rows of x (no scratch needed)
+pf_status nn_wgrad(const void* dy, int cout, const void* x, int ldx, int xoff, int cin, float* dw, int n, int d, int h,
+                   int wd, void* stream);
 }  // namespace pfgb
 
 namespace {
@@ -163,8 +166,6 @@ struct pfnn_net {
     float* grad[NBUF] = {};                // fp32 gradients of the activations
     float *logit_grad = nullptr, *prob = nullptr;
     void* dz_b = nullptr;
-    void* wg_work = nullptr;               // scratch of the weight gradients
-    long long wg_bytes = 0;
     double* loss = nullptr;
     bool have_target = false;
     std::vector<void*> allocs, act_allocs;
@@ -197,8 +198,6 @@ void free_acts(pfnn_net* net) {
     }
     net->logit_grad = net->prob = nullptr;
     net->dz_b = nullptr;
-    net->wg_work = nullptr;
-    net->wg_bytes = 0;
     net->n = net->S = 0;
 }
 
@@ -226,15 +225,7 @@ pf_status ensure_acts(pfnn_net* net, int n, int S) {
     net->dz_b = nalloc(net->act_allocs, 2 * dz);
     net->logit_grad = (float*)nalloc(net->act_allocs, 4 * nvox);
     net->prob = (float*)nalloc(net->act_allocs, 4 * nvox);
-    long long wg = 0;
-    for (int q = 0; q < NCONV; ++q) {
-        const int sd = S >> kLayers[q].lev;
-        const long long b = pfnn_conv3d_wgrad_work_bytes(kLayers[q].cout, kLayers[q].cin, n, sd, sd, sd);
-        wg = b > wg ? b : wg;
-    }
-    net->wg_work = nalloc(net->act_allocs, (size_t)wg);
-    net->wg_bytes = wg;
-    if (!net->dz_b || !net->logit_grad || !net->prob || !net->wg_work)
+    if (!net->dz_b || !net->logit_grad || !net->prob)
         return nfail(net, PF_E_OOM, "work buffers");
     net->n = n;
     net->S = S;
@@ -472,8 +463,8 @@ pf_status pfnn_net_backward(pfnn_net* net) {
         // ReLU backward on this layer's output slice, then the three products of the convolution
         NN_CK(net, pfgb::nn_relu_bwd_bias(net->grad[L.dst], ldy, L.doff, net->act[L.dst], ldy, L.doff, L.cout, nvox,
                                           net->dz_b, P.gb, s), "relu backward");
-        NN_CK(net, pfnn_conv3d_wgrad(net->dz_b, L.cout, 0, L.cout, net->act[L.src], kBufC[L.src], L.soff, L.cin, P.gw,
-                                     d[0], d[1], d[2], d[3], net->wg_work, net->wg_bytes, s), "weight gradient");
+        NN_CK(net, pfgb::nn_wgrad(net->dz_b, L.cout, net->act[L.src], kBufC[L.src], L.soff, L.cin, P.gw, d[0], d[1], d[2],
+                                  d[3], s), "weight gradient");
         if (L.src != IN0) {
             NN_CK(net, pfnn_conv3d(net->dz_b, L.cout, 0, P.wt, L.cout, L.cin, nullptr, 0, 1, nullptr, net->grad[L.src],
                                    kBufC[L.src], L.soff, 0, d[0], d[1], d[2], d[3], s), "data gradient");

@@ -338,7 +338,7 @@ constexpr int HT_X = HB_X + 2, HT_Y = HB_Y + 2;
 constexpr unsigned HT_ROW = HT_X * 16;        // bytes of one tile row of 8 channels
 
 // unswizzled K-major descriptor: start, stride along K (LBO) and along M/N (SBO), version 1
-__device__ __forceinline__ uint64_t desc_plain(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+__host__ __device__ __forceinline__ uint64_t desc_plain(uint32_t addr, uint32_t lbo, uint32_t sbo) {
     return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ULL << 46);
 }
@@ -550,50 +550,69 @@ k_conv_halo(const __grid_constant__ CUtensorMap tmX, const HaloArgs p) {
 }
 
 // ---------------------------------------------------------------- weight gradient on tcgen05
-// dW[t][co][ci] = sum over voxels v of dY[v][co] X[v + off(t)][ci] (zero padding) is, with u = v + off(t),
-// sum over u of dY[u - off(t)][co] X[u][ci]: a GEMM whose reduction runs over voxels.  Both tensors are
-// first packed channel-major over a zero-padded grid (rows of W' = W + 2 rounded up to 8 cells, planes of
-// (H + 2) W', samples of (D + 2) planes), so that a tap's offset is a constant shift of the packed voxel
-// index; dY is packed three times, shifted by dx = -1, 0, +1, so that the remaining shift
-// dz (H + 2) W' + dy W' keeps the TMA coordinate a multiple of 8 elements (16 bytes).
-//   A (M = 128 rows): 128 / cout taps x cout output channels; tap j's rows are one TMA box of the dx-copy,
-//                     64 voxels wide, shifted by the tap's offset (out-of-range voxels filled with zeros);
-//   B (N = cin):      one TMA box of the packed X, 64 voxels wide;
-//   K:                the packed voxels of the CTA's chunk, 64 per pipeline stage (4 MMAs of K = 16).
-// Both operands are K-major with 128-byte rows (the 128-byte swizzle), as in k_conv_umma.  Each CTA adds
-// its chunk's partial products into dW with FP32 atomics (split over voxel chunks).
+// dW[t][co][ci] = sum over voxels v of dY[v][co] X[v + off(t)][ci] (zero padding): GEMMs whose reduction
+// runs over voxels, with both operands taken as they lie in memory.  A channels-last tile in shared memory
+// whose cells are 16-byte rows (8 channels of one voxel) is an MN-major operand without swizzle: eight
+// consecutive x cells are one core matrix (8 channels x 8 voxels of the reduction), so neither tensor is
+// transposed or packed first.  (Packing both channel-major, dY three times, and streaming one shifted box
+// per tap took 1.6 + 0.8 ms of a training step on 4 x 64^3 voxels and was bound by the 27 reads of dY from
+// L2.)
+//   A block marches along z over a column of 8 x 16 cells.  Per plane it loads dY (8 x 16, no halo, laid out
+//   [chunk of 8 channels][y][x]) and X (10 x 18 with the halo, [y][chunk][x]), each by one TMA box, zeros
+//   outside the grid, and keeps three planes of X, so every value is loaded once (and its halo).
+//   A (M) = X: core matrices along M are 160 bytes apart, which walks the chunks of a row of the tile and
+//   then the next row, so for 16 or 32 channels the three taps dy = -1, 0, +1 lie along M by themselves
+//   ("stacked": 6 of 8 or 12 of 16 core matrices used); 64 and 128 channels fill M = 64 or 128 with one tap.
+//   B (N) = dY, N = cout.  K = 16 voxels: two rows of 8 cells, 8 MMAs per tap and plane.  The taps dx and
+//   dz are other start addresses (16 bytes further, another plane).
+//   Accumulators: cout TMEM columns per tap (per three taps when stacked); where the 27 taps need more than
+//   512 columns they are divided over blocks by dz, then by dy (rule in wgrad_plan).
+// Shared-memory reads bound it for 16 and 32 channels (2.5 to 5 KB per MMA of N = 16 or 32).
 struct WgArgs {
-    int cout, cin, taps_per_tile;
-    int kb_per_cta;               // k blocks (of 64 packed voxels) per CTA
-    long long nkb;                // k blocks in total
-    int plane_p, row_p;           // packed plane and row lengths
-    int stages;
-    unsigned a_bytes, stage_bytes;
+    int cin, cout;
+    int cb, nchunk;               // input channels of a block (16, 32, 64 or 128), cb / 8
+    int stacked, ndz, ndy;        // taps dy along M; dz and (unstacked) dy accumulated by one block
+    int D, H, W, tx, ty;
+    int zc, nzc;                  // planes per block, blocks along z
+    int slots;
+    unsigned x_tx, dy_tx;         // bytes of the two boxes
+    unsigned x_bytes, slot_bytes; // their places in a slot
     unsigned idesc;
-    unsigned long long desc_hi;
+    unsigned long long a_hi, b_hi;  // descriptors without the start address
+    int m64;                      // MMA M = 64 (else 128)
     int tmem_cols;
     long long tries;
     float* dw;
 };
 
+constexpr unsigned WX_ROW = 10 * 16;  // bytes of one X tile row of one chunk
+
 __global__ void __launch_bounds__(UTHR)
-k_wgrad_umma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const WgArgs p) {
+k_wgrad_umma(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmY, const WgArgs p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char* sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    const int S = p.stages;
-    unsigned char* ctl = sm + (size_t)S * p.stage_bytes;
-    const uint32_t full0 = smem_u32(ctl);
-    const uint32_t empty0 = full0 + 8u * S;
-    const uint32_t accum = empty0 + 8u * S;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ctl + 16 * S + 8);
+    const int S = p.slots;
+    __shared__ __align__(8) unsigned long long s_bar[2 * 8 + 1];
+    __shared__ uint32_t s_tmem;
     __shared__ int s_fail;
-
+    const uint32_t full0 = smem_u32(s_bar), empty0 = full0 + 8u * 8u, accum = empty0 + 8u * 8u;
+    const uint32_t sm0 = smem_u32(sm);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t0 = blockIdx.x * p.taps_per_tile;
-    const int ntap = min(p.taps_per_tile, 27 - t0);
-    const long long kb0 = (long long)blockIdx.y * p.kb_per_cta;
-    const int KB = (int)min((long long)p.kb_per_cta, p.nkb - kb0);
-    const unsigned tx_bytes = (unsigned)(ntap * p.cout * 128 + p.cin * 128);
+
+    // brick column, z chunk and sample
+    int b = blockIdx.x;
+    const int x0 = (b % p.tx) * 8;
+    b /= p.tx;
+    const int y0 = (b % p.ty) * 16;
+    b /= p.ty;
+    const int z0 = (b % p.nzc) * p.zc, bn = b / p.nzc;
+    const int nsteps = min(p.zc, p.D - z0);
+    // tap group and channel block
+    const int gdy = p.stacked ? 1 : 3 / p.ndy, ngrp = (3 / p.ndz) * gdy;
+    const int grp = blockIdx.y % ngrp, cb = blockIdx.y / ngrp;
+    const int dz0 = p.ndz == 3 ? 0 : grp / gdy, dy0 = p.ndy == 3 ? 0 : grp % gdy;
+    const int ndyu = p.stacked ? 1 : p.ndy;
+    const int nacc = p.ndz * ndyu * 3;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
@@ -605,7 +624,7 @@ k_wgrad_umma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 2) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
                      "r"(p.tmem_cols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -613,43 +632,50 @@ k_wgrad_umma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
-    const uint32_t sm0 = smem_u32(sm);
+    const uint32_t tmem = s_tmem;
+    tmem_zero(tmem + ((uint32_t)(warp * 32) << 16), nacc * p.cout);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
+    // load l brings X plane z0 + l + xoff and dY plane z0 + l (when in range); step k multiplies dY plane
+    // z0 + k with the X planes of loads k .. k + ndz - 1
+    const int xoff = p.ndz == 3 ? -1 : dz0 - 1, lead = p.ndz - 1, nloads = nsteps + lead;
     int issued = 0;
     if (threadIdx.x == 0) {
-        // ---- producer: one stage = the ntap shifted dY boxes and the X box of 64 packed voxels
-        for (int kb = 0; kb < KB; ++kb, ++issued) {
-            const int s = kb % S;
-            const uint32_t use = (uint32_t)(kb / S);
-            if (kb >= S && !mbar_wait(empty0 + 8u * s, (use & 1u) ^ 1u, p.tries)) break;
-            const uint32_t fb = full0 + 8u * s;
-            mbar_expect_tx(fb, tx_bytes);
-            const int k0 = (int)((kb0 + kb) * 64);
-            const uint32_t a_dst = sm0 + (uint32_t)s * p.stage_bytes;
-            for (int j = 0; j < ntap; ++j) {
-                const int t = t0 + j;
-                const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
-                tma_load_2d(a_dst + (uint32_t)(j * p.cout * 128), &tmA, fb, k0 - (dz * p.plane_p + dy * p.row_p),
-                            (dx + 1) * p.cout);
-            }
-            tma_load_2d(a_dst + p.a_bytes, &tmB, fb, k0, 0);
+        for (int l = 0; l < nloads; ++l, ++issued) {
+            const int s = l % S;
+            if (l >= S && !mbar_wait(empty0 + 8u * s, (uint32_t)(l / S - 1) & 1u, p.tries)) break;
+            const int zx = z0 + l + xoff;
+            const bool xin = zx >= 0 && zx < p.D, yin = l < nsteps;
+            const uint32_t fb = full0 + 8u * s, dst = sm0 + (uint32_t)s * p.slot_bytes;
+            mbar_expect_tx(fb, (xin ? p.x_tx : 0u) + (yin ? p.dy_tx : 0u));
+            if (xin) tma_load_5d(dst, &tmX, fb, 0, x0 - 1, cb * p.nchunk, y0 - 1, bn * p.D + zx);
+            if (yin) tma_load_5d(dst + p.x_bytes, &tmY, fb, 0, x0, y0, 0, bn * p.D + z0 + l);
         }
     } else if (threadIdx.x == 32) {
-        // ---- MMA issuer: 4 MMAs (K = 16 packed voxels each) per stage into the TMEM accumulator
         bool ok = true;
-        for (int kb = 0; kb < KB && ok; ++kb) {
-            const int s = kb % S;
-            const uint32_t use = (uint32_t)(kb / S);
-            ok = mbar_wait(full0 + 8u * s, use & 1u, p.tries);
+        int seen = 0;  // loads known to have landed
+        for (int k = 0; k < nsteps && ok; ++k) {
+            for (; seen <= k + lead && ok; ++seen) ok = mbar_wait(full0 + 8u * (seen % S), (uint32_t)(seen / S) & 1u, p.tries);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a_addr = sm0 + (uint32_t)s * p.stage_bytes;
-            const uint32_t b_addr = a_addr + p.a_bytes;
-            for (int k = 0; k < 4; ++k)
-                umma_f16(tmem, sdesc(a_addr + 32u * k, p.desc_hi), sdesc(b_addr + 32u * k, p.desc_hi), p.idesc,
-                         (kb > 0 || k > 0) ? 1u : 0u);
-            umma_commit(empty0 + 8u * s);
+            const uint32_t yb = sm0 + (uint32_t)(k % S) * p.slot_bytes + p.x_bytes;
+            for (int dz = 0; dz < p.ndz; ++dz) {
+                const int zx = z0 + k + dz + xoff;
+                if (zx < 0 || zx >= p.D) continue;  // the zero padding: nothing to add
+                const uint32_t xb = sm0 + (uint32_t)((k + dz) % S) * p.slot_bytes;
+                for (int dy = 0; dy < ndyu; ++dy)
+                    for (int dx = 0; dx < 3; ++dx) {
+                        const uint32_t d = tmem + (uint32_t)(((dz * ndyu + dy) * 3 + dx) * p.cout);
+                        const uint32_t a0 = xb + (uint32_t)((dy0 + dy) * p.nchunk) * WX_ROW + 16u * dx;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            umma_f16(d, sdesc(a0 + (uint32_t)(2 * j * p.nchunk) * WX_ROW, p.a_hi),
+                                     sdesc(yb + 256u * j, p.b_hi), p.idesc, 1u);
+                    }
+            }
+            umma_commit(empty0 + 8u * (k % S));
         }
         if (!ok) s_fail = 1;
         umma_commit(accum);
@@ -657,24 +683,32 @@ k_wgrad_umma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     __syncwarp();
     __syncthreads();
 
-    // ---- epilogue: TMEM lane r = row (tap t0 + r / cout, channel r % cout), columns = input channels
-    const bool ready = mbar_wait(accum, 0u, p.tries) && !s_fail && KB > 0;
+    // ---- epilogue: row r of the accumulators (TMEM lane r; with M = 64 rows 16w .. 16w + 15 lie in the first
+    // 16 lanes of warp w's quadrant) is channel r % 8 of core matrix r / 8
+    const bool ready = mbar_wait(accum, 0u, p.tries) && !s_fail;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const int r = warp * 32 + lane;
-    const int j = r / p.cout, co = r - j * p.cout;
-    const bool live = ready && j < ntap;
-    for (int c0 = 0; c0 < p.cin; c0 += 16) {
-        float o[16];
-        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, o);  // whole warp, always
-        if (!live) continue;
-        float* dst = p.dw + ((long long)(t0 + j) * p.cout + co) * p.cin + c0;
+    const int r = p.m64 ? warp * 16 + lane : warp * 32 + lane;
+    const int core = r >> 3;
+    const int dys = p.stacked ? core / p.nchunk : 0;
+    const int ci = cb * p.cb + (p.stacked ? core % p.nchunk : core) * 8 + (r & 7);
+    const bool live = ready && !(p.m64 && lane >= 16) && dys < 3;
+    for (int acc = 0; acc < nacc; ++acc) {
+        const int dx = acc % 3, q = acc / 3;
+        const int dy = p.stacked ? dys : dy0 + q % ndyu, dz = dz0 + q / ndyu;
+        float* dst = p.dw + ((long long)((dz * 3 + dy) * 3 + dx) * p.cout) * p.cin + ci;
+        for (int c0 = 0; c0 < p.cout; c0 += 16) {
+            float o[16];
+            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * p.cout + c0), o);  // whole warp, always
+            if (!live) continue;
 #pragma unroll
-        for (int q = 0; q < 16; ++q) atomicAdd(dst + q, o[q]);
+            for (int k = 0; k < 16; ++k) atomicAdd(dst + (long long)(c0 + k) * p.cin, o[k]);
+        }
     }
 
+    // after a failed wait, the loads still in flight land before the shared memory is released
     if (threadIdx.x == 0 && !ready) {
-        for (int kb = issued - S < 0 ? 0 : issued - S; kb < issued; ++kb)
-            mbar_wait(full0 + 8u * (kb % S), (uint32_t)(kb / S) & 1u, p.tries);
+        for (int l = issued - S < 0 ? 0 : issued - S; l < issued; ++l)
+            mbar_wait(full0 + 8u * (l % S), (uint32_t)(l / S) & 1u, p.tries);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -684,26 +718,11 @@ k_wgrad_umma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     }
 }
 
-// Packing for the weight gradient: X and the three dx-shifted copies of dY, channel-major over the padded
-// grid (see k_wgrad_umma); the buffers are zeroed before, so the padding stays zero.
-__global__ void k_wgrad_pack(const __nv_bfloat16* __restrict__ dy, int lddy, int dyoff, int cout,
-                             const __nv_bfloat16* __restrict__ x, int ldx, int xoff, int cin, int D, int H, int W,
-                             int Wp, long long nvox, long long vp64, __nv_bfloat16* __restrict__ A3,
-                             __nv_bfloat16* __restrict__ XB) {
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nvox; v += (long long)gridDim.x * blockDim.x) {
-        const int xx = (int)(v % W);
-        long long q = v / W;
-        const int yy = (int)(q % H);
-        q /= H;
-        const int zz = (int)(q % D);
-        const long long b = q / D;
-        const long long vp = ((b * (D + 2) + zz + 1) * (H + 2) + yy + 1) * (long long)Wp + xx + 1;
-        for (int c = 0; c < cout; ++c) {
-            const __nv_bfloat16 val = dy[v * lddy + dyoff + c];
-            for (int d = 0; d < 3; ++d) A3[((long long)d * cout + c) * vp64 + vp + (d - 1)] = val;
-        }
-        for (int c = 0; c < cin; ++c) XB[(long long)c * vp64 + vp] = x[v * ldx + xoff + c];
-    }
+// compact copy of a channel slice (operands whose rows do not start on 16 bytes)
+__global__ void k_compact(const __nv_bfloat16* __restrict__ x, int ld, int off, int c, long long n,
+                          __nv_bfloat16* __restrict__ out) {
+    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x)
+        out[q] = x[(q / c) * ld + off + q % c];
 }
 
 // ---------------------------------------------------------------- host side
@@ -794,6 +813,97 @@ pf_status conv_halo(const void* x, int ldx, int xoff, const void* w, int cin, in
     const long long blocks = (long long)a.tx * a.ty * a.tz * n;
     if (blocks > 0x7FFFFFFFLL) return PF_E_RANGE;
     k_conv_halo<<<(unsigned)blocks, UTHR, smem, stream>>>(mX, a);
+    pfgb::count_launch();
+    return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
+}
+
+// Division of a weight gradient's taps and channels over blocks.  cb: the largest of 128, 64, 32, 16 that
+// divides cin.  Stacked (dy along M) for 16 and 32 channels.  A block takes every dz (each X plane loaded
+// once) while its accumulators fit 512 TMEM columns, else one dz (dY loaded three times), else one (dz, dy).
+void wgrad_plan(WgArgs& a) {
+    a.cb = a.cin % 128 == 0 ? 128 : (a.cin % 64 == 0 ? 64 : (a.cin % 32 == 0 ? 32 : 16));
+    a.nchunk = a.cb / 8;
+    a.stacked = a.cb <= 32;
+    a.m64 = a.cb == 16 || a.cb == 64;
+    const int per_dz = (a.stacked ? 3 : 9) * a.cout;
+    a.ndz = 3 * per_dz <= 512 ? 3 : 1;
+    a.ndy = a.stacked || per_dz <= 512 ? 3 : 1;
+    const int cols = a.ndz * (a.stacked ? 1 : a.ndy) * 3 * a.cout;
+    a.tmem_cols = cols <= 64 ? 64 : (cols <= 128 ? 128 : (cols <= 256 ? 256 : 512));
+}
+
+pf_status wgrad(const void* dy, int lddy, int dyoff, int cout, const void* x, int ldx, int xoff, int cin, float* dw, int n,
+                int d, int h, int wd, cudaStream_t st) {
+    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+    if (!enc) return PF_E_CUDA;
+    WgArgs a{};
+    a.cin = cin;
+    a.cout = cout;
+    a.D = d;
+    a.H = h;
+    a.W = wd;
+    a.tries = WAIT_TRIES;
+    a.dw = dw;
+    wgrad_plan(a);
+    a.tx = (wd + 7) / 8;
+    a.ty = (h + 15) / 16;
+    a.x_tx = 18u * (unsigned)a.nchunk * WX_ROW;
+    a.dy_tx = 16u * 8u * 2u * (unsigned)cout;
+    a.x_bytes = (a.x_tx + 127u) & ~127u;
+    a.slot_bytes = (a.x_bytes + a.dy_tx + 127u) & ~127u;
+    // the unused core matrices of a stacked A operand reach one row past a plane: at least 4 KB follow the slots
+    const unsigned slack = 4096;
+    const int want = a.ndz == 3 ? 6 : 4;
+    int slots = (int)((200u * 1024u - slack) / a.slot_bytes);
+    a.slots = slots < want ? slots : want;
+    const size_t smem = 1024 + (size_t)a.slots * a.slot_bytes + slack;
+    // MN-major, no swizzle (bits 15, 16 of the instruction descriptor = 1): leading offset = stride between
+    // 8-voxel groups of K, stride offset = stride between 8-channel groups of M or N
+    a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((unsigned)(cout >> 3) << 17) |
+              ((unsigned)((a.m64 ? 64 : 128) >> 4) << 24);
+    a.a_hi = desc_plain(0, (unsigned)a.nchunk * WX_ROW, WX_ROW);
+    a.b_hi = desc_plain(0, 128u, 16u * 128u);
+    const int groups = (3 / a.ndz) * (a.stacked ? 1 : 3 / a.ndy) * (cin / a.cb);
+    // about one wave: resident blocks by shared memory (228 KB per SM) and TMEM columns (512)
+    int occ = (int)(228u * 1024u / (smem + 2048));
+    if (occ > 512 / a.tmem_cols) occ = 512 / a.tmem_cols;
+    if (occ < 1) occ = 1;
+    const long long columns = (long long)a.tx * a.ty * n * groups;
+    long long nzc = (152LL * occ + columns - 1) / columns;
+    if (nzc > d) nzc = d;
+    a.zc = (int)((d + nzc - 1) / nzc);
+    a.nzc = (d + a.zc - 1) / a.zc;
+    alignas(64) CUtensorMap mX, mY;
+    const cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    {
+        const cuuint64_t row = (cuuint64_t)ldx * 2;
+        const cuuint64_t dims[5] = {8, (cuuint64_t)wd, (cuuint64_t)(cin / 8), (cuuint64_t)h, (cuuint64_t)n * d};
+        const cuuint64_t strides[4] = {row, 16, row * wd, row * wd * h};
+        const cuuint32_t box[5] = {8, 10, (cuuint32_t)a.nchunk, 18, 1};
+        if (enc(&mX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)((const bf16*)x + xoff), dims, strides, box, es,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return PF_E_INVALID;
+    }
+    {
+        const cuuint64_t row = (cuuint64_t)lddy * 2;
+        const cuuint64_t dims[5] = {8, (cuuint64_t)wd, (cuuint64_t)h, (cuuint64_t)(cout / 8), (cuuint64_t)n * d};
+        const cuuint64_t strides[4] = {row, row * wd, 16, row * wd * h};
+        const cuuint32_t box[5] = {8, 8, 16, (cuuint32_t)(cout / 8), 1};
+        if (enc(&mY, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)((const bf16*)dy + dyoff), dims, strides, box, es,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return PF_E_INVALID;
+    }
+    static std::once_flag wg_once;
+    static cudaError_t wg_err = cudaSuccess;
+    std::call_once(wg_once, [] {
+        wg_err = cudaFuncSetAttribute(k_wgrad_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, 202 * 1024);
+    });
+    if (wg_err != cudaSuccess) return PF_E_CUDA;
+    const long long bx = (long long)a.tx * a.ty * a.nzc * n;
+    if (bx > 0x7FFFFFFFLL) return PF_E_RANGE;
+    k_wgrad_umma<<<dim3((unsigned)bx, (unsigned)groups), UTHR, smem, st>>>(mX, mY, a);
     pfgb::count_launch();
     return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
 }
@@ -895,19 +1005,11 @@ pf_status pfnn_conv3d(const void* x, int ldx, int xoff, const void* w, int cin, 
     return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
 }
 
-// packed layout of the weight gradient: padded row W' = W + 2 rounded up to 8, packed voxels rounded to 64
-static void wgrad_layout(int n, int d, int h, int wd, int* wp, long long* vp64) {
-    *wp = (wd + 2 + 7) / 8 * 8;
-    const long long vp = (long long)n * (d + 2) * (h + 2) * (*wp);
-    *vp64 = (vp + 63) / 64 * 64;
-}
-
+// (more than the compact copies of both operands that pfnn_conv3d_wgrad may need: 2 (cout + cin) bytes a voxel)
 long long pfnn_conv3d_wgrad_work_bytes(int cout, int cin, int n, int d, int h, int wd) {
     if (cout < 1 || cin < 1 || n < 1 || d < 1 || h < 1 || wd < 1) return -1;
-    int wp;
-    long long vp64;
-    wgrad_layout(n, d, h, wd, &wp, &vp64);
-    return 2LL * (3LL * cout + cin) * vp64;
+    const long long vp = (long long)n * (d + 2) * (h + 2) * ((wd + 2 + 7) / 8 * 8);
+    return 2LL * (3LL * cout + cin) * ((vp + 63) / 64 * 64);
 }
 
 pf_status pfnn_conv3d_wgrad(const void* dy, int lddy, int dyoff, int cout, const void* x, int ldx, int xoff, int cin,
@@ -918,76 +1020,24 @@ pf_status pfnn_conv3d_wgrad(const void* dy, int lddy, int dyoff, int cout, const
         return PF_E_INVALID;
     if (work_bytes < pfnn_conv3d_wgrad_work_bytes(cout, cin, n, d, h, wd) || reinterpret_cast<uintptr_t>(work) % 16)
         return PF_E_INVALID;
-    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
-    if (!enc) return PF_E_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
-    int wp;
-    long long vp64;
-    wgrad_layout(n, d, h, wd, &wp, &vp64);
-    bf16* A3 = (bf16*)work;
-    bf16* XB = A3 + 3LL * cout * vp64;
-    if (cudaMemsetAsync(work, 0, (size_t)pfnn_conv3d_wgrad_work_bytes(cout, cin, n, d, h, wd), st) != cudaSuccess)
-        return PF_E_CUDA;
+    // TMA reads rows that start on 16 bytes; other slices are copied to the scratch first
     const long long nvox = (long long)n * d * h * wd;
-    long long pb = (nvox + 255) / 256;
-    if (pb > 152LL * 32) pb = 152LL * 32;
-    k_wgrad_pack<<<(unsigned)pb, 256, 0, st>>>((const bf16*)dy, lddy, dyoff, cout, (const bf16*)x, ldx, xoff, cin, d, h,
-                                                wd, wp, nvox, vp64, A3, XB);
-    pfgb::count_launch();
-
-    alignas(64) CUtensorMap mA, mB;
-    {
-        const cuuint64_t dims[2] = {(cuuint64_t)vp64, (cuuint64_t)(3 * cout)};
-        const cuuint64_t strides[1] = {(cuuint64_t)vp64 * 2};
-        const cuuint32_t box[2] = {64, (cuuint32_t)cout};
-        const cuuint32_t es[2] = {1, 1};
-        if (enc(&mA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, A3, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return PF_E_INVALID;
-    }
-    {
-        const cuuint64_t dims[2] = {(cuuint64_t)vp64, (cuuint64_t)cin};
-        const cuuint64_t strides[1] = {(cuuint64_t)vp64 * 2};
-        const cuuint32_t box[2] = {64, (cuuint32_t)cin};
-        const cuuint32_t es[2] = {1, 1};
-        if (enc(&mB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, XB, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return PF_E_INVALID;
-    }
-    WgArgs a{};
-    a.cout = cout;
-    a.cin = cin;
-    a.taps_per_tile = UM / cout;
-    const int ntiles = (27 + a.taps_per_tile - 1) / a.taps_per_tile;
-    a.nkb = vp64 / 64;
-    // about four waves of CTAs over the 152 SMs
-    long long chunks = (4LL * 152 + ntiles - 1) / ntiles;
-    if (chunks > a.nkb) chunks = a.nkb;
-    a.kb_per_cta = (int)((a.nkb + chunks - 1) / chunks);
-    chunks = (a.nkb + a.kb_per_cta - 1) / a.kb_per_cta;
-    a.plane_p = (h + 2) * wp;
-    a.row_p = wp;
-    a.a_bytes = (unsigned)(UM * 128);
-    a.stage_bytes = a.a_bytes + round1024((unsigned)(cin * 128));
-    int stages = (int)(98304u / a.stage_bytes);
-    a.stages = stages < 2 ? 2 : (stages > 8 ? 8 : stages);
-    a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(cin >> 3) << 17) | ((unsigned)(UM >> 4) << 24);
-    a.desc_hi = (1ULL << 16) | ((1024ULL >> 4) << 32) | (1ULL << 46) | (umma_layout(64) << 61);
-    a.tmem_cols = cin <= 32 ? 32 : (cin <= 64 ? 64 : (cin <= 128 ? 128 : 256));
-    a.tries = WAIT_TRIES;
-    a.dw = dw;
-    const size_t smem = (size_t)a.stages * a.stage_bytes + 1024 + 16 * a.stages + 16;
-    static std::once_flag wg_once;
-    static cudaError_t wg_err = cudaSuccess;
-    std::call_once(wg_once, [] {
-        wg_err = cudaFuncSetAttribute(k_wgrad_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024 + 2048);
-    });
-    if (wg_err != cudaSuccess) return PF_E_CUDA;
-    k_wgrad_umma<<<dim3((unsigned)ntiles, (unsigned)chunks), UTHR, smem, st>>>(mA, mB, a);
-    pfgb::count_launch();
-    return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
+    bf16* scratch = (bf16*)work;
+    auto aligned = [&](const void*& q, int& ld, int& off, int c) {
+        if (ld % 8 == 0 && off % 8 == 0 && reinterpret_cast<uintptr_t>(q) % 16 == 0) return;
+        long long blocks = (nvox * c + 255) / 256;
+        if (blocks > 152LL * 32) blocks = 152LL * 32;
+        k_compact<<<(unsigned)blocks, 256, 0, st>>>((const bf16*)q, ld, off, c, nvox * c, scratch);
+        pfgb::count_launch();
+        q = scratch;
+        ld = c;
+        off = 0;
+        scratch += nvox * c;  // c is a multiple of 16: the next copy starts on 32 bytes
+    };
+    aligned(dy, lddy, dyoff, cout);
+    aligned(x, ldx, xoff, cin);
+    return wgrad(dy, lddy, dyoff, cout, x, ldx, xoff, cin, dw, n, d, h, wd, st);
 }
 
 pf_status pfnn_status(int* failed) {
@@ -1007,3 +1057,12 @@ pf_status pfnn_test_withhold_stage(int stage, long long tries) {
 }
 
 }  // extern "C"
+
+namespace pfgb {
+
+pf_status nn_wgrad(const void* dy, int cout, const void* x, int ldx, int xoff, int cin, float* dw, int n, int d, int h,
+                   int wd, void* stream) {
+    return wgrad(dy, cout, 0, cout, x, ldx, xoff, cin, dw, n, d, h, wd, (cudaStream_t)stream);
+}
+
+}  // namespace pfgb

@@ -116,3 +116,30 @@ def test_head(env, c, nvox):
     tol = (nvox + 10) * 2 ** -24
     assert np.all(np.abs(dw.double().cpu().numpy() - d @ xd) <= tol * (np.abs(d) @ np.abs(xd)) + 1e-30)
     assert abs(float(db) - d.sum()) <= tol * np.abs(d).sum() + 1e-30
+
+
+# every division of the taps over blocks (all dz in one block, one dz, one (dz, dy); dy stacked along M or not),
+# channel blocks of 16, 32, 64 and 128, several z chunks, ragged columns, slices that are not on 16 bytes
+@pytest.mark.parametrize("cin,cout,shape,skew", [
+    (16, 16, (1, 37, 17, 9), 0), (16, 32, (2, 5, 16, 8), 1), (16, 64, (1, 4, 33, 7), 0), (32, 32, (1, 21, 5, 17), 0),
+    (32, 128, (1, 3, 18, 10), 0), (64, 16, (1, 7, 20, 12), 3), (64, 32, (3, 2, 3, 8), 0), (64, 64, (1, 6, 15, 9), 0),
+    (128, 128, (1, 3, 9, 9), 0), (96, 16, (1, 2, 17, 8), 0), (256, 32, (1, 2, 3, 5), 0), (16, 16, (1, 1, 1, 1), 0)])
+def test_weight_gradient_plans(env, cin, cout, shape, skew):
+    torch, nn, L = env
+    from oracle import nn_oracle as O
+    g = np.random.default_rng(cin + 3 * cout)
+    n, d, h, w = shape
+    big = [torch.from_numpy(g.standard_normal((n, d, h, w, c + skew)).astype(np.float32)).cuda().to(torch.bfloat16)
+           for c in (cin, cout)]
+    x, dy = (b[..., skew:].double().cpu().numpy() for b in big)
+    dw = torch.zeros((27, cout, cin), device="cuda")
+    wb = L.pfnn_conv3d_wgrad_work_bytes(cout, cin, n, d, h, w)
+    work = torch.full((wb,), 255, dtype=torch.uint8, device="cuda")
+    assert L.pfnn_conv3d_wgrad(nn._p(big[1]), cout + skew, skew, cout, nn._p(big[0]), cin + skew, skew, cin, nn._p(dw),
+                               n, d, h, w, nn._p(work), wb, None) == 0
+    torch.cuda.synchronize()
+    ref = O.conv3d_bwd_weight(dy, x)
+    # binary32 sums of n d h w products in any order
+    assert np.abs(dw.double().cpu().numpy() - ref).max() <= 2e-5 * np.abs(ref).max()
+    flag = nn.C.c_int(-1)
+    assert L.pfnn_status(nn.C.byref(flag)) == 0 and flag.value == 0
