@@ -362,11 +362,12 @@ k_head_fwd_loss(const __nv_bfloat16* __restrict__ x, int c, const float* __restr
 // head backward: dx[v][c] = dlogit[v] w[c]; dw[c] += sum_v dlogit[v] x[v][c]; db += sum_v dlogit[v].
 // NV as above.  The sums go through warp shuffles and shared memory to one atomic per channel and block
 // (with one per channel and thread the atomics on c + 1 addresses took nearly all of its time: 2.75 ms for
-// 4 x 64^3 voxels of 16 channels).
+// 4 x 64^3 voxels of 16 channels).  The terms (sigmoid - target) / nvox largely cancel, so the warps' sums
+// are added in binary64; with `acc64` ([c] and one for the bias, zeroed) the blocks' are too.
 template <int NV>
 __global__ void __launch_bounds__(256)
 k_head_bwd(const __nv_bfloat16* __restrict__ x, int c, const float* __restrict__ w, const float* __restrict__ dlogit,
-           long long nvox, float* __restrict__ dx, float* dw, float* db) {
+           long long nvox, float* __restrict__ dx, float* dw, float* db, double* acc64) {
     constexpr int CM = NV > 0 ? 8 * NV : 32;
     float acc[CM + 1];
 #pragma unroll
@@ -404,11 +405,18 @@ k_head_bwd(const __nv_bfloat16* __restrict__ x, int c, const float* __restrict__
     __syncthreads();
     if (threadIdx.x <= CM) {
         const int ch = threadIdx.x;
-        float t = 0.f;
+        double t = 0.0;
         for (int q = 0; q < 8; ++q) t += sh[ch][q];
-        if (ch == CM) atomicAdd(db, t);
-        else if (NV > 0 || ch < c) atomicAdd(dw + ch, t);
+        if (ch < CM && NV == 0 && ch >= c) return;
+        if (acc64) atomicAdd(acc64 + (ch == CM ? c : ch), t);
+        else atomicAdd(ch == CM ? db : dw + ch, (float)t);
     }
+}
+
+__global__ void k_head_sums(const double* __restrict__ acc64, int c, float* dw, float* db) {
+    const int ch = threadIdx.x;
+    if (ch < c) dw[ch] += (float)acc64[ch];
+    else if (ch == c) db[0] += (float)acc64[ch];
 }
 
 // Adam with bias correction on FP32 master weights; writes the bf16 working copy.
@@ -569,16 +577,22 @@ pf_status pfnn_head_forward(const void* x, int c, const float* w, const float* b
     return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
 }
 
-pf_status pfnn_head_backward(const void* x, int c, const float* w, const float* dlogit, long long nvox, float* dx,
-                             float* dw, float* db, void* stream) {
+static pf_status head_backward(const void* x, int c, const float* w, const float* dlogit, long long nvox, float* dx,
+                               float* dw, float* db, double* acc64, void* stream) {
     if (!x || !w || !dlogit || !dx || !dw || !db || c < 1 || c > 32) return PF_E_INVALID;
     auto k = !vec_ok(8, {c}, {x, dx}) ? k_head_bwd<0> : c == 8 ? k_head_bwd<1> : c == 16 ? k_head_bwd<2>
              : c == 24 ? k_head_bwd<3> : k_head_bwd<4>;
     long long blocks = (nvox + 511) / 512;  // two voxels per thread at least, four blocks per SM at most
     if (blocks > 152 * 4) blocks = 152 * 4;
-    k<<<(unsigned)(blocks < 1 ? 1 : blocks), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, c, w, dlogit, nvox, dx, dw, db);
+    k<<<(unsigned)(blocks < 1 ? 1 : blocks), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, c, w, dlogit, nvox, dx, dw, db,
+                                                                            acc64);
     pfgb::count_launch();
     return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
+}
+
+pf_status pfnn_head_backward(const void* x, int c, const float* w, const float* dlogit, long long nvox, float* dx,
+                             float* dw, float* db, void* stream) {
+    return head_backward(x, c, w, dlogit, nvox, dx, dw, db, nullptr, stream);
 }
 
 pf_status pfnn_pack_input(const float* G, const float* feat, int nfeat, long long vox_per_sample, long long nvox,
@@ -612,6 +626,16 @@ namespace pfgb {
 pf_status nn_upsample_bwd_set(const float* dy, int lddy, int dyoff, int c, float* dx, int n, int d, int h, int wd,
                               void* stream) {
     return upsample_bwd(dy, lddy, dyoff, c, dx, n, d, h, wd, 1, stream);
+}
+
+pf_status nn_head_backward64(const void* x, int c, const float* w, const float* dlogit, long long nvox, float* dx,
+                             float* dw, float* db, double* acc64, void* stream) {
+    if (cudaMemsetAsync(acc64, 0, sizeof(double) * (c + 1), (cudaStream_t)stream) != cudaSuccess) return PF_E_CUDA;
+    pf_status s = head_backward(x, c, w, dlogit, nvox, dx, dw, db, acc64, stream);
+    if (s != PF_OK) return s;
+    k_head_sums<<<1, 64, 0, (cudaStream_t)stream>>>(acc64, c, dw, db);
+    count_launch();
+    return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
 }
 
 pf_status nn_relu_bwd_bias(const float* dy, int lddy, int dyoff, const void* y, int ldy, int yoff, int c, long long nvox,

@@ -28,6 +28,9 @@ pf_status nn_upsample_bwd_set(const float* dy, int lddy, int dyoff, int c, float
                               void* stream);
 pf_status nn_relu_bwd_bias(const float* dy, int lddy, int dyoff, const void* y, int ldy, int yoff, int c, long long nvox,
                            void* dz_bf16, float* db, void* stream);
+// pfnn_head_backward with the sums over blocks in binary64 (acc64: scratch of c + 1 values)
+pf_status nn_head_backward64(const void* x, int c, const float* w, const float* dlogit, long long nvox, float* dx,
+                             float* dw, float* db, double* acc64, void* stream);
 // pfnn_umma.cu: pfnn_conv3d_wgrad of a compact dy and 16-byte aligned rows of x (no scratch needed)
 pf_status nn_wgrad(const void* dy, int cout, const void* x, int ldx, int xoff, int cin, float* dw, int n, int d, int h,
                    int wd, void* stream);
@@ -166,7 +169,7 @@ struct pfnn_net {
     float* grad[NBUF] = {};                // fp32 gradients of the activations
     float *logit_grad = nullptr, *prob = nullptr;
     void* dz_b = nullptr;
-    double* loss = nullptr;
+    double* loss = nullptr;                // the loss, then the 17 sums of the head's backward pass
     bool have_target = false;
     std::vector<void*> allocs, act_allocs;
     std::string err;
@@ -347,7 +350,7 @@ pf_status pfnn_net_create(unsigned long long seed, void* stream, pfnn_net** out)
         pfnn_net_destroy(net);
         return PF_E_CUDA;
     }
-    net->loss = (double*)nalloc(net->allocs, sizeof(double));
+    net->loss = (double*)nalloc(net->allocs, 18 * sizeof(double));
     if (!net->loss) {
         pfnn_net_destroy(net);
         return PF_E_OOM;
@@ -451,8 +454,8 @@ pf_status pfnn_net_backward(pfnn_net* net) {
     // half of a skip buffer, whose decoder layer comes later in the forward order), so none is zeroed.
     const long long nvox0 = (long long)n * side * side * side;
     const Param& H = net->p[NCONV];
-    NN_CK(net, pfnn_head_backward(net->act[D1B], 16, H.w, net->logit_grad, nvox0, net->grad[D1B], H.gw, H.gb, s),
-          "head backward");
+    NN_CK(net, pfgb::nn_head_backward64(net->act[D1B], 16, H.w, net->logit_grad, nvox0, net->grad[D1B], H.gw, H.gb,
+                                        net->loss + 1, s), "head backward");
     for (int q = NCONV - 1; q >= 0; --q) {
         const Layer& L = kLayers[q];
         Param& P = net->p[q];

@@ -656,24 +656,26 @@ k_wgrad_umma(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
     } else if (threadIdx.x == 32) {
         bool ok = true;
         int seen = 0;  // loads known to have landed
+        const uint32_t alo = (uint32_t)p.a_hi, ahi = (uint32_t)(p.a_hi >> 32);
+        const uint32_t blo = (uint32_t)p.b_hi, bhi = (uint32_t)(p.b_hi >> 32);
+        const uint32_t yrow = (uint32_t)p.nchunk * (WX_ROW / 16);  // one row of the X tile, 16-byte units
         for (int k = 0; k < nsteps && ok; ++k) {
             for (; seen <= k + lead && ok; ++seen) ok = mbar_wait(full0 + 8u * (seen % S), (uint32_t)(seen / S) & 1u, p.tries);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t yb = sm0 + (uint32_t)(k % S) * p.slot_bytes + p.x_bytes;
+            // descriptor low words: the start field (16-byte units) is advanced by adding to them
+            const uint32_t yl = blo + ((sm0 + (uint32_t)(k % S) * p.slot_bytes + p.x_bytes) >> 4);
             for (int dz = 0; dz < p.ndz; ++dz) {
                 const int zx = z0 + k + dz + xoff;
                 if (zx < 0 || zx >= p.D) continue;  // the zero padding: nothing to add
-                const uint32_t xb = sm0 + (uint32_t)((k + dz) % S) * p.slot_bytes;
-                for (int dy = 0; dy < ndyu; ++dy)
-                    for (int dx = 0; dx < 3; ++dx) {
-                        const uint32_t d = tmem + (uint32_t)(((dz * ndyu + dy) * 3 + dx) * p.cout);
-                        const uint32_t a0 = xb + (uint32_t)((dy0 + dy) * p.nchunk) * WX_ROW + 16u * dx;
+                uint32_t xl = alo + ((sm0 + (uint32_t)((k + dz) % S) * p.slot_bytes) >> 4) + (uint32_t)dy0 * yrow;
+                uint32_t dt = tmem + (uint32_t)(dz * ndyu * 3) * p.cout;
+                for (int dy = 0; dy < ndyu; ++dy, xl += yrow)
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx, dt += p.cout)
 #pragma unroll
                         for (int j = 0; j < 8; ++j)
-                            umma_f16(d, sdesc(a0 + (uint32_t)(2 * j * p.nchunk) * WX_ROW, p.a_hi),
-                                     sdesc(yb + 256u * j, p.b_hi), p.idesc, 1u);
-                    }
+                            umma_f16_w(dt, xl + dx + 2 * j * yrow, ahi, yl + 16 * j, bhi, p.idesc, 1u);
             }
             umma_commit(empty0 + 8u * (k % S));
         }
@@ -868,11 +870,18 @@ pf_status wgrad(const void* dy, int lddy, int dyoff, int cout, const void* x, in
     int occ = (int)(228u * 1024u / (smem + 2048));
     if (occ > 512 / a.tmem_cols) occ = 512 / a.tmem_cols;
     if (occ < 1) occ = 1;
-    const long long columns = (long long)a.tx * a.ty * n * groups;
-    long long nzc = (152LL * occ + columns - 1) / columns;
-    if (nzc > d) nzc = d;
-    a.zc = (int)((d + nzc - 1) / nzc);
-    a.nzc = (d + a.zc - 1) / a.zc;
+    // z chunks: the fewest waves x (planes + about four for the prologue, the extra X planes and the epilogue)
+    const long long columns = (long long)a.tx * a.ty * n * groups, cap = 152LL * occ;
+    long long best = -1;
+    for (int nz = 1; nz <= d && nz <= 64; ++nz) {
+        const int zc = (d + nz - 1) / nz, chunks = (d + zc - 1) / zc;
+        const long long cost = ((columns * chunks + cap - 1) / cap) * (zc + 4);
+        if (best < 0 || cost < best) {
+            best = cost;
+            a.zc = zc;
+            a.nzc = chunks;
+        }
+    }
     alignas(64) CUtensorMap mX, mY;
     const cuuint32_t es[5] = {1, 1, 1, 1, 1};
     {
