@@ -97,6 +97,172 @@ __global__ void k_sf_apply(const float* __restrict__ prob, const double* __restr
     }
 }
 
+// ---- Bit form: one bit per cell, 32 cells of a row to a word, so a mask of 256^3 cells is 2 MB and stays in L2.
+// The byte form above swept 16.8 MB of flags from global memory once per cell of path length (10.1 ms for a 256^3 packing);
+// here a block brings a tile of words to its own fixed point in shared memory before the next sweep, a word is filled
+// along x by one carry, and the water indicator is kept as a mask, so G is read once: 0.68 ms.
+struct BitGrid {
+    int n1, n2, n3, W;  // W words per row
+    unsigned tail;      // cells of a row's last word
+};
+
+__device__ __forceinline__ unsigned valid_bits(const BitGrid& g, int wx) { return wx == g.W - 1 ? g.tail : 0xffffffffu; }
+
+// Masks of predicted ice, reached (seed) and water; a warp builds WPI words at a time, so that 3 WPI loads per lane
+// are in flight (the pass is bound by HBM: 20 bytes a cell).
+constexpr int WPI = 4;
+__global__ void __launch_bounds__(SF_THREADS) k_sb_init(const float* __restrict__ prob, const double* __restrict__ seed,
+                                                        const double* __restrict__ G, double zeta, const BitGrid g,
+                                                        unsigned* __restrict__ ice, unsigned* __restrict__ reached,
+                                                        unsigned* __restrict__ water) {
+    const int lane = threadIdx.x & 31;
+    const long long words = (long long)g.W * g.n2 * g.n3;
+    const long long warps = (long long)gridDim.x * (SF_THREADS / 32);
+    for (long long w0 = ((long long)blockIdx.x * (SF_THREADS / 32) + (threadIdx.x >> 5)) * WPI; w0 < words;
+         w0 += warps * WPI) {
+        float p[WPI];
+        double s[WPI], gl[WPI];
+        bool in[WPI];
+#pragma unroll
+        for (int r = 0; r < WPI; ++r) {
+            const long long w = w0 + r;
+            const long long row = w / g.W;
+            const int x = (int)(w - row * g.W) * 32 + lane;
+            in[r] = w < words && x < g.n1;
+            const long long q = row * g.n1 + x;
+            p[r] = in[r] ? prob[q] : 0.f;
+            s[r] = in[r] ? seed[q] : 0.0;
+            gl[r] = in[r] ? G[q] : 0.0;
+        }
+#pragma unroll
+        for (int r = 0; r < WPI; ++r) {
+            const bool wat = in[r] && 1.0 - zeta * gl[r] > 0.0;
+            const unsigned bw = __ballot_sync(0xffffffffu, wat);
+            const unsigned bi = __ballot_sync(0xffffffffu, wat && p[r] > 0.5f);
+            const unsigned br = __ballot_sync(0xffffffffu, in[r] && s[r] > 0.5);
+            if (lane == 0 && w0 + r < words) {
+                ice[w0 + r] = bi;
+                reached[w0 + r] = br;
+                water[w0 + r] = bw;
+            }
+        }
+    }
+}
+
+// The six face neighbours of every cell of word (wx, j, k), ORed; cells outside the grid count as `out` (0 or ~0).
+// With ERODE the masks are ANDed instead (pass out = ~0).
+template <bool ERODE>
+__device__ __forceinline__ unsigned face_neighbours(const unsigned* __restrict__ m, const BitGrid& g, int wx, int j, int k,
+                                                    long long w, unsigned own) {
+    const long long pl = (long long)g.W * g.n2;
+    const unsigned out = ERODE ? 0xffffffffu : 0u;
+    const unsigned lw = wx > 0 ? m[w - 1] : out, rw = wx < g.W - 1 ? m[w + 1] : out;
+    // the cell behind the row's last one is outside the grid
+    const unsigned o = ERODE ? own | ~valid_bits(g, wx) : own;
+    const unsigned l = (o << 1) | (lw >> 31), r = (o >> 1) | (rw << 31);
+    const unsigned a = j > 0 ? m[w - g.W] : out, b = j < g.n2 - 1 ? m[w + g.W] : out;
+    const unsigned c = k > 0 ? m[w - pl] : out, d = k < g.n3 - 1 ? m[w + pl] : out;
+    return ERODE ? (l & r & a & b & c & d) : (l | r | a | b | c | d);
+}
+
+// one erosion or dilation step from `in` to `to` (erosion: a cell with a face neighbour outside the mask leaves it;
+// dilation: face neighbours join, inside `within` if that is given)
+template <bool ERODE>
+__global__ void __launch_bounds__(SF_THREADS) k_sb_step(const unsigned* __restrict__ in, unsigned* __restrict__ to,
+                                                        const unsigned* __restrict__ within, const BitGrid g) {
+    const long long words = (long long)g.W * g.n2 * g.n3;
+    for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < words; w += (long long)gridDim.x * blockDim.x) {
+        const long long row = w / g.W;
+        const int wx = (int)(w - row * g.W), j = (int)(row % g.n2), k = (int)(row / g.n2);
+        const unsigned own = in[w], nb = face_neighbours<ERODE>(in, g, wx, j, k, w, own);
+        if constexpr (ERODE) to[w] = own & nb;
+        else to[w] = own | (nb & (within ? within[w] : valid_bits(g, wx)));
+    }
+}
+
+// bits of `m` connected along the word to a bit of s (s within m): adding s to m carries from each seed through the ones
+// above it, so the bits the sum cleared are the run from the lowest seed up; the other direction on the reversed word
+__device__ __forceinline__ unsigned fill_up(unsigned m, unsigned s) { return s | (m & ~(m + s)); }
+__device__ __forceinline__ unsigned fill_word(unsigned m, unsigned s) {
+    const unsigned u = fill_up(m, s);
+    return __brev(fill_up(__brev(m), __brev(u)));
+}
+
+// One flood-fill sweep: a block loads a tile of TW x TY x TZ words with a one-word halo and fills it until nothing changes
+// (the halo stays as loaded; masks only gain bits, so a word a neighbour block is about to extend is caught by the next
+// sweep).  Sweep r sets flag r & 3 when it changed something, reads that of the sweep before (nothing changed then: the
+// fixed point is reached, exit) and clears the next one's.
+constexpr int SB_TW = 2, SB_TY = 16, SB_TZ = 16;
+__global__ void __launch_bounds__(SB_TW* SB_TY* SB_TZ) k_sb_flood(const unsigned* __restrict__ mask, unsigned* reached,
+                                                                  const BitGrid g, int* flags, int r) {
+    __shared__ unsigned t[SB_TZ + 2][SB_TY + 2][SB_TW + 2];
+    if (blockIdx.x == 0 && threadIdx.x == 0) flags[(r + 1) & 3] = 0;
+    if (((volatile int*)flags)[(r + 3) & 3] == 0) return;  // uniform over the grid: written by earlier launches only
+    const int nbx = (g.W + SB_TW - 1) / SB_TW, nby = (g.n2 + SB_TY - 1) / SB_TY;
+    const int bx = blockIdx.x % nbx, by = (blockIdx.x / nbx) % nby, bz = blockIdx.x / (nbx * nby);
+    const int x0 = bx * SB_TW - 1, y0 = by * SB_TY - 1, z0 = bz * SB_TZ - 1;
+    constexpr int CELLS = (SB_TZ + 2) * (SB_TY + 2) * (SB_TW + 2), THREADS = SB_TW * SB_TY * SB_TZ;
+    for (int q = threadIdx.x; q < CELLS; q += THREADS) {
+        const int lx = q % (SB_TW + 2), ly = (q / (SB_TW + 2)) % (SB_TY + 2), lz = q / ((SB_TW + 2) * (SB_TY + 2));
+        const int x = x0 + lx, y = y0 + ly, z = z0 + lz;
+        const bool in = x >= 0 && x < g.W && y >= 0 && y < g.n2 && z >= 0 && z < g.n3;
+        t[lz][ly][lx] = in ? ((volatile unsigned*)reached)[((long long)z * g.n2 + y) * g.W + x] : 0u;
+    }
+    const int lx = threadIdx.x % SB_TW + 1, ly = (threadIdx.x / SB_TW) % SB_TY + 1, lz = threadIdx.x / (SB_TW * SB_TY) + 1;
+    const int x = x0 + lx, y = y0 + ly, z = z0 + lz;
+    const bool in = x < g.W && y < g.n2 && z < g.n3;
+    const long long w = ((long long)z * g.n2 + y) * g.W + x;
+    const unsigned m = in ? mask[w] : 0u;
+    __syncthreads();
+    const unsigned first = t[lz][ly][lx];
+    unsigned own = first;
+    // every pass but the last reaches at least one more cell of the tile
+    for (int it = 0; it <= 32 * THREADS; ++it) {
+        const unsigned nb = (own << 1) | (own >> 1) | (t[lz][ly][lx - 1] >> 31) | (t[lz][ly][lx + 1] << 31) |
+                            t[lz][ly - 1][lx] | t[lz][ly + 1][lx] | t[lz - 1][ly][lx] | t[lz + 1][ly][lx] | own;
+        const unsigned f = own | fill_word(m, nb & m);
+        const int ch = f != own;
+        own = f;
+        if (!__syncthreads_or(ch)) break;
+        if (ch) t[lz][ly][lx] = f;
+        __syncthreads();
+    }
+    if (in && own != first) {
+        reached[w] = own;
+        flags[r & 3] = 1;  // every writer stores the same value
+    }
+}
+
+__global__ void __launch_bounds__(SF_THREADS) k_sb_apply(const float* __restrict__ prob, const double* seed,
+                                                         const unsigned* __restrict__ reached,
+                                                         const unsigned* __restrict__ water, const BitGrid g, double* out) {
+    const int lane = threadIdx.x & 31;
+    const long long words = (long long)g.W * g.n2 * g.n3;
+    const long long warps = (long long)gridDim.x * (SF_THREADS / 32);
+    for (long long w0 = ((long long)blockIdx.x * (SF_THREADS / 32) + (threadIdx.x >> 5)) * WPI; w0 < words;
+         w0 += warps * WPI) {
+        float p[WPI];
+        double s[WPI];
+        long long q[WPI];
+        bool in[WPI], put[WPI];
+#pragma unroll
+        for (int r = 0; r < WPI; ++r) {
+            const long long w = w0 + r;
+            const long long row = w / g.W;
+            const int x = (int)(w - row * g.W) * 32 + lane;
+            in[r] = w < words && x < g.n1;
+            put[r] = in[r] && ((reached[w] & water[w]) >> lane & 1u);
+            q[r] = row * g.n1 + x;
+            s[r] = in[r] ? seed[q[r]] : 0.0;
+            p[r] = put[r] ? prob[q[r]] : 0.f;
+        }
+#pragma unroll
+        for (int r = 0; r < WPI; ++r)
+            // the seed itself stays ice where the prediction has less
+            if (in[r]) out[q[r]] = put[r] ? fmax((double)fminf(fmaxf(p[r], 0.f), 1.f), s[r]) : s[r];
+    }
+}
+
 }  // namespace
 
 extern "C" pf_status pfnn_seed_connect(const float* prob, const double* phi_seed, const double* G, int n1, int n2,
@@ -107,6 +273,57 @@ extern "C" pf_status pfnn_seed_connect(const float* prob, const double* phi_seed
         return PF_E_INVALID;
     cudaStream_t s = (cudaStream_t)stream;
     const long long n = (long long)n1 * n2 * n3;
+    {
+        // Bit form: masks of ice (eroded in place of the original), reached, a second buffer for the steps, water and, with
+        // erosion, the original ice, and four flags.  The scratch (one byte a cell) holds them but for rows of up to 16
+        // cells (up to 20 and 33 to 40 with erosion) and grids of a few cells, which take the byte form.
+        BitGrid g{n1, n2, n3, (n1 + 31) / 32, n1 % 32 ? (1u << (n1 % 32)) - 1u : 0xffffffffu};
+        const long long words = (long long)g.W * n2 * n3;
+        const int masks = erode ? 5 : 4;
+        const long long tiles = ((g.W + SB_TW - 1) / SB_TW) * (long long)((n2 + SB_TY - 1) / SB_TY) * ((n3 + SB_TZ - 1) / SB_TZ);
+        if (4 * masks * words + 16 <= 16 * ((n + 15) / 16) + 4 && tiles < (1LL << 31)) {
+            int* flags = reinterpret_cast<int*>(work);
+            unsigned* ice = reinterpret_cast<unsigned*>(work + 16);
+            unsigned *reached = ice + words, *spare = reached + words, *water = spare + words, *whole = water + words;
+            const int nbi = sf_blocks(words * 32 / WPI), nbw = sf_blocks(words);
+            k_sb_init<<<nbi, SF_THREADS, 0, s>>>(prob, phi_seed, G, zeta, g, ice, reached, water);
+            pfgb::count_launch();
+            if (erode && cudaMemcpyAsync(whole, ice, 4 * words, cudaMemcpyDeviceToDevice, s) != cudaSuccess) return PF_E_CUDA;
+            for (int r = 0; r < erode; ++r) {
+                k_sb_step<true><<<nbw, SF_THREADS, 0, s>>>(ice, spare, nullptr, g);
+                pfgb::count_launch();
+                unsigned* q = ice;
+                ice = spare;
+                spare = q;
+            }
+            long long done = 0;
+            // every sweep that changes something reaches at least one more cell: at most n sweeps
+            if (cudaMemsetAsync(flags, 0xff, 4 * sizeof(int), s) != cudaSuccess) return PF_E_CUDA;
+            for (;;) {
+                for (int r = 0; r < SWEEPS_PER_CHECK; ++r)
+                    k_sb_flood<<<(unsigned)tiles, SB_TW * SB_TY * SB_TZ, 0, s>>>(ice, reached, g, flags, (int)((done + r) & 3));
+                pfgb::count_launch(SWEEPS_PER_CHECK);
+                done += SWEEPS_PER_CHECK;
+                int h = 0;
+                if (cudaMemcpyAsync(&h, flags + ((done - 1) & 3), sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+                    cudaStreamSynchronize(s) != cudaSuccess)
+                    return PF_E_CUDA;
+                if (!h || done > n) break;
+            }
+            for (int r = 0; r < erode + halo; ++r) {
+                k_sb_step<false><<<nbw, SF_THREADS, 0, s>>>(reached, spare, r < erode ? whole : nullptr, g);
+                pfgb::count_launch();
+                unsigned* q = reached;
+                reached = spare;
+                spare = q;
+            }
+            k_sb_apply<<<nbi, SF_THREADS, 0, s>>>(prob, phi_seed, reached, water, g, phi_out);
+            pfgb::count_launch();
+            if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return PF_E_CUDA;
+            if (sweeps) *sweeps = done;
+            return PF_OK;
+        }
+    }
     unsigned char* fl = work;
     int* changed = reinterpret_cast<int*>(work + ((n + 15) / 16) * 16);
     const int nb = sf_blocks(n);
