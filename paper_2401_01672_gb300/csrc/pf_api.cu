@@ -604,13 +604,17 @@ static pf_status create_impl(int n1, int n2, int n3, double h, int model, int re
         ok = ok && q;
         return q ? q + esz * (size_t)(so.zg_lo * plane) : nullptr;
     };
+    // slopes: the binary32 stage kernels form u4 and u5 of the z neighbours from them
+    auto AK = [&]() -> void* { return is_f32(g) ? AG(sizeof(float)) : A(nf); };
     if (has_th(g)) {
         g->y_th[0] = (double*)AG(8); g->y_th[1] = (double*)AG(8);
-        g->ua_th = AG(fbytes(g)); g->ub_th = AG(fbytes(g)); g->k1_th = A(nf); g->k3_th = A(nf); g->k4_th = A(nf);
+        g->ua_th = AG(fbytes(g)); g->ub_th = AG(fbytes(g));
+        g->k1_th = AK(); g->k3_th = AK(); g->k4_th = AK();
     }
     if (has_ph(g)) {
         g->y_ph[0] = (double*)AG(8); g->y_ph[1] = (double*)AG(8);
-        g->ua_ph = AG(fbytes(g)); g->ub_ph = AG(fbytes(g)); g->k1_ph = A(nf); g->k3_ph = A(nf); g->k4_ph = A(nf);
+        g->ua_ph = AG(fbytes(g)); g->ub_ph = AG(fbytes(g));
+        g->k1_ph = AK(); g->k3_ph = AK(); g->k4_ph = AK();
     }
     if (is_f32(g) && model == PF_MODEL_FULL) {
         for (int b = 0; b < 2; ++b) {
@@ -1557,23 +1561,23 @@ long long pf_batch_iterations(const pf_batch* b) { return b ? b->iters : -1; }
 // error maximum and the pore counts accumulate over all slabs and one controller decides).
 
 namespace {
-// Pointers (local plane 0) of one slab's exchanged buffers: [theta, phi][y0, y1, ua, ub, y32_0, y32_1].
+// Pointers (local plane 0) of one slab's exchanged buffers: [theta, phi][y0, y1, ua, ub, y32_0, y32_1, k1, k3, k4].
 struct SlabTab {
-    void* f[2][6];
+    void* f[2][9];
     int n3;
     int pad;
 };
 
 // which: 0 = ua, 1 = ub (stage inputs written by the stage just run), 2 = y[cur ^ 1] (the step's
 // candidate state), 3 = y[cur] (the state), 4 = y32[cur ^ 1] (the binary32 copy of the candidate state
-// that stage 5 writes in the binary32 form of the full model).  blockIdx.y = cut * 4 + direction * 2 + field.
+// that stage 5 writes in the binary32 form of the full model), 5, 6, 7 = k1, k3, k4.  blockIdx.y = cut * 4 + direction * 2 + field.
 template <typename TF>
 __global__ void k_halo(const SlabTab* __restrict__ tab, long long plane, int which, int fields,
                        const Ctrl* __restrict__ c) {
     const int r = blockIdx.y;
     const int cut = r >> 2, dir = (r >> 1) & 1, f = r & 1;
     if (!((fields >> f) & 1)) return;
-    const int slot = which < 2 ? 2 + which : (which == 2 ? (c->cur ^ 1) : (which == 3 ? c->cur : 4 + (c->cur ^ 1)));
+    const int slot = which < 2 ? 2 + which : (which == 2 ? (c->cur ^ 1) : (which == 3 ? c->cur : (which == 4 ? 4 + (c->cur ^ 1) : which + 1)));
     const SlabTab& lo = tab[cut];
     const SlabTab& hi = tab[cut + 1];
     const TF* src;
@@ -1636,6 +1640,19 @@ static cudaError_t halo(pf_slabs* S, int which, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// The exchanges (see k_halo) after a stage: what a later stage reads beyond the cut.  Binary32 stages 2, 4 and 5 form
+// their inputs from the slopes (full model) or from u2 and the slopes (Temp and micro models).
+static std::vector<int> exchanges_after(const pf_grid* g, int stage) {
+    if (!is_f32(g)) return {stage == 5 ? 2 : (stage % 2 == 1 ? 0 : 1)};
+    switch (stage) {
+        case 1: return has_y32(g) ? std::vector<int>{5} : std::vector<int>{0, 5};
+        case 2: return {1};
+        case 3: return {6};
+        case 4: return {7};
+        default: return has_y32(g) ? std::vector<int>{2, 4} : std::vector<int>{2};
+    }
+}
+
 // One Merson attempt over all slabs: each stage on every slab, then the exchange of the planes the
 // next stage reads at the cuts; the controller once (shared control block).
 static cudaError_t slabs_enqueue_attempt(pf_slabs* S, cudaStream_t st) {
@@ -1644,9 +1661,10 @@ static cudaError_t slabs_enqueue_attempt(pf_slabs* S, cudaStream_t st) {
             cudaError_t e = launch_stage(g, stage, st);
             if (e != cudaSuccess) return e;
         }
-        cudaError_t e = halo(S, stage == 5 ? 2 : (stage % 2 == 1 ? 0 : 1), st);
-        if (e == cudaSuccess && stage == 5 && has_y32(S->s[0])) e = halo(S, 4, st);
-        if (e != cudaSuccess) return e;
+        for (int w : exchanges_after(S->s[0], stage)) {
+            const cudaError_t e = halo(S, w, st);
+            if (e != cudaSuccess) return e;
+        }
     }
     k_controller<<<1, 32, 0, st>>>(S->s[0]->dctrl);
     count_launch();
@@ -1654,8 +1672,9 @@ static cudaError_t slabs_enqueue_attempt(pf_slabs* S, cudaStream_t st) {
 }
 
 static long long slabs_attempt_launches(const pf_slabs* S) {
-    const int extra = (S->P > 1 && has_y32(S->s[0])) ? 1 : 0;
-    return 5LL * (S->P + (S->P > 1 ? 1 : 0)) + extra + 1;
+    long long n = 5LL * S->P + 1;
+    for (int stage = 1; stage <= 5 && S->P > 1; ++stage) n += (long long)exchanges_after(S->s[0], stage).size();
+    return n;
 }
 
 static void slabs_free_graph(pf_slabs* S) {
@@ -1738,6 +1757,8 @@ pf_status pf_slabs_create(int n1, int n2, int n3, double h, int model, int react
         t.f[1][0] = g->y_ph[0]; t.f[1][1] = g->y_ph[1]; t.f[1][2] = g->ua_ph; t.f[1][3] = g->ub_ph;
         t.f[0][4] = g->y32_th[0]; t.f[0][5] = g->y32_th[1];
         t.f[1][4] = g->y32_ph[0]; t.f[1][5] = g->y32_ph[1];
+        t.f[0][6] = g->k1_th; t.f[0][7] = g->k3_th; t.f[0][8] = g->k4_th;
+        t.f[1][6] = g->k1_ph; t.f[1][7] = g->k3_ph; t.f[1][8] = g->k4_ph;
         t.n3 = g->n3;
         t.pad = 0;
     }
@@ -1875,8 +1896,8 @@ pf_status pf_slabs_run_to(pf_slabs* S, double t_end, double tol, long long max_s
     // every replayed attempt exchanges the five stages' planes (attempts after the run ended copy
     // unchanged planes)
     long long per_attempt = 0;
-    for (int w : {0, 1, 0, 1, 2}) per_attempt += halo_exchange_bytes(S, w);
-    if (has_y32(S->s[0])) per_attempt += halo_exchange_bytes(S, 4);
+    for (int stage = 1; stage <= 5; ++stage)
+        for (int w : exchanges_after(S->s[0], stage)) per_attempt += halo_exchange_bytes(S, w);
     S->halo_bytes = replays * steps_per_graph * per_attempt;
     if (stats) {
         stats->n_accepted = c->n_acc;

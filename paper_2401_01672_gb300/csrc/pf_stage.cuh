@@ -17,7 +17,7 @@
 // column stay in registers.  The raw values of plane k+2 are loaded while plane
 // k is computed (three-plane shared-memory ring, one barrier per plane), and the
 // stage-combination operands are loaded before the right-hand-side arithmetic
-// (binary32 stages 2-4: one plane ahead), so memory latency overlaps computation.
+// (binary32 stage 2: one plane ahead), so memory latency overlaps computation.
 // Cells outside the grid are replaced by the nearest boundary cell (mirror ghost),
 // which makes the interior formula give zero flux on every face; Dirichlet faces
 // add their half-cell flux separately.  A z-slab of a multi-domain run instead reads
@@ -31,8 +31,8 @@
 //
 // Binary32 form (T = float): stage inputs chain from one stage input to the next
 // (u3 = u2 + dt/6 (k2 - k1), u4 = u2 - 5dt/24 k1 + 3dt/8 k3,
-// u5 = u4 + 3dt/8 k1 - 15dt/8 k3 + 2dt k4 -- algebraically the tableau rows) so that
-// only stages 1 and 5 touch the binary64 state; the state update y' = y + (dt/6 (k1 +
+// u5 = u4 + 3dt/8 k1 - 15dt/8 k3 + 2dt k4 -- algebraically the tableau rows; u4 and u5 are formed
+// where they are read and never stored) so that only stages 1 and 5 touch the binary64 state; the state update y' = y + (dt/6 (k1 +
 // 4k4 + k5)) adds a binary32 increment to binary64 y.  For the full model the chained quantities are
 // the increments d_s = u_s - y32 over a binary32 copy y32 of the state (set with the state, written by
 // stage 5 beside the candidate state, so stage 1 reads it instead of the binary64 state), and the
@@ -402,12 +402,23 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
         in_th = reinterpret_cast<const TIN*>(a.ub_th);
         in_ph = reinterpret_cast<const TIN*>(a.ub_ph);
     }
-    // increments: the stage buffer holds d, the values are read from y32
-    const T* in_dth = nullptr;
-    const T* in_dph = nullptr;
-    if constexpr (DIN) {
-        in_dth = reinterpret_cast<const T*>(in_th);
-        in_dph = reinterpret_cast<const T*>(in_ph);
+    // Binary32: only stages 1 and 2 write a stage input.  u4 and u5 are combinations of u2 and of the slopes that stages
+    // 4 and 5 read anyway, so every loader (halo cells too) forms them from NCH slopes and nothing is written for them:
+    // 188 bytes per cell and attempt in the full model instead of 252 (u2 - y = dt/3 k1 is formed from k1 too), 104
+    // instead of 120 in the micro model; the arithmetic is that of storing them, operation by operation.
+    constexpr bool CHAIN = F32 && STAGE >= 4;
+    constexpr int NCH = CHAIN ? STAGE - 1 : (DIN ? 1 : 0);
+    const T* ch_th[3] = {nullptr, nullptr, nullptr};
+    const T* ch_ph[3] = {nullptr, nullptr, nullptr};
+    if constexpr (CHAIN) {
+        in_th = reinterpret_cast<const TIN*>(a.ua_th);
+        in_ph = reinterpret_cast<const TIN*>(a.ua_ph);
+        ch_th[0] = a.k1_th; ch_th[1] = a.k3_th; ch_th[2] = a.k4_th;
+        ch_ph[0] = a.k1_ph; ch_ph[1] = a.k3_ph; ch_ph[2] = a.k4_ph;
+    }
+    if constexpr (DIN) {  // increments over y32: of stage 3 as stored, of the others from the slopes
+        ch_th[0] = STAGE == 3 ? a.ub_th : a.k1_th;
+        ch_ph[0] = STAGE == 3 ? a.ub_ph : a.k1_ph;
         in_th = reinterpret_cast<const TIN*>(a.y32_th[cur]);
         in_ph = reinterpret_cast<const TIN*>(a.y32_ph[cur]);
     }
@@ -431,39 +442,64 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
     const double* __restrict__ St_I = St + 8 * a.ncell;
     const long long NC = a.ncell;
     // raw loads of one cell of plane kk (clamped: mirror ghosts); G holds A_lam and B B_lam when STATIC
-    // (theta and phi stay in the input type until `cvt`, so that a conversion does not wait for its
-    // load where the load is issued)
-    auto fetch = [&](int kk, int off, TIN& th, TIN& ph, T& G, T& B, T& dt, T& dp) {
+    // (everything stays as loaded until `cvt`, so that no arithmetic waits for a load where it is issued)
+    struct Raw {
+        TIN th, ph;
+        T G, B;
+        T ct[NCH > 0 ? NCH : 1], cp[NCH > 0 ? NCH : 1];
+    };
+    auto fetch = [&](int kk, int off, Raw& r) {
         const int id = min(max(kk, a.cf.zlo), a.cf.zhi) * plane + off;
-        if constexpr (DIN) {
-            dt = in_dth[id];
-            dp = in_dph[id];
-        } else {
-            dt = T(0);
-            dp = T(0);
+#pragma unroll
+        for (int q = 0; q < NCH; ++q) {
+            if constexpr (HAS_TH) r.ct[q] = ch_th[q][id];
+            if constexpr (HAS_PH) r.cp[q] = ch_ph[q][id];
         }
         if constexpr (STATIC) {
-            G = T(St[id]);
-            B = T(St_B[id]);
+            r.G = T(St[id]);
+            r.B = T(St_B[id]);
         } else {
-            G = Gf[id];
-            B = T(0);
+            r.G = Gf[id];
+            r.B = T(0);
         }
-        if constexpr (HAS_TH) th = in_th[id];
-        else th = TIN(0);
-        if constexpr (HAS_PH) ph = in_ph[id];
-        else ph = TIN(0);
+        if constexpr (HAS_TH) r.th = in_th[id];
+        else r.th = TIN(0);
+        if constexpr (HAS_PH) r.ph = in_ph[id];
+        else r.ph = TIN(0);
     };
-    auto cvt = [&](TIN rth, TIN rph, T& th, T& ph) {
-        if constexpr (HAS_TH) th = to_T<T>(rth);
+    // u4 (or its increment) from u2 and k1, k3; u5 from u4 and k1, k3, k4
+    auto chain = [&](T u2, const T* c) {
+        T u = FMA(sc[3], c[1], FMA(-sc[8], c[0], u2));
+        if constexpr (STAGE == 5) u = FMA(sc[6], c[2], FMA(-sc[9], c[1], FMA(sc[3], c[0], u)));
+        return u;
+    };
+    auto incr = [&](const T* c) {
+        if constexpr (F32 && STAGE == 3) return c[0];
+        else if constexpr (F32 && CHAIN) return chain(__fmul_rn(sc[0], c[0]), c);
+        else if constexpr (F32) return __fmul_rn(sc[0], c[0]);
+        else return T(0);
+    };
+    auto cvt = [&](const Raw& r, T& th, T& ph, T& dt, T& dp) {
+        dt = T(0);
+        dp = T(0);
+        if constexpr (HAS_TH) th = to_T<T>(r.th);
         else th = K.theta_micro;
-        if constexpr (HAS_PH) ph = to_T<T>(rph);
+        if constexpr (HAS_PH) ph = to_T<T>(r.ph);
         else ph = T(0);
+        if constexpr (DIN) {
+            dt = incr(r.ct);
+            dp = incr(r.cp);
+        } else if constexpr (CHAIN) {
+            if constexpr (HAS_TH) th = chain(th, r.ct);
+            if constexpr (HAS_PH) ph = chain(ph, r.cp);
+        }
     };
     auto fetch_cvt = [&](int kk, int off, T& th, T& ph, T& G, T& B, T& dt, T& dp) {
-        TIN rth, rph;
-        fetch(kk, off, rth, rph, G, B, dt, dp);
-        cvt(rth, rph, th, ph);
+        Raw r;
+        fetch(kk, off, r);
+        cvt(r, th, ph, dt, dp);
+        G = r.G;
+        B = r.B;
     };
     // derived values: Temp phase field (eq. explicit-p-dependence-on-T) and blended conductivity (at
     // phi = y32 + d with increments)
@@ -533,25 +569,16 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
         nd_xy += ((dmask & 4) && j == 0) + ((dmask & 8) && j == n2 - 1);
     }
 
-    // Binary32 stages 2-4 move few bytes and do little arithmetic per cell, so memory latency
-    // bounds them: their stage-combination operands are loaded one plane ahead.  (Binary64 kernels
-    // are bound by the binary64 pipe, and binary32 stage 5 by its register budget: both load
-    // their operands within the plane.)
-    constexpr bool PF = F32 && STAGE >= 2 && STAGE <= 4;
-    T n_k1t = T(0), n_k1p = T(0), n_k3t = T(0), n_k3p = T(0), n_uat = T(0), n_uap = T(0);
+    // Binary32 stage 2 does little arithmetic per cell, so memory latency bounds it: its own operand is
+    // loaded one plane ahead.  (Binary64 kernels are bound by the binary64 pipe, and binary32 stage 5
+    // by its register budget: both load their operands within the plane.)
+    constexpr bool PF = F32 && STAGE == 2;
+    T n_k1t = T(0), n_k1p = T(0);
     if constexpr (PF) {
         if (inside && kb < ke) {
             const int q = kb * plane + j * n1 + i;
             if constexpr (HAS_TH) n_k1t = a.k1_th[q];
             if constexpr (HAS_PH) n_k1p = a.k1_ph[q];
-            if constexpr (STAGE == 3) {
-                if constexpr (HAS_TH) n_uat = a.ua_th[q];
-                if constexpr (HAS_PH) n_uap = a.ua_ph[q];
-            }
-            if constexpr (STAGE == 4) {
-                if constexpr (HAS_TH) n_k3t = a.k3_th[q];
-                if constexpr (HAS_PH) n_k3p = a.k3_ph[q];
-            }
         }
     }
 
@@ -589,10 +616,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
 #pragma unroll 3
     for (int k = kb; k < ke; ++k) {
         // 1. raw values of plane k+2 (consumed after the arithmetic of plane k)
-        TIN rth, rph, qth, qph;
-        T rG, rB, qG, qB, rdt, rdp, qdt, qdp;
-        fetch(k + 2, ooff, rth, rph, rG, rB, rdt, rdp);
-        if (hal) fetch(k + 2, hoff, qth, qph, qG, qB, qdt, qdp);
+        Raw rr, qq;
+        fetch(k + 2, ooff, rr);
+        if (hal) fetch(k + 2, hoff, qq);
 
         const int id = k * plane + j * n1 + i;
         // phase field of the lateral neighbours (Laplacian, gradient) and the bulk test
@@ -608,30 +634,21 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
         // 2. stage-combination operands of this cell
         T y_t = T(0), y_p = T(0), k1t = T(0), k1p = T(0), k3t = T(0), k3p = T(0), k4t = T(0), k4p = T(0);
         double y_t64 = 0.0, y_p64 = 0.0;
-        T ua_t = T(0), ua_p = T(0);
         T sW = T(0), sC0 = T(0), sC1 = T(0), sC2 = T(0), sD0 = T(0), sD1 = T(0), sIR = T(0);
         if constexpr (PF) {
-            // take the operands loaded during the previous plane, then load those of plane k+1
-            k1t = n_k1t; k1p = n_k1p; k3t = n_k3t; k3p = n_k3p; ua_t = n_uat; ua_p = n_uap;
+            // take the operand loaded during the previous plane, then load that of plane k+1
+            k1t = n_k1t; k1p = n_k1p;
             if (inside && k + 1 < ke) {
                 const int q = id + plane;
                 if constexpr (HAS_TH) n_k1t = a.k1_th[q];
                 if constexpr (HAS_PH) n_k1p = a.k1_ph[q];
-                if constexpr (STAGE == 3) {
-                    if constexpr (HAS_TH) n_uat = a.ua_th[q];
-                    if constexpr (HAS_PH) n_uap = a.ua_ph[q];
-                }
-                if constexpr (STAGE == 4) {
-                    if constexpr (HAS_TH) n_k3t = a.k3_th[q];
-                    if constexpr (HAS_PH) n_k3p = a.k3_ph[q];
-                }
             }
         } else if (inside) {
-            if constexpr (STAGE >= 2) {
+            if constexpr ((!F32 && STAGE >= 2) || STAGE == 5) {
                 if constexpr (HAS_TH) k1t = a.k1_th[id];
                 if constexpr (HAS_PH) k1p = a.k1_ph[id];
             }
-            if constexpr (STAGE >= 4) {
+            if constexpr ((!F32 && STAGE >= 4) || STAGE == 5) {
                 if constexpr (HAS_TH) k3t = a.k3_th[id];
                 if constexpr (HAS_PH) k3p = a.k3_ph[id];
             }
@@ -642,10 +659,6 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
             if constexpr (!F32 && STAGE >= 2 && STAGE <= 4) {
                 if constexpr (HAS_TH) y_t = a.y_th[cur][id];
                 if constexpr (HAS_PH) y_p = a.y_ph[cur][id];
-            }
-            if constexpr (F32 && STAGE == 3) {
-                if constexpr (HAS_TH) ua_t = a.ua_th[id];
-                if constexpr (HAS_PH) ua_p = a.ua_ph[id];
             }
             if constexpr (STATIC) {
                 // a cell whose dphi is exactly 0 with phi exactly 0 or 1 (bulk, or no water) needs only
@@ -812,8 +825,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
                 dph = dp * dth;
             }
 
-            // ---- fused stage combination (binary32 stages 2 and 4 continue from their own input: the
-            // increment with increments, else the stage value)
+            // ---- fused stage combination (binary32 stage 2 continues from its own input: the increment
+            // with increments, else the stage value)
             const T bth = DIN ? dtc : thc, bph = DIN ? dpc : phc;
             if constexpr (STAGE == 0) {
                 if (a.out_th) a.out_th[id] = dth;
@@ -821,9 +834,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
             } else if constexpr (STAGE == 1) {
                 if constexpr (INC) {
                     a.k1_th[id] = dth;
-                    a.ua_th[id] = sc[0] * dth;
                     a.k1_ph[id] = dph;
-                    a.ua_ph[id] = sc[0] * dph;
                 } else {
                     if constexpr (HAS_TH) { a.k1_th[id] = dth; a.ua_th[id] = FMA(sc[0], dth, thc); }
                     if constexpr (HAS_PH) { a.k1_ph[id] = dph; a.ua_ph[id] = FMA(sc[0], dph, phc); }
@@ -850,16 +861,16 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
                 }
             } else if constexpr (STAGE == 3) {
                 if constexpr (F32) {
-                    if constexpr (HAS_TH) { a.k3_th[id] = dth; a.ua_th[id] = FMA(sc[3], dth, FMA(-sc[8], k1t, ua_t)); }
-                    if constexpr (HAS_PH) { a.k3_ph[id] = dph; a.ua_ph[id] = FMA(sc[3], dph, FMA(-sc[8], k1p, ua_p)); }
+                    if constexpr (HAS_TH) a.k3_th[id] = dth;
+                    if constexpr (HAS_PH) a.k3_ph[id] = dph;
                 } else {
                     if constexpr (HAS_TH) { a.k3_th[id] = dth; a.ua_th[id] = FMA(sc[3], dth, FMA(sc[2], k1t, y_t)); }
                     if constexpr (HAS_PH) { a.k3_ph[id] = dph; a.ua_ph[id] = FMA(sc[3], dph, FMA(sc[2], k1p, y_p)); }
                 }
             } else if constexpr (STAGE == 4) {
                 if constexpr (F32) {
-                    if constexpr (HAS_TH) { a.k4_th[id] = dth; a.ub_th[id] = FMA(sc[6], dth, FMA(-sc[9], k3t, FMA(sc[3], k1t, bth))); }
-                    if constexpr (HAS_PH) { a.k4_ph[id] = dph; a.ub_ph[id] = FMA(sc[6], dph, FMA(-sc[9], k3p, FMA(sc[3], k1p, bph))); }
+                    if constexpr (HAS_TH) a.k4_th[id] = dth;
+                    if constexpr (HAS_PH) a.k4_ph[id] = dph;
                 } else {
                     if constexpr (HAS_TH) { a.k4_th[id] = dth; a.ub_th[id] = FMA(sc[6], dth, FMA(-sc[5], k3t, FMA(sc[4], k1t, y_t))); }
                     if constexpr (HAS_PH) { a.k4_ph[id] = dph; a.ub_ph[id] = FMA(sc[6], dph, FMA(-sc[5], k3p, FMA(sc[4], k1p, y_p))); }
@@ -893,19 +904,19 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
         // 3. finish plane k+2 into the ring slot of plane k-1; rotate the own column
         const int b2 = (b + 2) % 3;
         {
-            T cth, cph, lam2, tg2 = T(0);
-            cvt(rth, rph, cth, cph);
-            finish(cth, cph, rG, rB, lam2, tg2, rdp);
+            T cth, cph, lam2, rdt, rdp, tg2 = T(0);
+            cvt(rr, cth, cph, rdt, rdp);
+            finish(cth, cph, rr.G, rr.B, lam2, tg2, rdp);
             put(b2, ty + 1, tx + 1, cth, cph, lam2, rdt, rdp);
             thm = thc; phm = phc; lamm = lamc; tgm = tgc; dtm = dtc; dpm = dpc;
             thc = thp; phc = php; lamc = lamp; Gc = Gp; tgc = tgp; dtc = dtp; dpc = dpp;
-            thp = cth; php = cph; lamp = lam2; Gp = rG; tgp = tg2; dtp = rdt; dpp = rdp;
+            thp = cth; php = cph; lamp = lam2; Gp = rr.G; tgp = tg2; dtp = rdt; dpp = rdp;
         }
         if (hal) {
-            T h_th, h_ph, h_lam, h_tg;
-            cvt(qth, qph, h_th, h_ph);
-            finish(h_th, h_ph, qG, qB, h_lam, h_tg, qdp);
-            put(b2, hy + 1, hx + 1, h_th, h_ph, h_lam, qdt, qdp);
+            T h_th, h_ph, h_lam, h_tg, h_dt, h_dp;
+            cvt(qq, h_th, h_ph, h_dt, h_dp);
+            finish(h_th, h_ph, qq.G, qq.B, h_lam, h_tg, h_dp);
+            put(b2, hy + 1, hx + 1, h_th, h_ph, h_lam, h_dt, h_dp);
         }
         b = (b + 1) % 3;
         __syncthreads();
