@@ -167,7 +167,7 @@ pf_status pf_max_phase_rate(pf_grid* g, double* max_rate);
 pf_status pf_profile_stages(pf_grid* g, int n_attempts, double* stage_ms);
 
 /* Tile shape of the stage kernels: blocks of 32 x by threads (by = 4, 8 or 16) marching along z over
- * zc >= 1 planes.  Any shape gives the same results; only speed changes.  Default 8 x 32. */
+ * zc >= 1 planes.  Any shape gives the same results; only speed changes.  Default: by the grid's size. */
 pf_status pf_set_tiles(pf_grid* g, int by, int zc);
 pf_status pf_get_tiles(pf_grid* g, int* by, int* zc);
 

@@ -37,7 +37,8 @@ struct pf_grid {
     CoefT<float> k32{};
     cudaStream_t stream = nullptr;
     cudaStream_t cap_stream = nullptr;
-    int by = 8, zc = 32;
+    bool tiles_set = false;         // by pf_set_tiles or a tuner
+    int by = 4, zc = 8;             // until tiles are set or tuned: default_tiles
     double* y_th[2] = {nullptr, nullptr};
     double* y_ph[2] = {nullptr, nullptr};
     void* ua_th = nullptr; void* ua_ph = nullptr;
@@ -271,6 +272,7 @@ __device__ void controller_step(Ctrl* c) {
 }
 
 __global__ void k_controller(Ctrl* c) {
+    wait_for_previous_kernel();
     if (threadIdx.x == 0 && blockIdx.x == 0) controller_step(c);
 }
 
@@ -452,9 +454,30 @@ static StageArgs<T> make_args(pf_grid* g) {
     if constexpr (std::is_same<T, float>::value) a.G = g->G32;
     else a.G = g->G64;
     a.zc = g->zc;
+    const TileShape ts = tile_shape(g->n1, g->n2, g->by);
+    a.tw = ts.w;
+    a.th = ts.h;
     a.statics = g->statics;
     a.ncell = g->NA;
     return a;
+}
+
+// Tiles of a grid that nobody set or tuned: blocks of 32 x 4 threads (never slower than 8 by more than 3 %, 16 always),
+// and planes per block by the planes of tiles each place on the chip gets, m = plane tiles / resident blocks: a large grid
+// amortises a block's prologue (3 planes loaded, one block's latency) over many planes, a small one needs every block it
+// can get.  Measured best: binary64 1 plane at 32^3 and 64^3 (m = 2.2), 3 at 128^3 (m = 18), 5 to 12 at 256^3 (m = 144);
+// binary32 1 at 32^3, 3 at 64^3 (m = 1.9), 4 at 70^3, 10 at 128^3 (m = 15), 24 at 256^3; the formula stays within about
+// 8 % of the best of 24 shapes on nine grids of 32^3 to 256^3.  (32 planes of 32 x 8 threads everywhere: 302 us an attempt
+// at 32^3 in the binary64 micro model, now 23; 128^3 742 and 315 us.)
+static void default_tiles(const pf_grid* g, double plane_tiles, int* by, int* zc) {
+    *by = 4;
+    const double m = plane_tiles / (152.0 * (is_f32(g) ? 7 : 6));
+    const double z = (is_f32(g) ? 2.2 : 0.8) * std::sqrt(m);
+    *zc = z < 1.5 ? 1 : (z > 24.0 ? 24 : (int)(z + 0.5));
+}
+static double plane_tiles(const pf_grid* g, int by) {
+    const TileShape ts = tile_shape(g->n1, g->n2, by);
+    return (double)((g->n1 + ts.w - 1) / ts.w) * ((g->n2 + ts.h - 1) / ts.h) * g->n3;
 }
 
 static cudaError_t launch_stage(pf_grid* g, int stage, cudaStream_t s) {
@@ -469,10 +492,10 @@ static cudaError_t enqueue_attempt(pf_grid* g, cudaStream_t s) {
         cudaError_t e = launch_stage(g, st, s);
         if (e != cudaSuccess) return e;
     }
-    k_controller<<<1, 32, 0, s>>>(g->dctrl);
+    const cudaError_t e = launch_dependent(k_controller, dim3(1), dim3(32), s, g->dctrl);
     count_launch();
     g->launches++;
-    return cudaGetLastError();
+    return e;
 }
 
 static void free_graph(pf_grid* g) {
@@ -589,6 +612,7 @@ static pf_status create_impl(int n1, int n2, int n3, double h, int model, int re
     c.theta_freeze = p->theta_freeze; c.theta_thaw = p->theta_thaw; c.t_freeze = p->t_freeze;
     fill_coefs(g->k64, *p, h);
     fill_coefs(g->k32, *p, h);
+    default_tiles(g, plane_tiles(g, 4), &g->by, &g->zc);
     auto alloc = [&](size_t bytes) -> void* {
         void* q = nullptr;
         if (cudaMalloc(&q, bytes) != cudaSuccess) return nullptr;
@@ -604,8 +628,8 @@ static pf_status create_impl(int n1, int n2, int n3, double h, int model, int re
         ok = ok && q;
         return q ? q + esz * (size_t)(so.zg_lo * plane) : nullptr;
     };
-    // slopes: the binary32 stage kernels form u4 and u5 of the z neighbours from them
-    auto AK = [&]() -> void* { return is_f32(g) ? AG(sizeof(float)) : A(nf); };
+    // slopes: in the binary32 form of the full model the stage inputs of the z neighbours are formed from them
+    auto AK = [&]() -> void* { return is_f32(g) && model == PF_MODEL_FULL ? AG(sizeof(float)) : A(nf); };
     if (has_th(g)) {
         g->y_th[0] = (double*)AG(8); g->y_th[1] = (double*)AG(8);
         g->ua_th = AG(fbytes(g)); g->ub_th = AG(fbytes(g));
@@ -907,25 +931,39 @@ pf_status pf_rkm_step(pf_grid* g, double* dt_inout, double tol, int force_accept
     return PF_OK;
 }
 
+// Attempts in groups of 16 from a graph, what is left over (all of a short run) launched one by one: nothing is launched
+// past the attempts asked for, and a run of a few steps builds no graph.  A run of fixed steps cannot end early, so it is
+// only waited for at its end (and every 256 attempts, which bounds the launch queue); an adaptive one every 16 or 4.
 static pf_status run_loop(pf_grid* g, pf_run_stats* stats) {
+    constexpr int GROUP = 16;
     const long long want = g->hctrl->max_attempts;
-    const int steps_per_graph = want >= 16 ? 16 : (want >= 4 ? 4 : 1);
-    if (!g->graph || g->graph_steps != steps_per_graph) {
-        pf_status s = build_graph(g, steps_per_graph);
+    const bool fixed = g->hctrl->fixed;
+    if (want >= GROUP && (!g->graph || g->graph_steps != GROUP)) {
+        pf_status s = build_graph(g, GROUP);
         if (s != PF_OK) return s;
     }
-    long long launched = 0;
+    const long long before = g->launches;
     pf_status s = push_ctrl(g);
     if (s != PF_OK) return s;
-    for (;;) {
-        PF_CUDA(g, cudaGraphLaunch(g->graph, g->stream));
-        launched += 6LL * steps_per_graph;
+    for (long long left = want, since = 0; left > 0;) {
+        int n = GROUP;
+        if (left >= GROUP) {
+            PF_CUDA(g, cudaGraphLaunch(g->graph, g->stream));
+            count_launch(6LL * GROUP);
+            g->launches += 6LL * GROUP;
+        } else {
+            n = (int)(fixed ? left : std::min<long long>(left, 4));
+            for (int q = 0; q < n; ++q) PF_CUDA(g, enqueue_attempt(g, g->stream));
+        }
+        left -= n;
+        since += n;
+        if (fixed && left > 0 && since < 256) continue;
+        since = 0;
         s = sync_ctrl_to_host(g);
         if (s != PF_OK) return s;
         if (g->hctrl->done) break;
     }
-    count_launch(launched);
-    g->launches += launched;
+    const long long launched = g->launches - before;
     const Ctrl* c = g->hctrl;
     if (stats) {
         stats->n_accepted = c->n_acc;
@@ -1137,6 +1175,7 @@ static pf_status set_tiles_impl(pf_grid* g, int by, int zc) {
     if (by != 4 && by != 8 && by != 16) return fail(g, PF_E_INVALID, "by must be 4, 8 or 16");
     if (zc < 1) return fail(g, PF_E_INVALID, "zc must be >= 1");
     if (by != g->by || zc != g->zc) free_graph(g);
+    g->tiles_set = true;
     g->by = by;
     g->zc = zc;
     return PF_OK;
@@ -1304,7 +1343,8 @@ static pf_status batch_upload(pf_batch* b) {
     for (int q = 0; q < b->n; ++q) {
         pf_grid* g = b->g[q];
         g->by = b->by;
-        const int nbx = (g->n1 + TX - 1) / TX, nby = (g->n2 + b->by - 1) / b->by, nbz = (g->n3 + g->zc - 1) / g->zc;
+        const TileShape ts = tile_shape(g->n1, g->n2, b->by);
+        const int nbx = (g->n1 + ts.w - 1) / ts.w, nby = (g->n2 + ts.h - 1) / ts.h, nbz = (g->n3 + g->zc - 1) / g->zc;
         tiles[q] = make_int4(nbx, nby, nbz, nbx * nby * nbz);
     }
     PF_BCUDA(b, cudaMemcpy(b->d_tiles, tiles.data(), sizeof(int4) * b->n, cudaMemcpyHostToDevice));
@@ -1422,6 +1462,16 @@ pf_status pf_batch_create(int n, pf_grid* const* grids, pf_batch** out) {
     b->rx = grids[0]->rx;
     b->prec = grids[0]->prec;
     b->by = grids[0]->by;
+    // instances nobody set tiles for share the chip: their planes per block follow from the tiles of all
+    double total = 0.0;
+    for (int q = 0; q < n; ++q) total += plane_tiles(grids[q], b->by);
+    for (int q = 0; q < n; ++q)
+        if (!grids[q]->tiles_set) {
+            int by, zc;
+            default_tiles(grids[q], total, &by, &zc);
+            if (zc != grids[q]->zc) free_graph(grids[q]);
+            grids[q]->zc = zc;
+        }
     b->stream = grids[0]->stream;
     const size_t asz = b->prec == PF_PREC_FP32_FIELDS ? sizeof(StageArgs<float>) : sizeof(StageArgs<double>);
     bool ok = cudaMalloc(&b->d_args, asz * n) == cudaSuccess;
@@ -1640,16 +1690,16 @@ static cudaError_t halo(pf_slabs* S, int which, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// The exchanges (see k_halo) after a stage: what a later stage reads beyond the cut.  Binary32 stages 2, 4 and 5 form
-// their inputs from the slopes (full model) or from u2 and the slopes (Temp and micro models).
+// The exchanges (see k_halo) after a stage: what a later stage reads beyond the cut.  In the binary32 form of the full
+// model stages 2, 4 and 5 form their inputs from the slopes.
 static std::vector<int> exchanges_after(const pf_grid* g, int stage) {
-    if (!is_f32(g)) return {stage == 5 ? 2 : (stage % 2 == 1 ? 0 : 1)};
+    if (!has_y32(g)) return {stage == 5 ? 2 : (stage % 2 == 1 ? 0 : 1)};
     switch (stage) {
-        case 1: return has_y32(g) ? std::vector<int>{5} : std::vector<int>{0, 5};
+        case 1: return {5};
         case 2: return {1};
         case 3: return {6};
         case 4: return {7};
-        default: return has_y32(g) ? std::vector<int>{2, 4} : std::vector<int>{2};
+        default: return {2, 4};
     }
 }
 

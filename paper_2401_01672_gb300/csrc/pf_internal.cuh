@@ -117,6 +117,28 @@ struct BatchPlan {
     int tile_start[BATCH_MAX + 1];
 };
 
+// Lateral tile of a block of 32 x by threads: w <= 32 columns (the planes' pitch in shared memory) and h <= tile_rows(by)
+// rows (their shared memory) with w h <= 32 by.  32 x by, unless another shape keeps clearly more threads on cells: rows of
+// 50 cells take two tiles of 25 x 5 (0.98 of 128 threads on cells) where two of 32 x 4 leave 22 % of them idle, rows of 40
+// two of 21 x 6 (0.94 against 0.63).  The margin covers the narrower rows' loads, which start off 128-byte lines.
+constexpr int tile_rows(int by) { return by == 4 ? by + 2 : by + 1; }
+struct TileShape { int w, h; };
+inline TileShape tile_shape(int n1, int n2, int by) {
+    TileShape best{TX, by};
+    auto used = [&](int w, int h) {  // share of the threads that own a cell of the grid
+        return (double)n1 * n2 / ((double)((n1 + w - 1) / w) * ((n2 + h - 1) / h) * TX * by);
+    };
+    double most = used(TX, by) * 1.05;
+    for (int h = by + 1; h <= tile_rows(by); ++h) {
+        const int w = TX * by / h;
+        if (used(w, h) > most) {
+            most = used(w, h);
+            best = {w, h};
+        }
+    }
+    return best;
+}
+
 template <typename T>
 struct StageArgs {
     Coefs cf;
@@ -145,6 +167,7 @@ struct StageArgs {
     T* out_th; T* out_ph;
     double t_rhs;
     int zc;                  // planes per block along z
+    int tw, th;              // lateral tile (tile_shape)
 };
 
 // Launch one stage (0 = plain RHS, 1..5 = Merson stages) of the given model.
@@ -160,6 +183,29 @@ cudaError_t launch_batch_stage_f64(int model, int rx, int stage, const StageArgs
 cudaError_t launch_batch_stage_f32(int model, int rx, int stage, const StageArgs<float>* args,
                                    const BatchPlan* plan, const int4* tilegrid, int by, int blocks,
                                    cudaStream_t s);
+
+// Programmatic dependent launch: a kernel launched by launch_dependent may start once every block of the kernel before it
+// in the stream (or graph) has ended or called let_next_kernel_start, and wait_for_previous_kernel, the first thing it does,
+// holds it until that kernel has ended and its writes are visible.  The blocks' launch then overlaps the last stores and
+// reductions of the kernel before; between the short kernels of a small grid the gap is a large part of the time.  Blocks
+// call let_next_kernel_start at their end: called at their start, blocks that only wait took places on the SMs while the
+// kernel before still ran and then stayed unevenly spread (33 x 33 x 66 cells, Temp model: 140 us an attempt without
+// dependent launches, 420 us with early ones).
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A&&... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
 
 // Launch accounting (process-wide).
 void count_launch(long long n = 1);

@@ -10,14 +10,14 @@
 //   stage 5: k5 = F(u5), y' = y + dt/6 (k1 + 4k4 + k5), E = max |dt/30 (2k1 - 9k3 + 8k4 - k5)|
 // k2 and k5 are never stored.  Stage 0 is the plain right-hand side.
 //
-// Tiling: a block of 32 x BY threads owns a 32 x BY column of cells and marches
-// along z over ZC planes.  Plane k (with a one-cell lateral halo) sits in shared
+// Tiling: a block of 32 x BY threads owns a column of cells, 32 x BY or narrower and taller where that leaves fewer
+// threads idle (tile_shape), and marches along z over ZC planes.  Plane k (with a one-cell lateral halo) sits in shared
 // memory together with the blended conductivity of every cell, so each cell's
 // lambda is evaluated once per plane visit; the z neighbours of a thread's own
 // column stay in registers.  The raw values of plane k+2 are loaded while plane
 // k is computed (three-plane shared-memory ring, one barrier per plane), and the
 // stage-combination operands are loaded before the right-hand-side arithmetic
-// (binary32 stage 2: one plane ahead), so memory latency overlaps computation.
+// (binary32 stages 2-4: one plane ahead), so memory latency overlaps computation.
 // Cells outside the grid are replaced by the nearest boundary cell (mirror ghost),
 // which makes the interior formula give zero flux on every face; Dirichlet faces
 // add their half-cell flux separately.  A z-slab of a multi-domain run instead reads
@@ -31,8 +31,8 @@
 //
 // Binary32 form (T = float): stage inputs chain from one stage input to the next
 // (u3 = u2 + dt/6 (k2 - k1), u4 = u2 - 5dt/24 k1 + 3dt/8 k3,
-// u5 = u4 + 3dt/8 k1 - 15dt/8 k3 + 2dt k4 -- algebraically the tableau rows; u4 and u5 are formed
-// where they are read and never stored) so that only stages 1 and 5 touch the binary64 state; the state update y' = y + (dt/6 (k1 +
+// u5 = u4 + 3dt/8 k1 - 15dt/8 k3 + 2dt k4 -- algebraically the tableau rows; the full model forms u4
+// and u5 where they are read and never stores them) so that only stages 1 and 5 touch the binary64 state; the state update y' = y + (dt/6 (k1 +
 // 4k4 + k5)) adds a binary32 increment to binary64 y.  For the full model the chained quantities are
 // the increments d_s = u_s - y32 over a binary32 copy y32 of the state (set with the state, written by
 // stage 5 beside the candidate state, so stage 1 reads it instead of the binary64 state), and the
@@ -314,10 +314,10 @@ __device__ __forceinline__ void publish_block(Ctrl* ctrl, unsigned long long ebi
     }
 }
 
-// One tile (32 x BY columns, one z chunk) of one stage.  (bxi, byi, bzi) is the tile's position in
+// One tile (a lateral tile of up to 32 x BY columns, one z chunk) of one stage.  (bxi, byi, bzi) is the tile's position in
 // the grid's tile lattice.  Called by the single-grid kernel (one block per tile) and by the batched
 // persistent kernel (blocks loop over the tiles of all active instances).
-template <int MODEL, int RX, typename T, typename TIN, int STAGE, int BY>
+template <int MODEL, int RX, typename T, typename TIN, int STAGE, int BY, bool LAST>
 __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi, const int byi, const int bzi) {
     static_assert((STAGE == 1 && !(std::is_same<T, float>::value && MODEL == M_FULL))
                       ? std::is_same<TIN, double>::value : std::is_same<TIN, T>::value,
@@ -359,28 +359,33 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
     const CoefT<T>& K = a.k;
     const int n1 = a.cf.n1, n2 = a.cf.n2, n3 = a.cf.n3;
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const int i0 = bxi * TX, j0 = byi * BY;
-    const int i = i0 + tx, j = j0 + ty;
+    // the block's threads over a tile of tw x th cells in row order (tile_shape; threads past the last cell repeat it
+    // and store nothing)
+    const int tw = a.tw, th_ = a.th;
+    const int tid = ty * TX + tx;
+    const int tc = min(tid, tw * th_ - 1);
+    const int cy = tc / tw, cx = tc - cy * tw;
+    const int i0 = bxi * tw, j0 = byi * th_;
+    const int i = i0 + cx, j = j0 + cy;
     const int kb = bzi * a.zc;
     const int ke = min(kb + a.zc, n3);
-    const bool inside = (i < n1) && (j < n2);
+    const bool inside = (tid == tc) && (i < n1) && (j < n2);
     // 32-bit cell indices (grids are limited to fewer than 2^31 cells, ghost planes included, at creation)
     const int plane = n1 * n2;
     const int ooff = min(j, n2 - 1) * n1 + min(i, n1 - 1);
 
-    // one halo cell per thread for the first 2 TX + 2 BY threads: y rows, then x columns
-    const int tid = ty * TX + tx;
+    // one halo cell per thread for the first 2 tw + 2 th threads: y rows, then x columns
     bool hal = false;
     int hx = 0, hy = 0;
-    if (tid < 2 * TX) {
+    if (tid < 2 * tw) {
         hal = true;
-        hx = tid % TX;
-        hy = (tid < TX) ? -1 : BY;
-    } else if (tid < 2 * TX + 2 * BY) {
+        hx = tid < tw ? tid : tid - tw;
+        hy = (tid < tw) ? -1 : th_;
+    } else if (tid < 2 * tw + 2 * th_) {
         hal = true;
-        const int r = tid - 2 * TX;
-        hy = r % BY;
-        hx = (r < BY) ? -1 : TX;
+        const int r = tid - 2 * tw;
+        hy = r < th_ ? r : r - th_;
+        hx = (r < th_) ? -1 : tw;
     }
     const int hoff = min(max(j0 + hy, 0), n2 - 1) * n1 + min(max(i0 + hx, 0), n1 - 1);
 
@@ -402,19 +407,18 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
         in_th = reinterpret_cast<const TIN*>(a.ub_th);
         in_ph = reinterpret_cast<const TIN*>(a.ub_ph);
     }
-    // Binary32: only stages 1 and 2 write a stage input.  u4 and u5 are combinations of u2 and of the slopes that stages
-    // 4 and 5 read anyway, so every loader (halo cells too) forms them from NCH slopes and nothing is written for them:
-    // 188 bytes per cell and attempt in the full model instead of 252 (u2 - y = dt/3 k1 is formed from k1 too), 104
-    // instead of 120 in the micro model; the arithmetic is that of storing them, operation by operation.
-    constexpr bool CHAIN = F32 && STAGE >= 4;
+    // Increments: only stage 2 writes one (d3).  d2 = dt/3 k1, and d4 and d5 are combinations of d2 and of the slopes that
+    // stages 4 and 5 read anyway, so every loader (halo cells too) forms them from NCH slopes and nothing is written for
+    // them: 188 bytes per cell and attempt instead of 252; the arithmetic is that of storing them, operation by operation.
+    // (The same for the Temp and micro models was measured: fewer bytes, 104 for 120, but up to twice the loads per
+    // cell, and the kernels with one field are bound by issue: the 12-instance sweep 24.4 -> 28.8 ms.  They store u4, u5.)
+    constexpr bool CHAIN = DIN && STAGE >= 4;
     constexpr int NCH = CHAIN ? STAGE - 1 : (DIN ? 1 : 0);
     const T* ch_th[3] = {nullptr, nullptr, nullptr};
     const T* ch_ph[3] = {nullptr, nullptr, nullptr};
     if constexpr (CHAIN) {
-        in_th = reinterpret_cast<const TIN*>(a.ua_th);
-        in_ph = reinterpret_cast<const TIN*>(a.ua_ph);
-        ch_th[0] = a.k1_th; ch_th[1] = a.k3_th; ch_th[2] = a.k4_th;
-        ch_ph[0] = a.k1_ph; ch_ph[1] = a.k3_ph; ch_ph[2] = a.k4_ph;
+        ch_th[1] = a.k3_th; ch_th[2] = a.k4_th;
+        ch_ph[1] = a.k3_ph; ch_ph[2] = a.k4_ph;
     }
     if constexpr (DIN) {  // increments over y32: of stage 3 as stored, of the others from the slopes
         ch_th[0] = STAGE == 3 ? a.ub_th : a.k1_th;
@@ -424,7 +428,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
     }
     const T* __restrict__ Gf = a.G;
 
-    constexpr int SX = TX + 2, SY = BY + 2;
+    constexpr int SX = TX + 2, SY = tile_rows(BY) + 2;
     // with increments, each cell's (y32, d) pair of a field sits in one 8-byte entry (one shared load)
     constexpr bool TH1 = HAS_TH && !DIN;
     __shared__ T s_th[TH1 ? 3 : 1][TH1 ? SY : 1][TH1 ? SX : 1];
@@ -467,17 +471,16 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
         if constexpr (HAS_PH) r.ph = in_ph[id];
         else r.ph = TIN(0);
     };
-    // u4 (or its increment) from u2 and k1, k3; u5 from u4 and k1, k3, k4
-    auto chain = [&](T u2, const T* c) {
-        T u = FMA(sc[3], c[1], FMA(-sc[8], c[0], u2));
-        if constexpr (STAGE == 5) u = FMA(sc[6], c[2], FMA(-sc[9], c[1], FMA(sc[3], c[0], u)));
-        return u;
-    };
+    // d3 as stored; d2 from k1, d4 from d2 and k1, k3, d5 from d4 and k1, k3, k4
     auto incr = [&](const T* c) {
-        if constexpr (F32 && STAGE == 3) return c[0];
-        else if constexpr (F32 && CHAIN) return chain(__fmul_rn(sc[0], c[0]), c);
-        else if constexpr (F32) return __fmul_rn(sc[0], c[0]);
-        else return T(0);
+        if constexpr (!DIN) return T(0);
+        else if constexpr (STAGE == 3) return c[0];
+        else {
+            T d = __fmul_rn(sc[0], c[0]);
+            if constexpr (CHAIN) d = FMA(sc[3], c[1], FMA(-sc[8], c[0], d));
+            if constexpr (STAGE == 5) d = FMA(sc[6], c[2], FMA(-sc[9], c[1], FMA(sc[3], c[0], d)));
+            return d;
+        }
     };
     auto cvt = [&](const Raw& r, T& th, T& ph, T& dt, T& dp) {
         dt = T(0);
@@ -489,9 +492,6 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
         if constexpr (DIN) {
             dt = incr(r.ct);
             dp = incr(r.cp);
-        } else if constexpr (CHAIN) {
-            if constexpr (HAS_TH) th = chain(th, r.ct);
-            if constexpr (HAS_PH) ph = chain(ph, r.cp);
         }
     };
     auto fetch_cvt = [&](int kk, int off, T& th, T& ph, T& G, T& B, T& dt, T& dp) {
@@ -569,17 +569,25 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
         nd_xy += ((dmask & 4) && j == 0) + ((dmask & 8) && j == n2 - 1);
     }
 
-    // Binary32 stage 2 does little arithmetic per cell, so memory latency bounds it: its own operand is
-    // loaded one plane ahead.  (Binary64 kernels are bound by the binary64 pipe, and binary32 stage 5
-    // by its register budget: both load their operands within the plane.)
-    constexpr bool PF = F32 && STAGE == 2;
-    T n_k1t = T(0), n_k1p = T(0);
-    if constexpr (PF) {
-        if (inside && kb < ke) {
-            const int q = kb * plane + j * n1 + i;
-            if constexpr (HAS_TH) n_k1t = a.k1_th[q];
-            if constexpr (HAS_PH) n_k1p = a.k1_ph[q];
+    // Binary32 stages 2-4 do little arithmetic per cell, so memory latency bounds them: their own operands
+    // (with increments only stage 2 has one) are loaded one plane ahead.  (Binary64 kernels are bound by the binary64
+    // pipe, and binary32 stage 5 by its register budget: both load their operands within the plane.)
+    constexpr bool PF = F32 && STAGE >= 2 && STAGE <= (INC ? 2 : 4);
+    T n_k1t = T(0), n_k1p = T(0), n_k3t = T(0), n_k3p = T(0), n_uat = T(0), n_uap = T(0);
+    auto operands_ahead = [&](int q) {
+        if constexpr (HAS_TH) n_k1t = a.k1_th[q];
+        if constexpr (HAS_PH) n_k1p = a.k1_ph[q];
+        if constexpr (STAGE == 3) {
+            if constexpr (HAS_TH) n_uat = a.ua_th[q];
+            if constexpr (HAS_PH) n_uap = a.ua_ph[q];
         }
+        if constexpr (STAGE == 4) {
+            if constexpr (HAS_TH) n_k3t = a.k3_th[q];
+            if constexpr (HAS_PH) n_k3p = a.k3_ph[q];
+        }
+    };
+    if constexpr (PF) {
+        if (inside && kb < ke) operands_ahead(kb * plane + j * n1 + i);
     }
 
     // ---- prologue: own column at kb-1, kb, kb+1; planes kb, kb+1 into the ring
@@ -592,10 +600,10 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
         finish(thm, phm, Gm, Bm, lamm, tgm, dpm);
         fetch_cvt(kb, ooff, thc, phc, Gc, Bc, dtc, dpc);
         finish(thc, phc, Gc, Bc, lamc, tgc, dpc);
-        put(0, ty + 1, tx + 1, thc, phc, lamc, dtc, dpc);
+        put(0, cy + 1, cx + 1, thc, phc, lamc, dtc, dpc);
         fetch_cvt(kb + 1, ooff, thp, php, Gp, Bp, dtp, dpp);
         finish(thp, php, Gp, Bp, lamp, tgp, dpp);
-        put(1, ty + 1, tx + 1, thp, php, lamp, dtp, dpp);
+        put(1, cy + 1, cx + 1, thp, php, lamp, dtp, dpp);
         if (hal) {
             T h_th, h_ph, h_G, h_B, h_lam, h_tg, h_dt, h_dp;
             fetch_cvt(kb, hoff, h_th, h_ph, h_G, h_B, h_dt, h_dp);
@@ -627,22 +635,19 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
         T p_xm = T(0), p_xp = T(0), p_ym = T(0), p_yp = T(0);
         bool bulk = false;
         if constexpr (!TEMP && !F32) {
-            p_xm = s_ph[b][ty + 1][tx]; p_xp = s_ph[b][ty + 1][tx + 2];
-            p_ym = s_ph[b][ty][tx + 1]; p_yp = s_ph[b][ty + 2][tx + 1];
+            p_xm = s_ph[b][cy + 1][cx]; p_xp = s_ph[b][cy + 1][cx + 2];
+            p_ym = s_ph[b][cy][cx + 1]; p_yp = s_ph[b][cy + 2][cx + 1];
             bulk = uniform_01(phc, p_xm, p_xp, p_ym, p_yp, phm, php);
         }
         // 2. stage-combination operands of this cell
         T y_t = T(0), y_p = T(0), k1t = T(0), k1p = T(0), k3t = T(0), k3p = T(0), k4t = T(0), k4p = T(0);
         double y_t64 = 0.0, y_p64 = 0.0;
+        T ua_t = T(0), ua_p = T(0);
         T sW = T(0), sC0 = T(0), sC1 = T(0), sC2 = T(0), sD0 = T(0), sD1 = T(0), sIR = T(0);
         if constexpr (PF) {
-            // take the operand loaded during the previous plane, then load that of plane k+1
-            k1t = n_k1t; k1p = n_k1p;
-            if (inside && k + 1 < ke) {
-                const int q = id + plane;
-                if constexpr (HAS_TH) n_k1t = a.k1_th[q];
-                if constexpr (HAS_PH) n_k1p = a.k1_ph[q];
-            }
+            // take the operands loaded during the previous plane, then load those of plane k+1
+            k1t = n_k1t; k1p = n_k1p; k3t = n_k3t; k3p = n_k3p; ua_t = n_uat; ua_p = n_uap;
+            if (inside && k + 1 < ke) operands_ahead(id + plane);
         } else if (inside) {
             if constexpr ((!F32 && STAGE >= 2) || STAGE == 5) {
                 if constexpr (HAS_TH) k1t = a.k1_th[id];
@@ -677,12 +682,12 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
         if (inside) {
             if constexpr (MODEL != M_MICRO) {
                 T t_xm, t_xp, t_ym, t_yp, d_xm, d_xp, d_ym, d_yp;
-                nb_th(b, ty + 1, tx, t_xm, d_xm);
-                nb_th(b, ty + 1, tx + 2, t_xp, d_xp);
-                nb_th(b, ty, tx + 1, t_ym, d_ym);
-                nb_th(b, ty + 2, tx + 1, t_yp, d_yp);
-                const T l_xm = s_lam[b][ty + 1][tx], l_xp = s_lam[b][ty + 1][tx + 2];
-                const T l_ym = s_lam[b][ty][tx + 1], l_yp = s_lam[b][ty + 2][tx + 1];
+                nb_th(b, cy + 1, cx, t_xm, d_xm);
+                nb_th(b, cy + 1, cx + 2, t_xp, d_xp);
+                nb_th(b, cy, cx + 1, t_ym, d_ym);
+                nb_th(b, cy + 2, cx + 1, t_yp, d_yp);
+                const T l_xm = s_lam[b][cy + 1][cx], l_xp = s_lam[b][cy + 1][cx + 2];
+                const T l_ym = s_lam[b][cy][cx + 1], l_yp = s_lam[b][cy + 2][cx + 1];
                 // theta_j - theta_c; with increments (y32_j - y32_c) + (d_j - d_c)
                 T g_xm = t_xm - thc, g_xp = t_xp - thc, g_ym = t_ym - thc, g_yp = t_yp - thc;
                 T g_zm = thm - thc, g_zp = thp - thc, g_b = th_b - thc;
@@ -751,7 +756,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
                 }
                 const int slot = base + __popc(m & ((1u << tx) - 1u));
                 if (need) {
-                    s_slot_xy[slot] = tx | (ty << 8);
+                    s_slot_xy[slot] = cx | (cy << 8);
                     s_slot[0][slot] = phm;
                     s_slot[1][slot] = php;
                     s_slot[2][slot] = thc;
@@ -788,10 +793,10 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
             } else if (need) {
                 T q_xm = T(0), q_xp = T(0), q_ym = T(0), q_yp = T(0);
                 if constexpr (F32) {
-                    nb_ph(b, ty + 1, tx, p_xm, q_xm);
-                    nb_ph(b, ty + 1, tx + 2, p_xp, q_xp);
-                    nb_ph(b, ty, tx + 1, p_ym, q_ym);
-                    nb_ph(b, ty + 2, tx + 1, p_yp, q_yp);
+                    nb_ph(b, cy + 1, cx, p_xm, q_xm);
+                    nb_ph(b, cy + 1, cx + 2, p_xp, q_xp);
+                    nb_ph(b, cy, cx + 1, p_ym, q_ym);
+                    nb_ph(b, cy + 2, cx + 1, p_yp, q_yp);
                 }
                 if constexpr (DIN)
                     dph = allen_cahn_rate_inc<RX>(K, phc, dpc, p_xm, p_xp, p_ym, p_yp, phm, php, q_xm, q_xp, q_ym, q_yp,
@@ -825,8 +830,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
                 dph = dp * dth;
             }
 
-            // ---- fused stage combination (binary32 stage 2 continues from its own input: the increment
-            // with increments, else the stage value)
+            // ---- fused stage combination (binary32 stages 2 and 4 continue from their own input: the
+            // increment with increments, else the stage value)
             const T bth = DIN ? dtc : thc, bph = DIN ? dpc : phc;
             if constexpr (STAGE == 0) {
                 if (a.out_th) a.out_th[id] = dth;
@@ -863,6 +868,10 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
                 if constexpr (F32) {
                     if constexpr (HAS_TH) a.k3_th[id] = dth;
                     if constexpr (HAS_PH) a.k3_ph[id] = dph;
+                    if constexpr (!INC) {
+                        if constexpr (HAS_TH) a.ua_th[id] = FMA(sc[3], dth, FMA(-sc[8], k1t, ua_t));
+                        if constexpr (HAS_PH) a.ua_ph[id] = FMA(sc[3], dph, FMA(-sc[8], k1p, ua_p));
+                    }
                 } else {
                     if constexpr (HAS_TH) { a.k3_th[id] = dth; a.ua_th[id] = FMA(sc[3], dth, FMA(sc[2], k1t, y_t)); }
                     if constexpr (HAS_PH) { a.k3_ph[id] = dph; a.ua_ph[id] = FMA(sc[3], dph, FMA(sc[2], k1p, y_p)); }
@@ -871,6 +880,10 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
                 if constexpr (F32) {
                     if constexpr (HAS_TH) a.k4_th[id] = dth;
                     if constexpr (HAS_PH) a.k4_ph[id] = dph;
+                    if constexpr (!INC) {
+                        if constexpr (HAS_TH) a.ub_th[id] = FMA(sc[6], dth, FMA(-sc[9], k3t, FMA(sc[3], k1t, bth)));
+                        if constexpr (HAS_PH) a.ub_ph[id] = FMA(sc[6], dph, FMA(-sc[9], k3p, FMA(sc[3], k1p, bph)));
+                    }
                 } else {
                     if constexpr (HAS_TH) { a.k4_th[id] = dth; a.ub_th[id] = FMA(sc[6], dth, FMA(-sc[5], k3t, FMA(sc[4], k1t, y_t))); }
                     if constexpr (HAS_PH) { a.k4_ph[id] = dph; a.ub_ph[id] = FMA(sc[6], dph, FMA(-sc[5], k3p, FMA(sc[4], k1p, y_p))); }
@@ -907,7 +920,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
             T cth, cph, lam2, rdt, rdp, tg2 = T(0);
             cvt(rr, cth, cph, rdt, rdp);
             finish(cth, cph, rr.G, rr.B, lam2, tg2, rdp);
-            put(b2, ty + 1, tx + 1, cth, cph, lam2, rdt, rdp);
+            put(b2, cy + 1, cx + 1, cth, cph, lam2, rdt, rdp);
             thm = thc; phm = phc; lamm = lamc; tgm = tgc; dtm = dtc; dpm = dpc;
             thc = thp; phc = php; lamc = lamp; Gc = Gp; tgc = tgp; dtc = dtp; dpc = dpp;
             thp = cth; php = cph; lamp = lam2; Gp = rr.G; tgp = tg2; dtp = rdt; dpp = rdp;
@@ -922,6 +935,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
         __syncthreads();
     }
 
+    if constexpr (LAST) let_next_kernel_start();  // the block's only tile: stores are issued, the reductions remain
     publish_block<STAGE, HAS_PH, F32, BY>(ctrl, ebits, icount, pcount, rbits);
     __syncthreads();  // the block may start another tile: shared memory is reused
     (void)tgm;
@@ -930,7 +944,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& a, const int bxi,
 template <int MODEL, int RX, typename T, typename TIN, int STAGE, int BY>
 __global__ void __launch_bounds__(TX * BY)
 stage_kernel(const StageArgs<T> a) {
-    stage_tile<MODEL, RX, T, TIN, STAGE, BY>(a, blockIdx.x, blockIdx.y, blockIdx.z);
+    wait_for_previous_kernel();
+    stage_tile<MODEL, RX, T, TIN, STAGE, BY, true>(a, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 // Binary64 form: resident blocks per SM the register bound is set for: 24 warps for blocks of 32 x 4 and
@@ -938,13 +953,14 @@ stage_kernel(const StageArgs<T> a) {
 // faster than 16 warps at 128 registers with 32 x 4, 3.5 % with 32 x 8; 28 and 32 warps slower), one
 // block of 32 x 16 (16 warps at 128 registers; one 8-warp block at 136 registers was slower).  The
 // binary32 kernels keep the compiler's own register choice (an explicit bound, even of one block, made
-// it take more registers).
+// it take more registers), but for stage 5 of the full model, where it took 96 (20 resident warps).
 constexpr int f64_min_blocks(int by) { return by <= 8 ? 24 / by : 1; }
 
 template <int MODEL, int RX, typename T, typename TIN, int STAGE, int BY>
 __global__ void __launch_bounds__(TX * BY, f64_min_blocks(BY))
 stage_kernel_r128(const StageArgs<T> a) {
-    stage_tile<MODEL, RX, T, TIN, STAGE, BY>(a, blockIdx.x, blockIdx.y, blockIdx.z);
+    wait_for_previous_kernel();
+    stage_tile<MODEL, RX, T, TIN, STAGE, BY, true>(a, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 // Batched persistent form: a fixed grid of blocks walks, in order, the tiles of the instances
@@ -959,7 +975,7 @@ __device__ __forceinline__ void batch_tiles(const StageArgs<T>* __restrict__ arg
         const int inst = plan->inst[s];
         const int local = t - plan->tile_start[s];
         const int4 tg = tilegrid[inst];
-        stage_tile<MODEL, RX, T, TIN, STAGE, BY>(args[inst], local % tg.x, (local / tg.x) % tg.y,
+        stage_tile<MODEL, RX, T, TIN, STAGE, BY, false>(args[inst], local % tg.x, (local / tg.x) % tg.y,
                                                   local / (tg.x * tg.y));
     }
 }
@@ -980,30 +996,31 @@ batch_stage_kernel_r128(const StageArgs<T>* __restrict__ args, const BatchPlan* 
 
 // ---------------------------------------------------------------- launchers (one per field type)
 template <typename T, int MODEL, int RX, int STAGE, int BY>
-void launch_one(const StageArgs<T>& a, dim3 grid, cudaStream_t s) {
+cudaError_t launch_one(const StageArgs<T>& a, dim3 grid, cudaStream_t s) {
     using TIN = typename std::conditional<STAGE == 1 && !(std::is_same<T, float>::value && MODEL == M_FULL), double,
                                           T>::type;
-    if constexpr (std::is_same<T, double>::value)
-        stage_kernel_r128<MODEL, RX, T, TIN, STAGE, BY><<<grid, dim3(TX, BY), 0, s>>>(a);
+    if constexpr (std::is_same<T, double>::value || (MODEL == M_FULL && STAGE == 5))
+        return launch_dependent(stage_kernel_r128<MODEL, RX, T, TIN, STAGE, BY>, grid, dim3(TX, BY), s, a);
     else
-        stage_kernel<MODEL, RX, T, TIN, STAGE, BY><<<grid, dim3(TX, BY), 0, s>>>(a);
+        return launch_dependent(stage_kernel<MODEL, RX, T, TIN, STAGE, BY>, grid, dim3(TX, BY), s, a);
 }
 
 template <typename T, int MODEL, int RX, int BY>
 cudaError_t launch_by(int stage, const StageArgs<T>& a, cudaStream_t s) {
     const int n1 = a.cf.n1, n2 = a.cf.n2, n3 = a.cf.n3;
-    dim3 grid((n1 + TX - 1) / TX, (n2 + BY - 1) / BY, (n3 + a.zc - 1) / a.zc);
+    dim3 grid((n1 + a.tw - 1) / a.tw, (n2 + a.th - 1) / a.th, (n3 + a.zc - 1) / a.zc);
+    cudaError_t e;
     switch (stage) {
-        case 0: launch_one<T, MODEL, RX, 0, BY>(a, grid, s); break;
-        case 1: launch_one<T, MODEL, RX, 1, BY>(a, grid, s); break;
-        case 2: launch_one<T, MODEL, RX, 2, BY>(a, grid, s); break;
-        case 3: launch_one<T, MODEL, RX, 3, BY>(a, grid, s); break;
-        case 4: launch_one<T, MODEL, RX, 4, BY>(a, grid, s); break;
-        case 5: launch_one<T, MODEL, RX, 5, BY>(a, grid, s); break;
+        case 0: e = launch_one<T, MODEL, RX, 0, BY>(a, grid, s); break;
+        case 1: e = launch_one<T, MODEL, RX, 1, BY>(a, grid, s); break;
+        case 2: e = launch_one<T, MODEL, RX, 2, BY>(a, grid, s); break;
+        case 3: e = launch_one<T, MODEL, RX, 3, BY>(a, grid, s); break;
+        case 4: e = launch_one<T, MODEL, RX, 4, BY>(a, grid, s); break;
+        case 5: e = launch_one<T, MODEL, RX, 5, BY>(a, grid, s); break;
         default: return cudaErrorInvalidValue;
     }
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 template <typename T, int MODEL, int RX, int STAGE, int BY>
