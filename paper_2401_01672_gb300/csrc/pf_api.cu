@@ -197,8 +197,9 @@ __global__ void k_temp_phi(const double* __restrict__ th, const double* __restri
 // current state (measured in stage 1) has stayed within eq_rel_tol x (pore-bulk cells) of a reference
 // value for eq_window seconds and, when eq_rate > 0, the largest |dphi/dt| over the pore-bulk cells of
 // that state is at most eq_rate (the state is then the one at t_eq = t).
-__device__ void controller_step(Ctrl* c) {
-    if (c->done) return;
+// Returns whether another step follows (its dt_step is set, its coefficients are not yet).
+__device__ bool controller_step(Ctrl* c) {
+    if (c->done) return false;
     const double E = __longlong_as_double((long long)c->err_bits);
     const long long cnt = (long long)c->ice_count;
     const double tolc = c->eq_rel_tol * (double)c->pore_count;
@@ -218,7 +219,7 @@ __device__ void controller_step(Ctrl* c) {
             c->t_eq = c->t;
             c->accepted = 0;
             c->done = 1;
-            return;
+            return false;
         }
     }
     const bool finite = E <= DBL_MAX;
@@ -227,7 +228,7 @@ __device__ void controller_step(Ctrl* c) {
     if (!finite && !c->fixed) {
         c->status = PF_E_NONFINITE;
         c->done = 1;
-        return;
+        return false;
     }
     if (accept) {
         c->t = c->land ? c->target : c->t + c->dt_step;
@@ -250,13 +251,13 @@ __device__ void controller_step(Ctrl* c) {
         if (!c->fixed && dn < c->dt_min) {
             c->status = PF_E_DT_UNDERFLOW;
             c->done = 1;
-            return;
+            return false;
         }
     }
-    if (c->single) return;
+    if (c->single) return false;
     if (c->t >= c->t_end || c->n_acc + c->n_rej >= c->max_attempts) {
         c->done = 1;
-        return;
+        return false;
     }
     double target = c->t_end;
     if (c->t < c->t_freeze && c->t_freeze < target) target = c->t_freeze;
@@ -268,39 +269,87 @@ __device__ void controller_step(Ctrl* c) {
         c->dt_step = c->dt;
         c->land = 0;
     }
-    prepare_step(c);
+    return true;
+}
+
+// Step control by one warp.  One thread alone spent a round trip to memory on each of the control block's fields it decides
+// on and ten binary64 divisions, one after another, on the next step's coefficients; the block is copied to shared memory
+// and back by the whole warp, and each lane takes one coefficient (the same products and quotients as prepare_step).
+__device__ void controller_warp(Ctrl* c, Ctrl* sh) {
+    constexpr int WORDS = (int)(sizeof(Ctrl) / 8);
+    static_assert(sizeof(Ctrl) % 8 == 0, "the control block is copied in 8-byte words");
+    const int lane = threadIdx.x & 31;
+    for (int q = lane; q < WORDS; q += 32) ((unsigned long long*)sh)[q] = ((const unsigned long long*)c)[q];
+    __syncwarp();
+    if (sh->done) return;
+    int more = 0;
+    if (lane == 0) more = controller_step(sh);
+    __syncwarp();
+    if (__shfl_sync(0xffffffffu, more, 0)) {
+        if (lane < NSC) {
+            const double mul[NSC] = {1.0, 1.0, 1.0, 3.0, 1.0, 1.5, 2.0, 1.0, 5.0, 15.0};
+            const double den[NSC] = {3.0, 6.0, 8.0, 8.0, 2.0, 1.0, 1.0, 30.0, 24.0, 8.0};
+            double m = mul[0], d = den[0];
+#pragma unroll
+            for (int q = 1; q < NSC; ++q)
+                if (lane == q) { m = mul[q]; d = den[q]; }
+            const double v = m * sh->dt_step / d;
+            sh->sc[lane] = v;
+            sh->scf[lane] = (float)v;
+        }
+        if (lane == 31) {
+            sh->theta_b = (sh->t < sh->t_freeze) ? sh->theta_freeze : sh->theta_thaw;
+            sh->theta_bf = (float)sh->theta_b;
+        }
+        __syncwarp();
+    }
+    for (int q = lane; q < WORDS; q += 32) ((unsigned long long*)c)[q] = ((const unsigned long long*)sh)[q];
 }
 
 __global__ void k_controller(Ctrl* c) {
     wait_for_previous_kernel();
-    if (threadIdx.x == 0 && blockIdx.x == 0) controller_step(c);
+    __shared__ Ctrl sh;
+    controller_warp(c, &sh);
 }
 
-// Batched step control: one thread per active instance.
-__global__ void k_batch_controller(Ctrl* const* ctrls, const BatchPlan* plan) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < plan->nactive) controller_step(ctrls[plan->inst[s]]);
+// Batched step control: one warp per active instance.
+constexpr int BC_WARPS = 4;
+__global__ void __launch_bounds__(32 * BC_WARPS) k_batch_controller(Ctrl* const* ctrls, const BatchPlan* plan) {
+    __shared__ Ctrl sh[BC_WARPS];
+    const int w = threadIdx.x >> 5, s = blockIdx.x * BC_WARPS + w;
+    if (s < plan->nactive) controller_warp(ctrls[plan->inst[s]], &sh[w]);
 }
 
-// Rebuild the batched work list from the instances' done flags and decide whether the device-side
-// loop runs another step (at most max_iter steps, so the loop always ends).
-__global__ void k_batch_plan(Ctrl* const* ctrls, const int4* tilegrid, int n, BatchPlan* plan,
-                             cudaGraphConditionalHandle cond) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    int nt = 0, na = 0;
-    for (int q = 0; q < n; ++q) {
-        if (!ctrls[q]->done) {
-            plan->inst[na] = q;
-            plan->tile_start[na] = nt;
-            nt += tilegrid[q].w;
-            ++na;
-        }
+// Rebuild the batched work list from the instances' done flags and decide whether the device-side loop runs another step
+// (at most max_iter steps, so the loop always ends).  A thread per instance and a prefix sum: one thread walking the list
+// waited for memory twice per instance.
+__global__ void __launch_bounds__(BATCH_MAX) k_batch_plan(Ctrl* const* ctrls, const int4* tilegrid, int n, BatchPlan* plan,
+                                                          cudaGraphConditionalHandle cond) {
+    __shared__ int s_act[BATCH_MAX], s_tiles[BATCH_MAX];
+    const int q = threadIdx.x;
+    const int act = q < n && !ctrls[q]->done, tiles = act ? tilegrid[q].w : 0;
+    s_act[q] = act;
+    s_tiles[q] = tiles;
+    __syncthreads();
+    for (int o = 1; o < BATCH_MAX; o <<= 1) {  // inclusive sums
+        const int a = q >= o ? s_act[q - o] : 0, t = q >= o ? s_tiles[q - o] : 0;
+        __syncthreads();
+        s_act[q] += a;
+        s_tiles[q] += t;
+        __syncthreads();
     }
-    plan->tile_start[na] = nt;
-    plan->ntiles = nt;
-    plan->nactive = na;
-    plan->iter += 1;
-    cudaGraphSetConditional(cond, (na > 0 && plan->iter <= plan->max_iter) ? 1u : 0u);
+    if (act) {
+        plan->inst[s_act[q] - 1] = q;
+        plan->tile_start[s_act[q] - 1] = s_tiles[q] - tiles;
+    }
+    if (q == 0) {
+        const int na = s_act[BATCH_MAX - 1], nt = s_tiles[BATCH_MAX - 1];
+        plan->tile_start[na] = nt;
+        plan->ntiles = nt;
+        plan->nactive = na;
+        plan->iter += 1;
+        cudaGraphSetConditional(cond, (na > 0 && plan->iter <= plan->max_iter) ? 1u : 0u);
+    }
 }
 
 // UWC partial sums over a half-open box; one slot of 4 words per block:
@@ -1371,8 +1420,8 @@ static cudaError_t batch_enqueue_step(pf_batch* b, cudaStream_t s, int blocks, c
                                        b->by, blocks, s);
     }
     if (e != cudaSuccess) return e;
-    k_batch_controller<<<(BATCH_MAX + 127) / 128, 128, 0, s>>>(b->d_ctrls, b->d_plan);
-    k_batch_plan<<<1, 32, 0, s>>>(b->d_ctrls, b->d_tiles, b->n, b->d_plan, h);
+    k_batch_controller<<<(b->n + BC_WARPS - 1) / BC_WARPS, 32 * BC_WARPS, 0, s>>>(b->d_ctrls, b->d_plan);
+    k_batch_plan<<<1, BATCH_MAX, 0, s>>>(b->d_ctrls, b->d_tiles, b->n, b->d_plan, h);
     count_launch(2);
     return cudaGetLastError();
 }
@@ -1392,7 +1441,7 @@ static pf_status batch_build_graph(pf_batch* b) {
     const int blocks = sms * (2048 / (TX * b->by)) / 2;
     if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(b->cap, graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        k_batch_plan<<<1, 32, 0, b->cap>>>(b->d_ctrls, b->d_tiles, b->n, b->d_plan, h);
+        k_batch_plan<<<1, BATCH_MAX, 0, b->cap>>>(b->d_ctrls, b->d_tiles, b->n, b->d_plan, h);
         cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = e2;
