@@ -348,6 +348,7 @@ __global__ void __launch_bounds__(BATCH_MAX) k_batch_plan(Ctrl* const* ctrls, co
         plan->ntiles = nt;
         plan->nactive = na;
         plan->iter += 1;
+        for (int k = 0; k < 6; ++k) plan->next[k] = 0;
         cudaGraphSetConditional(cond, (na > 0 && plan->iter <= plan->max_iter) ? 1u : 0u);
     }
 }
@@ -1409,15 +1410,15 @@ static pf_status batch_upload(pf_batch* b) {
     return PF_OK;
 }
 
-static cudaError_t batch_enqueue_step(pf_batch* b, cudaStream_t s, int blocks, cudaGraphConditionalHandle h) {
+static cudaError_t batch_enqueue_step(pf_batch* b, cudaStream_t s, int sms, cudaGraphConditionalHandle h) {
     cudaError_t e = cudaSuccess;
     for (int st = 1; st <= 5 && e == cudaSuccess; ++st) {
         if (b->prec == PF_PREC_FP32_FIELDS)
             e = launch_batch_stage_f32(b->model, b->rx, st, (const StageArgs<float>*)b->d_args, b->d_plan, b->d_tiles,
-                                       b->by, blocks, s);
+                                       b->by, sms, s);
         else
             e = launch_batch_stage_f64(b->model, b->rx, st, (const StageArgs<double>*)b->d_args, b->d_plan, b->d_tiles,
-                                       b->by, blocks, s);
+                                       b->by, sms, s);
     }
     if (e != cudaSuccess) return e;
     k_batch_controller<<<(b->n + BC_WARPS - 1) / BC_WARPS, 32 * BC_WARPS, 0, s>>>(b->d_ctrls, b->d_plan);
@@ -1434,11 +1435,9 @@ static pf_status batch_build_graph(pf_batch* b) {
     PF_BCUDA(b, cudaGraphCreate(&graph, 0));
     cudaGraphConditionalHandle h;
     cudaError_t e = cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault);
-    // persistent stage grid: enough blocks to fill every SM (the blocks loop over tiles)
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int blocks = sms * (2048 / (TX * b->by)) / 2;
     if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(b->cap, graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         k_batch_plan<<<1, BATCH_MAX, 0, b->cap>>>(b->d_ctrls, b->d_tiles, b->n, b->d_plan, h);
@@ -1460,7 +1459,7 @@ static pf_status batch_build_graph(pf_batch* b) {
         cudaGraph_t body = cp.conditional.phGraph_out[0];
         e = cudaStreamBeginCaptureToGraph(b->cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            cudaError_t e1 = batch_enqueue_step(b, b->cap, blocks, h);
+            cudaError_t e1 = batch_enqueue_step(b, b->cap, sms, h);
             cudaError_t e2 = cudaStreamEndCapture(b->cap, &body);
             e = e1 != cudaSuccess ? e1 : e2;
         }

@@ -113,6 +113,7 @@ struct BatchPlan {
     int nactive;
     int iter;
     int max_iter;
+    int next[6];  // per stage: tiles handed out beyond the first of each block
     int inst[BATCH_MAX];
     int tile_start[BATCH_MAX + 1];
 };
@@ -178,10 +179,10 @@ cudaError_t launch_stage_f32(int model, int rx, int stage, const StageArgs<float
                              cudaStream_t s);
 
 cudaError_t launch_batch_stage_f64(int model, int rx, int stage, const StageArgs<double>* args,
-                                   const BatchPlan* plan, const int4* tilegrid, int by, int blocks,
+                                   BatchPlan* plan, const int4* tilegrid, int by, int sms,
                                    cudaStream_t s);
 cudaError_t launch_batch_stage_f32(int model, int rx, int stage, const StageArgs<float>* args,
-                                   const BatchPlan* plan, const int4* tilegrid, int by, int blocks,
+                                   BatchPlan* plan, const int4* tilegrid, int by, int sms,
                                    cudaStream_t s);
 
 // Programmatic dependent launch: a kernel launched by launch_dependent may start once every block of the kernel before it

@@ -8,9 +8,9 @@ cudaError_t launch_stage_f64(int model, int rx, int stage, const StageArgs<doubl
     return launch_stage_t<double>(model, rx, stage, a, by, s);
 }
 
-cudaError_t launch_batch_stage_f64(int model, int rx, int stage, const StageArgs<double>* args, const BatchPlan* plan,
-                                   const int4* tg, int by, int blocks, cudaStream_t s) {
-    return launch_batch_stage_t<double>(model, rx, stage, args, plan, tg, by, blocks, s);
+cudaError_t launch_batch_stage_f64(int model, int rx, int stage, const StageArgs<double>* args, BatchPlan* plan,
+                                   const int4* tg, int by, int sms, cudaStream_t s) {
+    return launch_batch_stage_t<double>(model, rx, stage, args, plan, tg, by, sms, s);
 }
 
 }  // namespace pfgb
