@@ -28,6 +28,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <mutex>
 
@@ -147,6 +148,33 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(r[q]);
 }
 
+// sixteen output channels of one cell at element offset `at`: bf16, or fp32 (added to what is there when accumulating)
+__device__ __forceinline__ void store_cell16(bf16* y, float* yf, long long at, int accumulate, const float (&o)[16]) {
+    if (yf) {
+        float4* dst = reinterpret_cast<float4*>(yf + at);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float4 w = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+            if (accumulate) {
+                const float4 r = dst[q];
+                w.x += r.x; w.y += r.y; w.z += r.z; w.w += r.w;
+            }
+            dst[q] = w;
+        }
+    } else {
+        uint4 pk[2];
+        uint32_t* u = reinterpret_cast<uint32_t*>(pk);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(o[2 * q], o[2 * q + 1]);
+            u[q] = *reinterpret_cast<const uint32_t*>(&h2);
+        }
+        uint4* dst = reinterpret_cast<uint4*>(y + at);
+        dst[0] = pk[0];
+        dst[1] = pk[1];
+    }
+}
+
 __global__ void __launch_bounds__(UTHR)
 k_conv_umma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const UmmaArgs p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -257,29 +285,7 @@ k_conv_umma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 #pragma unroll
             for (int q = 0; q < 16; ++q) o[q] = fmaxf(o[q], 0.f);
         }
-        if (p.yf) {
-            float4* dst = reinterpret_cast<float4*>(p.yf + v * p.ldy + p.yoff + c0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                float4 w = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
-                if (p.accumulate) {
-                    const float4 r = dst[q];
-                    w.x += r.x; w.y += r.y; w.z += r.z; w.w += r.w;
-                }
-                dst[q] = w;
-            }
-        } else {
-            uint4 pk[2];
-            uint32_t* u = reinterpret_cast<uint32_t*>(pk);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const __nv_bfloat162 h2 = __floats2bfloat162_rn(o[2 * q], o[2 * q + 1]);
-                u[q] = *reinterpret_cast<const uint32_t*>(&h2);
-            }
-            uint4* dst = reinterpret_cast<uint4*>(p.y + v * p.ldy + p.yoff + c0);
-            dst[0] = pk[0];
-            dst[1] = pk[1];
-        }
+        store_cell16(p.y, p.yf, v * p.ldy + p.yoff + c0, p.accumulate, o);
     }
 
     // after a failed wait, the TMA loads still in flight must land before the block's shared memory
@@ -296,35 +302,43 @@ k_conv_umma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     }
 }
 
-// ---------------------------------------------------------------- narrow layers: one halo tile per brick
-// For 16 or 32 channels the per-tap boxes of k_conv_umma are 32- or 64-byte rows and the 27 boxes of a
-// 128-voxel tile move 27 times its input through TMA.  Here a block loads the input of its whole brick
-// (8 x 16 x DZ cells, x fastest) once, with a one-cell halo: a (DZ + 2) x 18 x 10 tile per 8-channel
-// chunk, unswizzled, so that every cell is a 16-byte row and a row of 10 cells is 160 contiguous bytes.
-// The A operand is a window of that tile: for tile plane z' and lateral offset (dy, dx), the 128 rows
-// (8 x by 16 y) start at cell (dx + 1, dy + 1, z'); 8 consecutive x cells are one 8 x 16-byte core
-// matrix, consecutive y rows are 160 bytes apart (the stride between core matrices along M) and
-// consecutive 8-channel chunks one chunk apart (the stride along K); the start is a multiple of 16 bytes,
-// as the unswizzled layout requires.  One window serves the three taps (dz = -1, 0, +1) of its (dy, dx):
-// tile plane z' feeds output planes o = z' - 1 - dz.  The B operand stacks the three taps' weights along
-// N (3 cout rows: dz = -1, 0, +1), and the accumulators of the output planes lie in TMEM at decreasing
-// columns, plane o at (DZ + 1 - o) cout, so the three column groups of one MMA are the accumulators of
-// planes z', z' - 1 and z' - 2 (planes -2, -1, DZ and DZ + 1 are scratch).  Per brick: (DZ + 2) x 9 x
-// cin/16 MMAs of M = 128, N = 3 cout, K = 16 (a third of the A reads from shared memory of one MMA per
-// tap); the accumulators start from zero written by tcgen05.st.  The weights of all taps stay in shared
-// memory as [dy, dx][chunk][dz, cout][8 channels]; backward data (flipped taps) copies tap 26 - t there.
-struct HaloArgs {
-    int cin, cout, dz_planes;     // channels in/out, output planes per brick
+// ---------------------------------------------------------------- layers whose weights fit: marching bricks
+// For cin x cout up to 2048 the weights of all taps stay in shared memory and a brick's input is loaded once, with a
+// one-cell halo, instead of 27 shifted boxes per 128 voxels (k_conv_umma: bound by that traffic from L2, 775 us for
+// 64 -> 32 channels on 128^3 voxels).  A brick is 8 x 16 columns of dz planes; its tile planes (10 x 18 cells, dz + 2 of
+// them) come one by one through a ring of shared-memory slots, each written by one TMA box (zeros outside the grid) as
+// rows of the cin channels of a cell (32, 64 or 128 bytes), swizzled with the span of a row.  (One box of
+// 16-byte rows per 8 channels, unswizzled, took twice as long to load as the MMAs to run.)
+//   A window of a plane at lateral offset (dy, dx) is the A operand: 128 rows (8 x by 16 y) from cell (dx + 1, dy + 1); 8
+// consecutive x cells are an 8-row group, the next y row is 10 rows further.  The swizzle is a function of the address and
+// the planes start on 1024 bytes, the longest pattern's period, so a window may start at any row.
+//   One window serves the three taps dz of its (dy, dx): tile plane z' feeds the output planes o = z' - 1 - dz.  The B
+// operand stacks the three taps' weights along N ([dy, dx][8-channel chunk][dz, cout][8 channels], unswizzled; backward data
+// copies tap 26 - t there), and the accumulators of the planes lie in TMEM at decreasing columns, so the column groups of
+// one MMA (N = 3 cout; 1 or 2 cout at the ends of the brick) are the accumulators of planes z', z' - 1, z' - 2.  Every output
+// adds its products tap by tap in the order dz, dy, dx, channels.  MIRROR: backward data with the planes from the top down
+// and the windows reversed, so that the products are added in the order of the weights' taps (as k_conv_umma does)
+// without a flipped copy; used with 64 channels on a side, the flipped copy with 16 and 32.
+//   Persistent: the blocks walk the bricks with a stride of the grid.  Warp 0 loads planes ahead, warp 1 issues MMAs, warps
+// 2-5 store the accumulators of one brick while the next brick's MMAs fill the other set, so loads, MMAs and stores
+// overlap (the form with one brick per block ran them one after another where only one block fits an SM).
+//   Shared-memory reads bound it: an MMA reads 4 KB of A and 32 bytes per column of B, 43 clocks for N = 48 at 128 bytes a
+// clock against 24 of multiplications.  Before (one brick per block, or
+// k_conv_umma) and now: 256^3 voxels 16 -> 16 channels 390 and 325 us, 32 -> 16 958 and 470; 128^3 32 -> 32 305 and 96 us,
+// 64 -> 32 772 and 179 (1296 TFLOP/s); 64^3 32 -> 64 109 and 37 us.
+struct MarchArgs {
+    int cin, cout;                // channels in/out
+    int dz;                       // output planes per brick
+    int slots;                    // tile plane slots
     int D, H, W;                  // grid of one sample
     int tx, ty, tz;               // bricks per sample
     int flip, relu, accumulate;
-    int withhold;                 // >= 0: the tile loads are withheld (failure-path test)
-    long long tries;
-    unsigned chunk_bytes;         // shared bytes of one 8-channel chunk of the tile (1024-byte multiple)
-    unsigned tile_bytes;          // all chunks
+    int withhold;                 // >= 0: this plane of every brick is not loaded (failure-path test)
+    long long tries, items;
+    unsigned plane_bytes, plane_tx;  // slot pitch (1024-byte multiple), bytes a plane's load delivers
     unsigned w_bytes;             // weights of all taps
-    unsigned tx_bytes;            // bytes the tile loads deliver
-    unsigned idesc;
+    unsigned idesc;               // MMA instruction descriptor without N
+    unsigned long long a_hi;      // constant part of the A descriptors
     int tmem_cols;
     const float* bias;
     const bf16* w;
@@ -333,9 +347,11 @@ struct HaloArgs {
     int ldy, yoff;
 };
 
+constexpr int MR_THR = 192;    // warp 0: TMA, warp 1: MMA, warps 2-5: epilogue
+constexpr int MR_SLOTS = 8;    // most plane slots
+
 constexpr int HB_X = 8, HB_Y = 16;            // brick extent along x and y (one plane = 128 voxels)
 constexpr int HT_X = HB_X + 2, HT_Y = HB_Y + 2;
-constexpr unsigned HT_ROW = HT_X * 16;        // bytes of one tile row of 8 channels
 
 // unswizzled K-major descriptor: start, stride along K (LBO) and along M/N (SBO), version 1
 __host__ __device__ __forceinline__ uint64_t desc_plain(uint32_t addr, uint32_t lbo, uint32_t sbo) {
@@ -356,55 +372,37 @@ __device__ __forceinline__ void umma_f16_w(uint32_t tmem_d, uint32_t alo, uint32
         : "memory");
 }
 
-// The MMAs of one brick.  a_lo / b_lo: low descriptor words of the tile and weight bases; the start field
-// (bits 0-13, 16-byte units) is advanced by adding to the low word (the shared window lies below 256 KB,
-// so it never carries out).
-template <int NKB>
-__device__ __forceinline__ void halo_issue(uint32_t tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                           uint32_t idesc, int planes, int cout, uint32_t chunk16) {
-    for (int zt = 0; zt < planes + 2; ++zt) {
-        const uint32_t d = tmem + (uint32_t)((planes + 1 - zt) * cout);  // accumulator of output plane zt
-        const uint32_t a_z = a_lo + (uint32_t)(zt * HT_Y * HT_X);
-#pragma unroll
-        for (int l = 0; l < 9; ++l) {  // l = 3 (dy + 1) + (dx + 1)
-            const uint32_t off = (uint32_t)((l / 3) * HT_X + l % 3);
-#pragma unroll
-            for (int kb = 0; kb < NKB; ++kb)
-                umma_f16_w(d, a_z + off + (uint32_t)(2 * kb) * chunk16, a_hi,
-                           b_lo + (uint32_t)((l * 2 * NKB + 2 * kb) * 3 * cout), b_hi, idesc, 1u);
-        }
-    }
+// The issuing warps below run their loops with all 32 lanes, and only the MMA and commit instructions are predicated on one
+// elected lane: addresses and descriptors are then the same for the warp, and the compiler keeps them in uniform
+// registers, where tcgen05.mma takes them from.  (In a branch for one thread every MMA moved its operands there first: about 60
+// clocks per MMA and 700 to 900 per tile plane: 64 -> 32 channels on 128^3 voxels 229 us, 128 -> 64 on 64^3 223 us; with
+// uniform operands 188 and 124 us.)
+__device__ __forceinline__ uint32_t elect_lane() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e;
 }
-
-// Weights of all taps into shared memory as [dy, dx][chunk][dz, cout][8] (tap t = 9 (dz + 1) + l,
-// l = 3 (dy + 1) + (dx + 1); flipped: the tap 26 - t), in rounds of 7 16-byte vectors per thread: each
-// round loads all of its vectors (read-only path) before storing them, so the copy costs one round trip
-// to L2 per 14 KB (one for 16 x 16 channels, four for 32 x 32).
-__device__ __forceinline__ void halo_weights(const bf16* __restrict__ w, unsigned char* dst, int cout, int nkc,
-                                             int flip) {
-    constexpr int CAP = 7;
-    const int nvec = 27 * cout * nkc;
-    const uint4* src = reinterpret_cast<const uint4*>(w);
-    for (int base = 0; base < nvec; base += CAP * UTHR) {
-        uint4 v[CAP];
-#pragma unroll
-        for (int j = 0; j < CAP; ++j) {
-            const int q = base + threadIdx.x + j * UTHR;
-            if (q < nvec) v[j] = __ldg(src + q);
-        }
-#pragma unroll
-        for (int j = 0; j < CAP; ++j) {
-            const int q = base + threadIdx.x + j * UTHR;
-            if (q < nvec) {
-                const int kc = q % nkc;
-                const int co = (q / nkc) % cout;
-                int t = q / (nkc * cout);
-                if (flip) t = 26 - t;
-                const int dzi = t / 9, l = t % 9;
-                *reinterpret_cast<uint4*>(dst + ((size_t)(l * nkc + kc) * 3 * cout + dzi * cout + co) * 16) = v[j];
-            }
-        }
-    }
+__device__ __forceinline__ void umma_elected(uint32_t lane, uint32_t tmem_d, uint32_t alo, uint32_t ahi, uint32_t blo,
+                                             uint32_t bhi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "setp.ne.b32 q, %7, 0;\n\t"
+        "mov.b64 da, {%1, %2};\n\t"
+        "mov.b64 db, {%3, %4};\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}" ::"r"(tmem_d),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate), "r"(lane)
+        : "memory");
+}
+__device__ __forceinline__ void commit_elected(uint32_t lane, uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar),
+        "r"(lane)
+        : "memory");
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, long long tries) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, tries));
 }
 
 // zero the accumulator columns [0, cols) of this warp's TMEM lane quadrant
@@ -418,132 +416,219 @@ __device__ __forceinline__ void tmem_zero(uint32_t taddr, int cols) {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-// One block per brick: thread 0 issues the tile's TMA loads (one box per 8-channel chunk, zero fill
-// outside the grid) while all threads copy the weights; thread 32 issues the MMAs once the tile has
-// landed and commits them to one barrier; all four warps read the accumulators (bias and ReLU applied
-// from registers).  Three or two blocks share an SM (shared memory), so one block's loads overlap
-// another's MMAs and epilogue.  Both waits are bounded.
-__global__ void __launch_bounds__(UTHR)
-k_conv_halo(const __grid_constant__ CUtensorMap tmX, const HaloArgs p) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    unsigned char* sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    unsigned char* ctl = sm + p.tile_bytes + p.w_bytes;
-    const uint32_t full = smem_u32(ctl);
-    const uint32_t accum = full + 8u;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ctl + 16);
-    __shared__ int s_fail;
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nkc = p.cin / 8;
-    long long b = blockIdx.x;
-    const int bx = (int)(b % p.tx);
-    b /= p.tx;
-    const int by = (int)(b % p.ty);
-    b /= p.ty;
-    const int bz = (int)(b % p.tz);
-    const int bn = (int)(b / p.tz);
-    const int x0 = bx * HB_X, y0 = by * HB_Y, z0 = bz * p.dz_planes;
-    const uint32_t tile0 = smem_u32(sm);
-    const uint32_t w0 = tile0 + p.tile_bytes;
-
-    if (threadIdx.x == 0) {
-        mbar_init(full, 1);
-        mbar_init(accum, 1);
-        s_fail = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        mbar_expect_tx(full, p.tx_bytes);
-        if (p.withhold < 0) {  // failure-path test: the tile never arrives
-            for (int kc = 0; kc < nkc; ++kc)
-                tma_load_5d(tile0 + (uint32_t)kc * p.chunk_bytes, &tmX, full, kc * 8, x0 - 1, y0 - 1, z0 - 1, bn);
+// Weights of all taps into shared memory as [dy, dx][chunk][dz, cout][8] (tap t = 9 (dz + 1) + l,
+// l = 3 (dy + 1) + (dx + 1); flipped: the tap 26 - t), in rounds of 7 16-byte vectors per thread: each
+// round loads all of its vectors (read-only path) before storing them, so the copy costs one round trip
+// to L2 per 14 KB (one for 16 x 16 channels, four for 32 x 32).
+__device__ __forceinline__ void halo_weights(const bf16* __restrict__ w, unsigned char* dst, int cout, int nkc,
+                                             int flip) {
+    constexpr int CAP = 7;
+    const int nvec = 27 * cout * nkc;
+    const uint4* src = reinterpret_cast<const uint4*>(w);
+    for (int base = 0; base < nvec; base += CAP * MR_THR) {
+        uint4 v[CAP];
+#pragma unroll
+        for (int j = 0; j < CAP; ++j) {
+            const int q = base + threadIdx.x + j * MR_THR;
+            if (q < nvec) v[j] = __ldg(src + q);
+        }
+#pragma unroll
+        for (int j = 0; j < CAP; ++j) {
+            const int q = base + threadIdx.x + j * MR_THR;
+            if (q < nvec) {
+                const int kc = q % nkc;
+                const int co = (q / nkc) % cout;
+                int t = q / (nkc * cout);
+                if (flip) t = 26 - t;
+                const int dzi = t / 9, l = t % 9;
+                *reinterpret_cast<uint4*>(dst + ((size_t)(l * nkc + kc) * 3 * cout + dzi * cout + co) * 16) = v[j];
+            }
         }
     }
-    if (warp == 2) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+}
+
+struct Brick {
+    int x0, y0, z0, n, planes;  // planes: output planes inside the grid
+};
+__device__ __forceinline__ Brick brick_of(const MarchArgs& p, long long q) {
+    Brick r;
+    r.x0 = (int)(q % p.tx) * HB_X;
+    q /= p.tx;
+    r.y0 = (int)(q % p.ty) * HB_Y;
+    q /= p.ty;
+    r.z0 = (int)(q % p.tz) * p.dz;
+    r.n = (int)(q / p.tz);
+    r.planes = min(p.dz, p.D - r.z0);
+    return r;
+}
+
+// The MMAs of one tile plane: a, b: low descriptor words (the start field, bits 0-13 in 16-byte units, is advanced by adding
+// to them; the shared window lies below 256 KB, so it never carries out).  d: accumulator of the first column group; idesc
+// with N.  The accumulators start from zeros that the storing warps write: starting them by MMAs that overwrite
+// takes an MMA per column group first.
+template <int CK, bool MIRROR>
+__device__ __forceinline__ void march_issue(uint32_t lane, uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi,
+                                            uint32_t idesc, int cout) {
+    const uint32_t bk = 6u * (uint32_t)cout;  // two 8-channel chunks of 3 cout rows
+    uint32_t bl = b;
+#pragma unroll
+    for (int l = 0; l < 9; ++l) {
+        const int at = MIRROR ? 8 - l : l;
+        const uint32_t win = a + (uint32_t)(((at / 3) * HT_X + at % 3) * (CK / 8));
+#pragma unroll
+        for (int k = 0; k < CK / 16; ++k, bl += bk)
+            umma_elected(lane, d, win + 2u * k, a_hi, bl, b_hi, idesc, 1u);
+    }
+}
+
+template <int CK, bool MIRROR>
+__global__ void __launch_bounds__(MR_THR)
+k_conv_march(const __grid_constant__ CUtensorMap tmX, const MarchArgs p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned char* sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const uint32_t tile0 = smem_u32(sm), w0 = tile0 + (uint32_t)p.slots * p.plane_bytes;
+    // barriers: plane full, plane empty, accumulators full, empty, all MMAs retired
+    __shared__ __align__(8) unsigned long long bars[2 * MR_SLOTS + 5];
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int s_fail;
+    const uint32_t pfull = smem_u32(bars), pempty = pfull + 8 * MR_SLOTS, afull = pempty + 8 * MR_SLOTS;
+    const uint32_t aempty = afull + 16, retired = aempty + 16;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int q = 0; q < 2 * MR_SLOTS; ++q) mbar_init(pfull + 8u * q, 1);
+        for (int q = 0; q < 2; ++q) {
+            mbar_init(afull + 8u * q, 1);
+            mbar_init(aempty + 8u * q, 4);
+        }
+        mbar_init(retired, 1);
+        s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                      "r"(p.tmem_cols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    halo_weights(p.w, sm + p.tile_bytes, p.cout, nkc, p.flip);
+    halo_weights(p.w, sm + (size_t)p.slots * p.plane_bytes, p.cout, CK / 8, p.flip);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();  // the TMEM address is in shared memory
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    tmem_zero(*tmem_slot + ((uint32_t)(warp * 32) << 16), (p.dz_planes + 4) * p.cout);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+    const uint32_t set_cols = (uint32_t)p.tmem_cols / 2u;
 
-    if (threadIdx.x == 32) {
-        const bool ok = mbar_wait(full, 0u, p.tries);
-        if (ok) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t da = desc_plain(tile0, p.chunk_bytes, HT_ROW);
-            const uint64_t db = desc_plain(w0, 3u * (uint32_t)p.cout * 16u, 128u);
-            const uint32_t alo = (uint32_t)da, ahi = (uint32_t)(da >> 32), blo = (uint32_t)db, bhi = (uint32_t)(db >> 32);
-            const uint32_t c16 = p.chunk_bytes >> 4;
-            if (nkc == 2) halo_issue<1>(tmem, alo, ahi, blo, bhi, p.idesc, p.dz_planes, p.cout, c16);
-            else halo_issue<2>(tmem, alo, ahi, blo, bhi, p.idesc, p.dz_planes, p.cout, c16);
-        } else {
-            s_fail = 1;
+    uint32_t filled = 0, phase = 0, pending = 0;  // producer, per slot: filled before, phase of the next fill, load issued
+    if (threadIdx.x == 0) {
+        bool ok = true;
+        int slot = 0;
+        for (long long q = blockIdx.x; q < p.items && ok; q += gridDim.x) {
+            const Brick br = brick_of(p, q);
+            for (int z = 0; z < br.planes + 2; ++z) {
+                const uint32_t bit = 1u << slot;
+                if (filled & bit) ok = mbar_wait(pempty + 8u * slot, ((phase >> slot) & 1u) ^ 1u, p.tries);
+                if (!ok || s_fail) { ok = false; break; }
+                mbar_expect_tx(pfull + 8u * slot, p.plane_tx);
+                if (z != p.withhold) {
+                    tma_load_5d(tile0 + (uint32_t)slot * p.plane_bytes, &tmX, pfull + 8u * slot, 0, br.x0 - 1, br.y0 - 1,
+                                br.z0 - 1 + (MIRROR ? br.planes + 1 - z : z), br.n);
+                    pending |= bit;
+                } else {
+                    pending &= ~bit;
+                }
+                filled |= bit;
+                phase ^= bit;
+                slot = slot + 1 == p.slots ? 0 : slot + 1;
+            }
         }
-        umma_commit(accum);  // also after a failed wait: every issued MMA has retired when it completes
+    } else if (warp == 1) {
+        const uint32_t one = elect_lane();
+        bool ok = true;
+        uint32_t ph = 0;
+        int slot = 0, k = 0;
+        const uint64_t db = desc_plain(w0, 3u * (uint32_t)p.cout * 16u, 128u);
+        const uint32_t blo = (uint32_t)db, bhi = (uint32_t)(db >> 32);
+        for (long long q = blockIdx.x; q < p.items && ok; q += gridDim.x, ++k) {
+            const Brick br = brick_of(p, q);
+            const int set = k & 1;
+            const uint32_t acc = tmem + (uint32_t)set * set_cols;
+            ok = mbar_wait_warp(aempty + 8u * set, (uint32_t)(k >> 1) & 1u, p.tries);  // stored and zeroed
+            for (int z = 0; z < br.planes + 2 && ok; ++z) {
+                ok = mbar_wait_warp(pfull + 8u * slot, (ph >> slot) & 1u, p.tries);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                // group g (tap dz = g - 1) feeds plane z - g, whose accumulator is at (planes - 1 - z + g) cout
+                const int g0 = max(0, z - br.planes + 1), g1 = min(2, z);
+                march_issue<CK, MIRROR>(one, acc + (uint32_t)((br.planes - 1 - z + g0) * p.cout),
+                                (uint32_t)p.a_hi | (((tile0 + (uint32_t)slot * p.plane_bytes) >> 4) & 0x3FFFu),
+                                (uint32_t)(p.a_hi >> 32), blo + (uint32_t)(g0 * p.cout), bhi,
+                                p.idesc | ((uint32_t)(((g1 - g0 + 1) * p.cout) >> 3) << 17), p.cout);
+                commit_elected(one, pempty + 8u * slot);
+                ph ^= 1u << slot;
+                slot = slot + 1 == p.slots ? 0 : slot + 1;
+            }
+            if (!ok) s_fail = 1;
+            commit_elected(one, afull + 8u * set);  // also after a failed wait: the storing warps see s_fail and stop
+        }
+        commit_elected(one, retired);  // completes once every MMA issued above has
+    } else if (warp >= 2) {
+        const int m = (warp & 3) * 32 + lane;  // a warp reads the TMEM lanes of its quarter: x = m % 8, y = m / 8
+        tmem_zero(tmem + ((uint32_t)((warp & 3) * 32) << 16), p.tmem_cols);
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane < 2) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(aempty + 8u * lane) : "memory");
+        int k = 0;
+        for (long long q = blockIdx.x; q < p.items; q += gridDim.x, ++k) {
+            const Brick br = brick_of(p, q);
+            const int set = k & 1;
+            const bool done = mbar_wait(afull + 8u * set, (uint32_t)(k >> 1) & 1u, p.tries);
+            if (__any_sync(0xffffffffu, !done || s_fail)) {
+                s_fail = 1;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int x = br.x0 + m % HB_X, y = br.y0 + m / HB_X;
+            const bool inside = x < p.W && y < p.H;
+            const uint32_t acc = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)set * set_cols;
+            for (int c0 = 0; c0 < p.cout; c0 += 16) {
+                float bias[16];
+#pragma unroll
+                for (int e = 0; e < 16; ++e) bias[e] = p.bias ? __ldg(p.bias + c0 + e) : 0.f;
+                for (int zo = 0; zo < br.planes; ++zo) {
+                    const int z = br.z0 + (MIRROR ? br.planes - 1 - zo : zo);
+                    const long long v = (((long long)br.n * p.D + z) * p.H + y) * p.W + x;
+                    float o[16];
+                    tmem_ld16(acc + (uint32_t)((br.planes - 1 - zo) * p.cout + c0), o);
+                    if (!inside) continue;
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) o[e] += bias[e];
+                    if (p.relu) {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) o[e] = fmaxf(o[e], 0.f);
+                    }
+                    store_cell16(p.y, p.yf, v * p.ldy + p.yoff + c0, p.accumulate, o);
+                }
+            }
+            tmem_zero(acc, br.planes * p.cout);
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(aempty + 8u * set) : "memory");
+        }
     }
     __syncwarp();
     __syncthreads();
-
-    const bool ready = mbar_wait(accum, 0u, p.tries) && !s_fail;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const int m = warp * 32 + lane;           // accumulator row: x = m % 8, y = m / 8
-    const int x = x0 + (m % HB_X), y = y0 + m / HB_X;
-    const bool inxy = ready && x < p.W && y < p.H;
-    for (int c0 = 0; c0 < p.cout; c0 += 16) {
-        float bias[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) bias[q] = p.bias ? __ldg(p.bias + c0 + q) : 0.f;
-        for (int zo = 0; zo < p.dz_planes; ++zo) {
-            const int z = z0 + zo;
-            const bool inside = inxy && z < p.D;
-            const long long v = (((long long)bn * p.D + z) * p.H + y) * p.W + x;
-            float o[16];
-            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)((p.dz_planes + 1 - zo) * p.cout + c0), o);
-            if (!inside) continue;
-#pragma unroll
-            for (int q = 0; q < 16; ++q) o[q] += bias[q];
-            if (p.relu) {
-#pragma unroll
-                for (int q = 0; q < 16; ++q) o[q] = fmaxf(o[q], 0.f);
-            }
-            if (p.yf) {
-                float4* dst = reinterpret_cast<float4*>(p.yf + v * p.ldy + p.yoff + c0);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    float4 w = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
-                    if (p.accumulate) {
-                        const float4 r = dst[q];
-                        w.x += r.x; w.y += r.y; w.z += r.z; w.w += r.w;
-                    }
-                    dst[q] = w;
-                }
-            } else {
-                uint4 pk[2];
-                uint32_t* u = reinterpret_cast<uint32_t*>(pk);
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const __nv_bfloat162 h2 = __floats2bfloat162_rn(o[2 * q], o[2 * q + 1]);
-                    u[q] = *reinterpret_cast<const uint32_t*>(&h2);
-                }
-                uint4* dst = reinterpret_cast<uint4*>(p.y + v * p.ldy + p.yoff + c0);
-                dst[0] = pk[0];
-                dst[1] = pk[1];
-            }
-        }
+    // every MMA has retired (TMEM and the operands are free) and, after a failed wait, every load in flight has landed before
+    // the block's memory is released; both waits are bounded
+    mbar_wait(retired, 0u, p.tries);
+    if (threadIdx.x == 0 && s_fail) {
+        for (int q = 0; q < p.slots; ++q)
+            if ((pending >> q) & 1u) mbar_wait(pfull + 8u * q, ((phase >> q) & 1u) ^ 1u, p.tries);
     }
-    // a tile load still in flight after a failed wait lands before the shared memory is released
-    if (threadIdx.x == 0 && !ready && p.withhold < 0) mbar_wait(full, 0u, p.tries);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 2) {
+    if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem_cols) : "memory");
     }
@@ -752,43 +837,70 @@ unsigned long long umma_layout(int ck) { return ck == 16 ? 6ULL : (ck == 32 ? 4U
 
 unsigned round1024(unsigned v) { return (v + 1023u) & ~1023u; }
 
-// the narrow-layer kernel takes 16 or 32 channels in and out on grids at least one brick across
-bool halo_shape(int cin, int cout, int d, int h, int wd) {
-    return (cin == 16 || cin == 32) && (cout == 16 || cout == 32) && wd >= HB_X && h >= HB_Y && d >= 4;
+// the marching kernel: weights of all taps in up to 108 KB, on grids at least one brick across
+bool march_shape(int cin, int cout, int d, int h, int wd) {
+    return (cin == 16 || cin == 32 || cin == 64) && (cout == 16 || cout == 32 || cout == 64) && cin * cout <= 2048 &&
+           wd >= HB_X && h >= HB_Y && d >= 4;
 }
 
-pf_status conv_halo(const void* x, int ldx, int xoff, const void* w, int cin, int cout, const float* bias, int relu,
-                    int flip, void* y_bf16, float* y_f32, int ldy, int yoff, int accumulate, int n, int d, int h,
-                    int wd, cudaStream_t stream, PFN_cuTensorMapEncodeTiled_v12000 enc) {
-    HaloArgs a{};
+pf_status conv_march(const void* x, int ldx, int xoff, const void* w, int cin, int cout, const float* bias, int relu,
+                     int flip, void* y_bf16, float* y_f32, int ldy, int yoff, int accumulate, int n, int d, int h,
+                     int wd, cudaStream_t stream, PFN_cuTensorMapEncodeTiled_v12000 enc) {
+    MarchArgs a{};
     a.cin = cin;
     a.cout = cout;
     a.D = d;
     a.H = h;
     a.W = wd;
-    a.flip = flip;
     a.relu = relu;
     a.accumulate = accumulate;
-    a.withhold = g_test_withhold;
     a.tries = g_test_tries > 0 ? g_test_tries : WAIT_TRIES;
+    const int withhold = g_test_withhold;
     g_test_withhold = -1;
     g_test_tries = 0;
     a.w_bytes = (unsigned)(27 * cout * cin * 2);
-    // 4 output planes per brick: 16 -> 16 channels then fit four blocks per SM (48.6 KB of shared memory,
-    // 8 x 16 TMEM columns each), the wider layers two (32 x 32: one)
-    const int dzp = 4;
-    auto chunk = [](int dz) { return round1024((unsigned)(HT_ROW * HT_Y * (dz + 2))); };
-    a.dz_planes = dzp;
-    a.chunk_bytes = chunk(dzp);
-    a.tile_bytes = (unsigned)(cin / 8) * a.chunk_bytes;
-    a.tx_bytes = (unsigned)(cin / 8) * (HT_ROW * HT_Y * (dzp + 2));
     a.tx = (wd + HB_X - 1) / HB_X;
     a.ty = (h + HB_Y - 1) / HB_Y;
-    a.tz = (d + dzp - 1) / dzp;
-    // MMA N = 3 cout: the taps dz = -1, 0, +1 of one lateral offset
-    a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(3 * cout >> 3) << 17) | ((unsigned)(UM >> 4) << 24);
-    const int cols = (dzp + 4) * cout;
-    a.tmem_cols = cols <= 32 ? 32 : (cols <= 64 ? 64 : (cols <= 128 ? 128 : 256));
+    const unsigned row = (unsigned)cin * 2;
+    a.plane_tx = (unsigned)(HT_X * HT_Y) * row;
+    a.plane_bytes = round1024(a.plane_tx);
+    // Blocks per SM and planes per brick: the fewest clocks.  Up to four blocks share the 512 TMEM columns (two accumulator
+    // sets each) and the shared memory.  An MMA of m cout columns takes the longer of its multiplications and its reads from
+    // shared memory; a block's issuing warp takes about 38 clocks per MMA and 550 per plane (fitted to 16, 32 and 64 input
+    // channels), so several blocks keep the tensor core busy where a plane has few MMAs.  The ends of a brick (m = 1, 2) cost
+    // nearly as much as its middle.
+    long long best = -1;
+    int occ = 1;
+    for (int o = 1; o <= 4; ++o) {
+        const unsigned room = 216u * 1024u / o - 2048u * (o > 1);
+        const int slots = room > a.w_bytes ? (int)((room - a.w_bytes) / a.plane_bytes) : 0;
+        if (slots < 3) continue;
+        for (int dz = 1; dz <= d && 2 * dz * cout <= (o == 3 ? 128 : 512 / o); ++dz) {
+            const long long tz = (d + dz - 1) / dz, items = (long long)a.tx * a.ty * tz * n;
+            long long clocks = 0;
+            for (int z = 0; z < dz + 2; ++z) {
+                const int m = std::min(2, z) - std::max(0, z - dz + 1) + 1;
+                clocks += std::max(m * cout / 2, 32 + m * cout / 4);
+            }
+            const long long mmas = 9 * (cin / 16), issue = (dz + 2) * (550 + 38 * mmas);
+            const long long cost = ((items + 152 * o - 1) / (152 * o)) * std::max(o * clocks * mmas, issue) + 3000;
+            if (best < 0 || cost < best) {
+                best = cost;
+                occ = o;
+                a.dz = dz;
+                a.tz = (int)tz;
+                a.items = items;
+                a.slots = slots < MR_SLOTS ? slots : MR_SLOTS;
+            }
+        }
+    }
+    if (best < 0) return PF_E_INVALID;
+    a.withhold = withhold < 0 ? -1 : withhold % (a.dz + 2);
+    a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(UM >> 4) << 24);
+    // K-major, swizzled with the span of a row; stride between 8-row groups: one tile row of 10 cells
+    a.a_hi = (1ULL << 16) | (1ULL << 46) | (umma_layout(cin) << 61) | ((unsigned long long)(HT_X * row >> 4) << 32);
+    const int cols = 2 * a.dz * cout;
+    a.tmem_cols = cols <= 32 ? 32 : (cols <= 64 ? 64 : (cols <= 128 ? 128 : (cols <= 256 ? 256 : 512)));
     a.bias = bias;
     a.w = (const bf16*)w;
     a.y = (bf16*)y_bf16;
@@ -797,24 +909,31 @@ pf_status conv_halo(const void* x, int ldx, int xoff, const void* w, int cin, in
     a.yoff = yoff;
     alignas(64) CUtensorMap mX;
     const cuuint64_t dims[5] = {(cuuint64_t)cin, (cuuint64_t)wd, (cuuint64_t)h, (cuuint64_t)d, (cuuint64_t)n};
-    const cuuint64_t row = (cuuint64_t)ldx * 2;
-    const cuuint64_t strides[4] = {row, row * wd, row * wd * h, row * wd * h * d};
-    const cuuint32_t box[5] = {8, (cuuint32_t)HT_X, (cuuint32_t)HT_Y, (cuuint32_t)(dzp + 2), 1};
+    const cuuint64_t xr = (cuuint64_t)ldx * 2;
+    const cuuint64_t strides[4] = {xr, xr * wd, xr * wd * h, xr * wd * h * d};
+    const cuuint32_t box[5] = {(cuuint32_t)cin, (cuuint32_t)HT_X, (cuuint32_t)HT_Y, 1, 1};
     const cuuint32_t es[5] = {1, 1, 1, 1, 1};
     if (enc(&mX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)((const bf16*)x + xoff), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, tma_swizzle(cin), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return PF_E_INVALID;
-    const size_t smem = 1024 + (size_t)a.tile_bytes + a.w_bytes + 32;
+    const size_t smem = 1024 + (size_t)a.slots * a.plane_bytes + a.w_bytes;
+    const bool mirror = flip && (cin == 64 || cout == 64);
+    a.flip = flip && !mirror;
+    auto k = cin == 16 ? (mirror ? k_conv_march<16, true> : k_conv_march<16, false>)
+             : cin == 32 ? (mirror ? k_conv_march<32, true> : k_conv_march<32, false>)
+                         : (mirror ? k_conv_march<64, true> : k_conv_march<64, false>);
     static std::once_flag attr_once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(attr_once, [] {
-        attr_err = cudaFuncSetAttribute(k_conv_halo, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        for (auto f : {k_conv_march<16, false>, k_conv_march<32, false>, k_conv_march<64, false>, k_conv_march<16, true>,
+                       k_conv_march<32, true>, k_conv_march<64, true>}) {
+            const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 218 * 1024);
+            if (e != cudaSuccess) attr_err = e;
+        }
     });
-    if (attr_err != cudaSuccess || smem > 200u * 1024u) return PF_E_CUDA;
-    const long long blocks = (long long)a.tx * a.ty * a.tz * n;
-    if (blocks > 0x7FFFFFFFLL) return PF_E_RANGE;
-    k_conv_halo<<<(unsigned)blocks, UTHR, smem, stream>>>(mX, a);
+    if (attr_err != cudaSuccess || smem > 218u * 1024u) return PF_E_CUDA;
+    k<<<(unsigned)std::min<long long>(a.items, 152LL * occ), MR_THR, smem, stream>>>(mX, a);
     pfgb::count_launch();
     return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
 }
@@ -933,8 +1052,8 @@ pf_status pfnn_conv3d(const void* x, int ldx, int xoff, const void* w, int cin, 
         return PF_E_INVALID;
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
     if (!enc) return PF_E_CUDA;
-    if (halo_shape(cin, cout, d, h, wd))
-        return conv_halo(x, ldx, xoff, w, cin, cout, bias, relu, flip, y_bf16, y_f32, ldy, yoff, accumulate, n, d, h,
+    if (march_shape(cin, cout, d, h, wd))
+        return conv_march(x, ldx, xoff, w, cin, cout, bias, relu, flip, y_bf16, y_f32, ldy, yoff, accumulate, n, d, h,
                          wd, (cudaStream_t)stream, enc);
 
     UmmaArgs a{};
