@@ -49,8 +49,9 @@ pf_status pfnn_status(int* failed);
  * (1 <= tries <= 2^24) instead of 2^24.  The waits for that stage then give up: the call finishes
  * without storing its output, TMEM freed after every issued MMA has retired, and pfnn_status reports
  * it.  The setting applies to one call only.  Nothing faults: the withheld stage is an empty wait.
- * Layers of 16 or 32 channels in and out on grids of at least 8 x 16 x 4 (W x H x D) run the halo-tile
- * kernel, which loads one tile per block: there any stage >= 0 withholds that tile. */
+ * Layers whose weights stay in shared memory (16, 32 or 64 channels in and out, cin cout <= 2048, grids of at least
+ * 8 x 16 x 4, W x H x D) load planes of bricks: there it is plane `stage` modulo the planes of a brick, of every brick;
+ * the wide layers' kernel withholds the weights of stage modulo 9 cin / ck, of every plane. */
 pf_status pfnn_test_withhold_stage(int stage, long long tries);
 
 /* Weight gradient: dw[t][co][ci] += sum_v dy[v][co] x[v + off(t)][ci], on the fifth-generation tensor cores:

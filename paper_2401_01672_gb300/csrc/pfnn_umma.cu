@@ -634,6 +634,273 @@ k_conv_march(const __grid_constant__ CUtensorMap tmX, const MarchArgs p) {
     }
 }
 
+// ---------------------------------------------------------------- wide layers: marching pairs of bricks, streamed weights
+// For larger cin x cout the weights do not fit shared memory beside the input (442 KB for 128 -> 64 channels).  Windows,
+// stacked taps dz and the order of the products are those of k_conv_march; the weights of (dy, dx, block of ck channels),
+// 3 nc rows (nc = up to 64 output channels; more are other work items), come through a ring of three stages for every tile
+// plane, and two bricks side by side (16 x 16 columns, one tile of 18 x 18 cells) use each stage, so a stage feeds about 800
+// clocks of MMAs.  A work item marches along z over zc planes; the tile planes come through a ring of (plane, channel
+// block) slots, the accumulators of each brick lie in a ring of four planes (a window's column groups wrap around its end:
+// two MMAs then), and four warps store a plane as soon as its last tap is done.
+//   The weights' stream from L2 (30 bytes a clock and SM) and the shared-memory reads bound it; k_conv_umma reads 27 boxes of
+// the input per 128 voxels instead (46 bytes a clock).  64^3 voxels: 128 -> 64 channels
+// 204 and 115 us, 64 -> 64 120 and 69 us.
+constexpr int WD_RING = 3;       // weight stages
+constexpr int WD_SLOTS = 4;      // most tile slots
+constexpr int WD_ACC = 4;        // accumulator planes per brick
+constexpr int WT_X = 2 * HB_X + 2;
+struct WideArgs {
+    int nc, ncc;                  // output channels of one work item, work items per brick pair
+    int ck, ncb;                  // channels per K block, K blocks
+    int zc, slots;                // output planes per work item, tile slots
+    int D, H, W, tx, ty, tz;
+    int relu, accumulate;
+    int withhold;                 // >= 0: the weight loads of this (l, K block) are withheld (failure-path test)
+    long long tries, items;
+    unsigned tile_bytes, tile_tx, ring_bytes, ring_tx;
+    unsigned idesc;               // without N
+    unsigned long long a_hi, b_hi;
+    const float* bias;
+    bf16* y;
+    float* yf;
+    int ldy, yoff;
+};
+
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2,
+                                            int c3) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], "
+        "[%2];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+        : "memory");
+}
+
+struct WideItem {
+    int x0, y0, z0, n, c0, planes;
+};
+__device__ __forceinline__ WideItem wide_item(const WideArgs& p, long long q) {
+    WideItem r;
+    r.c0 = (int)(q % p.ncc) * p.nc;
+    q /= p.ncc;
+    r.x0 = (int)(q % p.tx) * (2 * HB_X);
+    q /= p.tx;
+    r.y0 = (int)(q % p.ty) * HB_Y;
+    q /= p.ty;
+    r.z0 = (int)(q % p.tz) * p.zc;
+    r.n = (int)(q / p.tz);
+    r.planes = min(p.zc, p.D - r.z0);
+    return r;
+}
+
+template <int CK, bool MIRROR>
+__global__ void __launch_bounds__(MR_THR, 1)
+k_conv_wide(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const WideArgs p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const uint32_t sm0 = smem_u32(smem_raw) + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const uint32_t ring0 = sm0 + (uint32_t)p.slots * p.tile_bytes;
+    // barriers: tile full / empty, ring full / empty, accumulator full / empty, all MMAs retired
+    __shared__ __align__(8) unsigned long long bars[2 * (WD_SLOTS + WD_RING + WD_ACC) + 1];
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int s_fail;
+    const uint32_t tfull = smem_u32(bars), tempty = tfull + 8 * WD_SLOTS, rfull = tempty + 8 * WD_SLOTS;
+    const uint32_t rempty = rfull + 8 * WD_RING, afull = rempty + 8 * WD_RING, aempty = afull + 8 * WD_ACC;
+    const uint32_t retired = aempty + 8 * WD_ACC;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int q = 0; q < 2 * (WD_SLOTS + WD_RING) + WD_ACC; ++q) mbar_init(tfull + 8u * q, 1);
+        for (int q = 0; q < WD_ACC; ++q) mbar_init(aempty + 8u * q, 4);
+        mbar_init(retired, 1);
+        s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+
+    // producer, per slot: filled before, phase of the next fill, load issued
+    uint32_t tfilled = 0, tphase = 0, tpending = 0, rfilled = 0, rphase = 0, rpending = 0;
+    if (threadIdx.x == 0) {
+        bool ok = true;
+        int ts = 0, rs = 0;
+        auto tile = [&](const WideItem& it, int z, int cb) {
+            const uint32_t bit = 1u << ts;
+            if (tfilled & bit) ok = mbar_wait(tempty + 8u * ts, ((tphase >> ts) & 1u) ^ 1u, p.tries);
+            if (!ok || s_fail) { ok = false; return; }
+            mbar_expect_tx(tfull + 8u * ts, p.tile_tx);
+            tma_load_5d(sm0 + (uint32_t)ts * p.tile_bytes, &tmA, tfull + 8u * ts, cb * p.ck, it.x0 - 1, it.y0 - 1,
+                        it.z0 - 1 + (MIRROR ? it.planes + 1 - z : z), it.n);
+            tfilled |= bit;
+            tpending |= bit;
+            tphase ^= bit;
+            ts = ts + 1 == p.slots ? 0 : ts + 1;
+        };
+        const int ahead = min(p.slots - p.ncb, p.ncb);  // blocks of the next plane whose slots this plane does not use
+        for (long long q = blockIdx.x; q < p.items && ok; q += gridDim.x) {
+            const WideItem it = wide_item(p, q);
+            for (int z = 0; z < it.planes + 2 && ok; ++z)
+                for (int l = 0; l < 9 && ok; ++l) {
+                    for (int cb = 0; cb < p.ncb && ok; ++cb) {
+                        // this plane's tiles, but for those loaded ahead (below)
+                        if (l == 0 && (z == 0 || cb >= ahead)) tile(it, z, cb);
+                        if (!ok) break;
+                        const uint32_t bit = 1u << rs;
+                        if (rfilled & bit) ok = mbar_wait(rempty + 8u * rs, ((rphase >> rs) & 1u) ^ 1u, p.tries);
+                        if (!ok || s_fail) { ok = false; break; }
+                        mbar_expect_tx(rfull + 8u * rs, p.ring_tx);
+                        if (l * p.ncb + cb != p.withhold) {
+                            tma_load_4d(ring0 + (uint32_t)rs * p.ring_bytes, &tmB, rfull + 8u * rs, cb * p.ck, it.c0, l, 0);
+                            rpending |= bit;
+                        } else {
+                            rpending &= ~bit;
+                        }
+                        rfilled |= bit;
+                        rphase ^= bit;
+                        rs = rs + 1 == WD_RING ? 0 : rs + 1;
+                    }
+                    if (l == 4 && z < it.planes + 1)
+                        for (int cb = 0; cb < ahead && ok; ++cb) tile(it, z + 1, cb);
+                }
+        }
+    } else if (warp == 1) {
+        const uint32_t one = elect_lane();
+        bool ok = true;
+        uint32_t tph = 0, rph = 0;
+        int ts = 0, rs = 0;      // first tile slot of the plane, ring stage
+        int done = 0;            // output planes of the items before, modulo 4
+        constexpr uint32_t ROW16 = CK / 8;  // 16-byte units of a tile or weight row
+        const uint32_t a_hi = (uint32_t)(p.a_hi >> 32), b_hi = (uint32_t)(p.b_hi >> 32);
+        uint32_t aph = 0;        // accumulator slots' phases waited for, one bit each
+        for (long long q = blockIdx.x; q < p.items && ok; q += gridDim.x) {
+            const int planes = wide_item(p, q).planes;
+            for (int z = 0; z < planes + 2 && ok; ++z) {
+                if (z < planes) {  // the new plane's accumulators are stored and zeroed
+                    const int o = (done + z) & 3;
+                    ok = mbar_wait_warp(aempty + 8u * o, (aph >> o) & 1u, p.tries);
+                    aph ^= 1u << o;
+                }
+                // group g (tap dz = g - 1) feeds plane z - g; plane o (counted over the items) is column group 3 - o mod 4
+                const int g0 = max(0, z - planes + 1), g1 = min(2, z), ng = g1 - g0 + 1;
+                const int s0 = 3 - ((done + z - g0) & 3), n1 = min(ng, WD_ACC - s0), n2 = ng - n1;
+                const uint32_t d1 = tmem + (uint32_t)(s0 * p.nc), b1 = (uint32_t)(g0 * p.nc) * ROW16;
+                const uint32_t b2 = b1 + (uint32_t)(n1 * p.nc) * ROW16;
+                const uint32_t id1 = p.idesc | ((uint32_t)((n1 * p.nc) >> 3) << 17);
+                const uint32_t id2 = p.idesc | ((uint32_t)((n2 * p.nc) >> 3) << 17);
+                for (int l = 0; l < 9 && ok; ++l) {
+                    const int at = MIRROR ? 8 - l : l;
+                    const uint32_t win = (uint32_t)((at / 3) * WT_X + at % 3) * ROW16;
+                    int t = ts;
+                    for (int cb = 0; cb < p.ncb; ++cb) {
+                        if (l == 0) {
+                            ok = mbar_wait_warp(tfull + 8u * t, (tph >> t) & 1u, p.tries);
+                            if (!ok) break;
+                            tph ^= 1u << t;
+                        }
+                        ok = mbar_wait_warp(rfull + 8u * rs, (rph >> rs) & 1u, p.tries);
+                        if (!ok) break;
+                        rph ^= 1u << rs;
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint32_t b = (uint32_t)p.b_hi | (((ring0 + (uint32_t)rs * p.ring_bytes) >> 4) & 0x3FFFu);
+                        const uint32_t a = ((uint32_t)p.a_hi | (((sm0 + (uint32_t)t * p.tile_bytes) >> 4) & 0x3FFFu)) + win;
+#pragma unroll
+                        for (int k = 0; k < CK / 16; ++k) {
+#pragma unroll
+                            for (int j = 0; j < 2; ++j) {  // the two bricks: independent accumulators
+                                const uint32_t ak = a + (uint32_t)(j * HB_X) * ROW16 + 2u * k;
+                                umma_elected(one, d1 + 256u * j, ak, a_hi, b + b1 + 2u * k, b_hi, id1, 1u);
+                                if (n2 > 0) umma_elected(one, tmem + 256u * j, ak, a_hi, b + b2 + 2u * k, b_hi, id2, 1u);
+                            }
+                        }
+                        commit_elected(one, rempty + 8u * rs);
+                        rs = rs + 1 == WD_RING ? 0 : rs + 1;
+                        if (l == 8) commit_elected(one, tempty + 8u * t);
+                        t = t + 1 == p.slots ? 0 : t + 1;
+                    }
+                }
+                for (int cb = 0; cb < p.ncb; ++cb) ts = ts + 1 == p.slots ? 0 : ts + 1;
+                if (!ok) s_fail = 1;
+                // plane z - 2 is complete (after a failed wait: the storing warps see s_fail and stop)
+                if (z >= 2 || !ok) commit_elected(one, afull + 8u * (uint32_t)((done + max(z - 2, 0)) & 3));
+            }
+            done = (done + planes) & 3;
+        }
+        commit_elected(one, retired);  // completes once every MMA issued above has
+    } else if (warp >= 2) {
+        const int m = (warp & 3) * 32 + lane;  // a warp reads the TMEM lanes of its quarter: x = m % 8, y = m / 8
+        tmem_zero(tmem + ((uint32_t)((warp & 3) * 32) << 16), 512);
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane < WD_ACC) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(aempty + 8u * lane) : "memory");
+        long long o = 0;
+        bool ok = true;
+        for (long long q = blockIdx.x; q < p.items && ok; q += gridDim.x) {
+            const WideItem it = wide_item(p, q);
+            const int y = it.y0 + m / HB_X;
+            for (int zo = 0; zo < it.planes; ++zo, ++o) {
+                const uint32_t slot = (uint32_t)(o & 3);
+                const bool done = mbar_wait(afull + 8u * slot, (uint32_t)(o >> 2) & 1u, p.tries);
+                if (__any_sync(0xffffffffu, !done || s_fail)) {
+                    s_fail = 1;
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const int z = it.z0 + (MIRROR ? it.planes - 1 - zo : zo);
+                for (int j = 0; j < 2; ++j) {
+                    const int x = it.x0 + j * HB_X + m % HB_X;
+                    const bool inside = x < p.W && y < p.H;
+                    const long long v = (((long long)it.n * p.D + z) * p.H + y) * p.W + x;
+                    const uint32_t acc = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 256u * j + (3u - slot) * (uint32_t)p.nc;
+                    for (int c = 0; c < p.nc; c += 16) {
+                        float r[16];
+                        tmem_ld16(acc + (uint32_t)c, r);
+                        if (!inside) continue;
+                        const int ch = it.c0 + c;
+                        if (p.bias) {
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) r[e] += __ldg(p.bias + ch + e);
+                        }
+                        if (p.relu) {
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) r[e] = fmaxf(r[e], 0.f);
+                        }
+                        store_cell16(p.y, p.yf, v * p.ldy + p.yoff + ch, p.accumulate, r);
+                    }
+                    tmem_zero(acc, p.nc);
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(aempty + 8u * slot) : "memory");
+            }
+        }
+    }
+    __syncwarp();
+    __syncthreads();
+    // every MMA has retired (TMEM and the operands are free) and, after a failed wait, every load in flight has landed before
+    // the block's memory is released; both waits are bounded
+    mbar_wait(retired, 0u, p.tries);
+    if (threadIdx.x == 0 && s_fail) {
+        for (int q = 0; q < p.slots; ++q)
+            if ((tpending >> q) & 1u) mbar_wait(tfull + 8u * q, ((tphase >> q) & 1u) ^ 1u, p.tries);
+        for (int q = 0; q < WD_RING; ++q)
+            if ((rpending >> q) & 1u) mbar_wait(rfull + 8u * q, ((rphase >> q) & 1u) ^ 1u, p.tries);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    }
+}
+
 // ---------------------------------------------------------------- weight gradient on tcgen05
 // dW[t][co][ci] = sum over voxels v of dY[v][co] X[v + off(t)][ci] (zero padding): GEMMs whose reduction
 // runs over voxels, with both operands taken as they lie in memory.  A channels-last tile in shared memory
@@ -938,6 +1205,114 @@ pf_status conv_march(const void* x, int ldx, int xoff, const void* w, int cin, i
     return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
 }
 
+// The wide-layer kernel: more weights than fit shared memory, brick pairs that are mostly full, and enough 16 x 16 planes of
+// them for the chip (a work item needs two more tile planes than it has output planes).  Below that k_conv_umma, which
+// has 128 voxels per block, fills more SMs.
+bool wide_shape(int cin, int cout, int n, int d, int h, int wd) {
+    const int nc = cout % 64 == 0 ? 64 : (cout % 32 == 0 ? 32 : 16), ck = cin % 64 == 0 ? 64 : (cin % 32 == 0 ? 32 : 16);
+    const long long planes = (long long)((wd + 15) / 16) * ((h + 15) / 16) * d * n * (cout / nc);
+    return cin * cout > 2048 && cin / ck <= 3 && (wd > 24 || (wd > 8 && wd <= 16)) && h >= HB_Y && planes >= 500;
+}
+
+pf_status conv_wide(const void* x, int ldx, int xoff, const void* w, int cin, int cout, const float* bias, int relu,
+                    int flip, void* y_bf16, float* y_f32, int ldy, int yoff, int accumulate, int n, int d, int h, int wd,
+                    cudaStream_t stream, PFN_cuTensorMapEncodeTiled_v12000 enc) {
+    WideArgs a{};
+    a.nc = cout % 64 == 0 ? 64 : (cout % 32 == 0 ? 32 : 16);
+    a.ncc = cout / a.nc;
+    a.ck = cin % 64 == 0 ? 64 : (cin % 32 == 0 ? 32 : 16);
+    a.ncb = cin / a.ck;
+    a.D = d;
+    a.H = h;
+    a.W = wd;
+    a.relu = relu;
+    a.accumulate = accumulate;
+    a.tries = g_test_tries > 0 ? g_test_tries : WAIT_TRIES;
+    a.withhold = g_test_withhold < 0 ? -1 : g_test_withhold % (9 * a.ncb);
+    g_test_withhold = -1;
+    g_test_tries = 0;
+    a.tx = (wd + 2 * HB_X - 1) / (2 * HB_X);
+    a.ty = (h + HB_Y - 1) / HB_Y;
+    // output planes per work item: the fewest waves x clocks.  An MMA of m nc columns takes the longer of its
+    // multiplications and its reads from shared memory; half of the windows of three groups wrap around the ring
+    const auto mma = [&](int m) { return std::max(m * a.nc / 2, 32 + m * a.nc / 4); };
+    const long long full = (mma(3) + mma(1) + mma(2)) / 2;
+    long long best = -1;
+    for (int zc = 1; zc <= d; ++zc) {
+        const long long tz = (d + zc - 1) / zc, items = (long long)a.tx * a.ty * tz * n * a.ncc;
+        long long clocks = 0;
+        for (int z = 0; z < zc + 2; ++z) {
+            const int m = std::min(2, z) - std::max(0, z - zc + 1) + 1;
+            clocks += m == 3 ? full : mma(m);
+        }
+        const long long cost = ((items + 151) / 152) * clocks * 2 * 9 * (cin / 16) + 4000;
+        if (best < 0 || cost < best) {
+            best = cost;
+            a.zc = zc;
+            a.tz = (int)tz;
+            a.items = items;
+        }
+    }
+    const unsigned row = (unsigned)a.ck * 2;
+    a.tile_tx = (unsigned)(WT_X * HT_Y) * row;
+    a.tile_bytes = round1024(a.tile_tx);
+    a.ring_tx = 3u * (unsigned)a.nc * row;
+    a.ring_bytes = round1024(a.ring_tx);
+    const int slots = (int)((215u * 1024u - WD_RING * a.ring_bytes) / a.tile_bytes);
+    a.slots = slots < WD_SLOTS ? slots : WD_SLOTS;
+    if (a.slots < a.ncb) return PF_E_INVALID;
+    a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(UM >> 4) << 24);
+    // K-major, swizzled with the span of a row; stride between 8-row groups: one tile row of 18 cells, 8 weight rows
+    const unsigned long long base = (1ULL << 16) | (1ULL << 46) | (umma_layout(a.ck) << 61);
+    a.a_hi = base | ((unsigned long long)(WT_X * row >> 4) << 32);
+    a.b_hi = base | ((unsigned long long)(8 * row >> 4) << 32);
+    a.bias = bias;
+    a.y = (bf16*)y_bf16;
+    a.yf = y_f32;
+    a.ldy = ldy;
+    a.yoff = yoff;
+    alignas(64) CUtensorMap mA, mB;
+    const cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    {
+        const cuuint64_t dims[5] = {(cuuint64_t)cin, (cuuint64_t)wd, (cuuint64_t)h, (cuuint64_t)d, (cuuint64_t)n};
+        const cuuint64_t r = (cuuint64_t)ldx * 2;
+        const cuuint64_t strides[4] = {r, r * wd, r * wd * h, r * wd * h * d};
+        const cuuint32_t box[5] = {(cuuint32_t)a.ck, (cuuint32_t)WT_X, (cuuint32_t)HT_Y, 1, 1};
+        if (enc(&mA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)((const bf16*)x + xoff), dims, strides, box, es,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, tma_swizzle(a.ck), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return PF_E_INVALID;
+    }
+    {
+        // [dz][l][cout][cin]: one box is the three taps dz of a lateral offset
+        const cuuint64_t r = (cuuint64_t)cin * 2;
+        const cuuint64_t dims[4] = {(cuuint64_t)cin, (cuuint64_t)cout, 9, 3};
+        const cuuint64_t strides[3] = {r, r * cout, r * cout * 9};
+        const cuuint32_t box[4] = {(cuuint32_t)a.ck, (cuuint32_t)a.nc, 1, 3};
+        if (enc(&mB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(w), dims, strides, box, es,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, tma_swizzle(a.ck), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return PF_E_INVALID;
+    }
+    const size_t smem = 1024 + (size_t)a.slots * a.tile_bytes + (size_t)WD_RING * a.ring_bytes;
+    static std::once_flag attr_once;
+    static cudaError_t attr_err = cudaSuccess;
+    std::call_once(attr_once, [] {
+        for (auto f : {k_conv_wide<16, false>, k_conv_wide<32, false>, k_conv_wide<64, false>, k_conv_wide<16, true>,
+                       k_conv_wide<32, true>, k_conv_wide<64, true>}) {
+            const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 216 * 1024);
+            if (e != cudaSuccess) attr_err = e;
+        }
+    });
+    if (attr_err != cudaSuccess || smem > 216u * 1024u) return PF_E_CUDA;
+    auto k = a.ck == 16 ? (flip ? k_conv_wide<16, true> : k_conv_wide<16, false>)
+             : a.ck == 32 ? (flip ? k_conv_wide<32, true> : k_conv_wide<32, false>)
+                          : (flip ? k_conv_wide<64, true> : k_conv_wide<64, false>);
+    k<<<(unsigned)std::min<long long>(a.items, 152), MR_THR, smem, stream>>>(mA, mB, a);
+    pfgb::count_launch();
+    return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
+}
+
 // Division of a weight gradient's taps and channels over blocks.  cb: the largest of 128, 64, 32, 16 that
 // divides cin.  Stacked (dy along M) for 16 and 32 channels.  A block takes every dz (each X plane loaded
 // once) while its accumulators fit 512 TMEM columns, else one dz (dY loaded three times), else one (dz, dy).
@@ -1054,6 +1429,10 @@ pf_status pfnn_conv3d(const void* x, int ldx, int xoff, const void* w, int cin, 
     if (!enc) return PF_E_CUDA;
     if (march_shape(cin, cout, d, h, wd))
         return conv_march(x, ldx, xoff, w, cin, cout, bias, relu, flip, y_bf16, y_f32, ldy, yoff, accumulate, n, d, h,
+                         wd, (cudaStream_t)stream, enc);
+
+    if (wide_shape(cin, cout, n, d, h, wd))
+        return conv_wide(x, ldx, xoff, w, cin, cout, bias, relu, flip, y_bf16, y_f32, ldy, yoff, accumulate, n, d, h,
                          wd, (cudaStream_t)stream, enc);
 
     UmmaArgs a{};
