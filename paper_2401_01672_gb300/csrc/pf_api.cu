@@ -1362,6 +1362,8 @@ struct pf_batch {
     int model = 0, rx = 0, prec = 0, by = 8;
     cudaStream_t stream = nullptr, cap = nullptr;
     void* d_args = nullptr;
+    std::vector<StageArgs<float>> args32;   // what d_args holds (one of the two)
+    std::vector<StageArgs<double>> args64;
     Ctrl** d_ctrls = nullptr;
     int4* d_tiles = nullptr;
     BatchPlan* d_plan = nullptr;
@@ -1399,13 +1401,13 @@ static pf_status batch_upload(pf_batch* b) {
     }
     PF_BCUDA(b, cudaMemcpy(b->d_tiles, tiles.data(), sizeof(int4) * b->n, cudaMemcpyHostToDevice));
     if (b->prec == PF_PREC_FP32_FIELDS) {
-        std::vector<StageArgs<float>> a(b->n);
-        for (int q = 0; q < b->n; ++q) a[q] = make_args<float>(b->g[q]);
-        PF_BCUDA(b, cudaMemcpy(b->d_args, a.data(), sizeof(StageArgs<float>) * b->n, cudaMemcpyHostToDevice));
+        b->args32.resize(b->n);
+        for (int q = 0; q < b->n; ++q) b->args32[q] = make_args<float>(b->g[q]);
+        PF_BCUDA(b, cudaMemcpy(b->d_args, b->args32.data(), sizeof(StageArgs<float>) * b->n, cudaMemcpyHostToDevice));
     } else {
-        std::vector<StageArgs<double>> a(b->n);
-        for (int q = 0; q < b->n; ++q) a[q] = make_args<double>(b->g[q]);
-        PF_BCUDA(b, cudaMemcpy(b->d_args, a.data(), sizeof(StageArgs<double>) * b->n, cudaMemcpyHostToDevice));
+        b->args64.resize(b->n);
+        for (int q = 0; q < b->n; ++q) b->args64[q] = make_args<double>(b->g[q]);
+        PF_BCUDA(b, cudaMemcpy(b->d_args, b->args64.data(), sizeof(StageArgs<double>) * b->n, cudaMemcpyHostToDevice));
     }
     return PF_OK;
 }
@@ -1414,11 +1416,11 @@ static cudaError_t batch_enqueue_step(pf_batch* b, cudaStream_t s, int sms, cuda
     cudaError_t e = cudaSuccess;
     for (int st = 1; st <= 5 && e == cudaSuccess; ++st) {
         if (b->prec == PF_PREC_FP32_FIELDS)
-            e = launch_batch_stage_f32(b->model, b->rx, st, (const StageArgs<float>*)b->d_args, b->d_plan, b->d_tiles,
-                                       b->by, sms, s);
+            e = launch_batch_stage_f32(b->model, b->rx, st, {b->args32.data(), (const StageArgs<float>*)b->d_args, b->n},
+                                       b->d_plan, b->d_tiles, b->by, sms, s);
         else
-            e = launch_batch_stage_f64(b->model, b->rx, st, (const StageArgs<double>*)b->d_args, b->d_plan, b->d_tiles,
-                                       b->by, sms, s);
+            e = launch_batch_stage_f64(b->model, b->rx, st, {b->args64.data(), (const StageArgs<double>*)b->d_args, b->n},
+                                       b->d_plan, b->d_tiles, b->by, sms, s);
     }
     if (e != cudaSuccess) return e;
     k_batch_controller<<<(b->n + BC_WARPS - 1) / BC_WARPS, 32 * BC_WARPS, 0, s>>>(b->d_ctrls, b->d_plan);

@@ -171,6 +171,21 @@ struct StageArgs {
     int tw, th;              // lateral tile (tile_shape)
 };
 
+// A batch's stage arguments: a host and a device copy; batches of up to BATCH_PARAMS instances pass them as kernel
+// parameters (at most 32764 bytes).
+constexpr int BATCH_PARAMS = 60;
+template <typename T>
+struct BatchParams {
+    StageArgs<T> a[BATCH_PARAMS];
+};
+static_assert(sizeof(BatchParams<double>) + 16 <= 32764, "kernel parameters");
+template <typename T>
+struct BatchArgs {
+    const StageArgs<T>* host;
+    const StageArgs<T>* device;
+    int n;
+};
+
 // Launch one stage (0 = plain RHS, 1..5 = Merson stages) of the given model.
 // Returns the CUDA error of the launch.
 cudaError_t launch_stage_f64(int model, int rx, int stage, const StageArgs<double>& a, int by,
@@ -178,10 +193,10 @@ cudaError_t launch_stage_f64(int model, int rx, int stage, const StageArgs<doubl
 cudaError_t launch_stage_f32(int model, int rx, int stage, const StageArgs<float>& a, int by,
                              cudaStream_t s);
 
-cudaError_t launch_batch_stage_f64(int model, int rx, int stage, const StageArgs<double>* args,
+cudaError_t launch_batch_stage_f64(int model, int rx, int stage, const BatchArgs<double>& args,
                                    BatchPlan* plan, const int4* tilegrid, int by, int sms,
                                    cudaStream_t s);
-cudaError_t launch_batch_stage_f32(int model, int rx, int stage, const StageArgs<float>* args,
+cudaError_t launch_batch_stage_f32(int model, int rx, int stage, const BatchArgs<float>& args,
                                    BatchPlan* plan, const int4* tilegrid, int by, int sms,
                                    cudaStream_t s);
 

@@ -967,8 +967,10 @@ stage_kernel_r128(const StageArgs<T> a) {
 // that are finished are not listed), the first one each by number, then the next from a counter that k_batch_plan zeroes;
 // a block asks for its next tile before it starts one, so the answer is there when it needs it.  (With a stride of the
 // grid, and a third more blocks than fit, one 128^3 instance in binary64 took 9.1 ms for 24 attempts; see batch_one.)
-template <int MODEL, int RX, typename T, typename TIN, int STAGE, int BY>
-__device__ __forceinline__ void batch_tiles(const StageArgs<T>* __restrict__ args, BatchPlan* __restrict__ plan,
+// `args`: the instances' stage arguments, in the kernel's parameters (constant bank, as for a single grid) where they
+// fit, else in global memory, where every use of a pointer or coefficient is a load or a register (12 binary32 instances, 16 attempts: 24.0 and 20.4 ms).
+template <int MODEL, int RX, typename T, typename TIN, int STAGE, int BY, typename ARGS>
+__device__ __forceinline__ void batch_tiles(const ARGS& args, BatchPlan* __restrict__ plan,
                                             const int4* __restrict__ tilegrid) {
     __shared__ int s_next;
     const int nt = plan->ntiles;
@@ -985,6 +987,20 @@ __device__ __forceinline__ void batch_tiles(const StageArgs<T>* __restrict__ arg
         t = s_next;
         __syncthreads();
     }
+}
+
+template <int MODEL, int RX, typename T, typename TIN, int STAGE, int BY>
+__global__ void __launch_bounds__(TX * BY)
+batch_param_kernel(const __grid_constant__ BatchParams<T> args, BatchPlan* __restrict__ plan,
+                   const int4* __restrict__ tilegrid) {
+    batch_tiles<MODEL, RX, T, TIN, STAGE, BY>(args.a, plan, tilegrid);
+}
+
+template <int MODEL, int RX, typename T, typename TIN, int STAGE, int BY>
+__global__ void __launch_bounds__(TX * BY, f64_min_blocks(BY))
+batch_param_kernel_r128(const __grid_constant__ BatchParams<T> args, BatchPlan* __restrict__ plan,
+                        const int4* __restrict__ tilegrid) {
+    batch_tiles<MODEL, RX, T, TIN, STAGE, BY>(args.a, plan, tilegrid);
 }
 
 template <int MODEL, int RX, typename T, typename TIN, int STAGE, int BY>
@@ -1031,20 +1047,38 @@ cudaError_t launch_by(int stage, const StageArgs<T>& a, cudaStream_t s) {
 }
 
 // one block for every place on the chip (occupancy of this kernel); `sms` multiprocessors
+template <typename ARGS>
+void batch_launch(void (*k)(ARGS, BatchPlan*, const int4*), const ARGS& args, int threads_y, BatchPlan* plan, const int4* tg,
+                  int sms, cudaStream_t s) {
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, TX * threads_y, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
+    k<<<sms * per_sm, dim3(TX, threads_y), 0, s>>>(args, plan, tg);
+}
 template <typename T, int MODEL, int RX, int STAGE, int BY>
-void batch_one(const StageArgs<T>* args, BatchPlan* plan, const int4* tg, int sms, cudaStream_t s) {
+void batch_one(const BatchArgs<T>& args, BatchPlan* plan, const int4* tg, int sms, cudaStream_t s) {
     using TIN = typename std::conditional<STAGE == 1 && !(std::is_same<T, float>::value && MODEL == M_FULL), double,
                                           T>::type;
-    void (*k)(const StageArgs<T>*, BatchPlan*, const int4*);
-    if constexpr (std::is_same<T, double>::value) k = batch_stage_kernel_r128<MODEL, RX, T, TIN, STAGE, BY>;
-    else k = batch_stage_kernel<MODEL, RX, T, TIN, STAGE, BY>;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, TX * BY, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
-    k<<<sms * per_sm, dim3(TX, BY), 0, s>>>(args, plan, tg);
+    constexpr bool BOUND = std::is_same<T, double>::value;
+    if (args.n <= BATCH_PARAMS) {
+        BatchParams<T> p;
+        for (int q = 0; q < args.n; ++q) p.a[q] = args.host[q];
+        for (int q = args.n; q < BATCH_PARAMS; ++q) p.a[q] = args.host[0];
+        using P = BatchParams<T>;
+        if constexpr (BOUND)
+            batch_launch<P>(batch_param_kernel_r128<MODEL, RX, T, TIN, STAGE, BY>, p, BY, plan, tg, sms, s);
+        else
+            batch_launch<P>(batch_param_kernel<MODEL, RX, T, TIN, STAGE, BY>, p, BY, plan, tg, sms, s);
+    } else {
+        using P = const StageArgs<T>*;
+        if constexpr (BOUND)
+            batch_launch<P>(batch_stage_kernel_r128<MODEL, RX, T, TIN, STAGE, BY>, args.device, BY, plan, tg, sms, s);
+        else
+            batch_launch<P>(batch_stage_kernel<MODEL, RX, T, TIN, STAGE, BY>, args.device, BY, plan, tg, sms, s);
+    }
 }
 
 template <typename T, int MODEL, int RX, int BY>
-cudaError_t batch_by(int stage, const StageArgs<T>* args, BatchPlan* plan, const int4* tg, int sms,
+cudaError_t batch_by(int stage, const BatchArgs<T>& args, BatchPlan* plan, const int4* tg, int sms,
                      cudaStream_t s) {
     switch (stage) {
         case 1: batch_one<T, MODEL, RX, 1, BY>(args, plan, tg, sms, s); break;
@@ -1083,7 +1117,7 @@ cudaError_t launch_stage_t(int model, int rx, int stage, const StageArgs<T>& a, 
 }
 
 template <typename T>
-cudaError_t launch_batch_stage_t(int model, int rx, int stage, const StageArgs<T>* args, BatchPlan* plan,
+cudaError_t launch_batch_stage_t(int model, int rx, int stage, const BatchArgs<T>& args, BatchPlan* plan,
                                  const int4* tg, int by, int sms, cudaStream_t s) {
     auto m = [&](auto M, auto R) -> cudaError_t {
         constexpr int MO = decltype(M)::value, RO = decltype(R)::value;

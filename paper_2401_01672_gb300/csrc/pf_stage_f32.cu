@@ -8,7 +8,7 @@ cudaError_t launch_stage_f32(int model, int rx, int stage, const StageArgs<float
     return launch_stage_t<float>(model, rx, stage, a, by, s);
 }
 
-cudaError_t launch_batch_stage_f32(int model, int rx, int stage, const StageArgs<float>* args, BatchPlan* plan,
+cudaError_t launch_batch_stage_f32(int model, int rx, int stage, const BatchArgs<float>& args, BatchPlan* plan,
                                    const int4* tg, int by, int sms, cudaStream_t s) {
     return launch_batch_stage_t<float>(model, rx, stage, args, plan, tg, by, sms, s);
 }

@@ -8,7 +8,7 @@ cudaError_t launch_stage_f64(int model, int rx, int stage, const StageArgs<doubl
     return launch_stage_t<double>(model, rx, stage, a, by, s);
 }
 
-cudaError_t launch_batch_stage_f64(int model, int rx, int stage, const StageArgs<double>* args, BatchPlan* plan,
+cudaError_t launch_batch_stage_f64(int model, int rx, int stage, const BatchArgs<double>& args, BatchPlan* plan,
                                    const int4* tg, int by, int sms, cudaStream_t s) {
     return launch_batch_stage_t<double>(model, rx, stage, args, plan, tg, by, sms, s);
 }
