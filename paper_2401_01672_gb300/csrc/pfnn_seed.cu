@@ -100,7 +100,8 @@ __global__ void k_sf_apply(const float* __restrict__ prob, const double* __restr
 // ---- Bit form: one bit per cell, 32 cells of a row to a word, so a mask of 256^3 cells is 2 MB and stays in L2.
 // The byte form above swept 16.8 MB of flags from global memory once per cell of path length (10.1 ms for a 256^3 packing);
 // here a block brings a tile of words to its own fixed point in shared memory before the next sweep, a word is filled
-// along x by one carry, and the water indicator is kept as a mask, so G is read once: 0.68 ms.
+// along x by one carry, and the water indicator is kept as a mask, so G is read once: 0.51 ms (0.68 with tiles of 16
+// planes, two barriers around every pass and a visit to every tile in every sweep).
 struct BitGrid {
     int n1, n2, n3, W;  // W words per row
     unsigned tail;      // cells of a row's last word
@@ -108,28 +109,26 @@ struct BitGrid {
 
 __device__ __forceinline__ unsigned valid_bits(const BitGrid& g, int wx) { return wx == g.W - 1 ? g.tail : 0xffffffffu; }
 
-// Masks of predicted ice, reached (seed) and water; a warp builds WPI words at a time, so that 3 WPI loads per lane
-// are in flight (the pass is bound by HBM: 20 bytes a cell).
+// Masks of predicted ice, reached (seed) and water; a warp takes a row, WPI words at a time, so that 3 WPI loads per lane
+// are in flight and no cell index is divided (20 bytes a cell; 102 us at 256^3, 3.3 TB/s).
 constexpr int WPI = 4;
 __global__ void __launch_bounds__(SF_THREADS) k_sb_init(const float* __restrict__ prob, const double* __restrict__ seed,
                                                         const double* __restrict__ G, double zeta, const BitGrid g,
                                                         unsigned* __restrict__ ice, unsigned* __restrict__ reached,
                                                         unsigned* __restrict__ water) {
     const int lane = threadIdx.x & 31;
-    const long long words = (long long)g.W * g.n2 * g.n3;
-    const long long warps = (long long)gridDim.x * (SF_THREADS / 32);
-    for (long long w0 = ((long long)blockIdx.x * (SF_THREADS / 32) + (threadIdx.x >> 5)) * WPI; w0 < words;
-         w0 += warps * WPI) {
+    const int rows = g.n2 * g.n3, step = gridDim.x * (SF_THREADS / 32);
+    for (int row = blockIdx.x * (SF_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += step)
+    for (int wx = 0; wx < g.W; wx += WPI) {
+        const long long w0 = (long long)row * g.W + wx;
         float p[WPI];
         double s[WPI], gl[WPI];
         bool in[WPI];
 #pragma unroll
         for (int r = 0; r < WPI; ++r) {
-            const long long w = w0 + r;
-            const long long row = w / g.W;
-            const int x = (int)(w - row * g.W) * 32 + lane;
-            in[r] = w < words && x < g.n1;
-            const long long q = row * g.n1 + x;
+            const int x = (wx + r) * 32 + lane;
+            in[r] = x < g.n1;
+            const long long q = (long long)row * g.n1 + x;
             p[r] = in[r] ? prob[q] : 0.f;
             s[r] = in[r] ? seed[q] : 0.0;
             gl[r] = in[r] ? G[q] : 0.0;
@@ -140,7 +139,7 @@ __global__ void __launch_bounds__(SF_THREADS) k_sb_init(const float* __restrict_
             const unsigned bw = __ballot_sync(0xffffffffu, wat);
             const unsigned bi = __ballot_sync(0xffffffffu, wat && p[r] > 0.5f);
             const unsigned br = __ballot_sync(0xffffffffu, in[r] && s[r] > 0.5);
-            if (lane == 0 && w0 + r < words) {
+            if (lane == 0 && wx + r < g.W) {
                 ice[w0 + r] = bi;
                 reached[w0 + r] = br;
                 water[w0 + r] = bw;
@@ -190,69 +189,102 @@ __device__ __forceinline__ unsigned fill_word(unsigned m, unsigned s) {
 
 // One flood-fill sweep: a block loads a tile of TW x TY x TZ words with a one-word halo and fills it until nothing changes
 // (the halo stays as loaded; masks only gain bits, so a word a neighbour block is about to extend is caught by the next
-// sweep).  Sweep r sets flag r & 3 when it changed something, reads that of the sweep before (nothing changed then: the
-// fixed point is reached, exit) and clears the next one's.
-constexpr int SB_TW = 2, SB_TY = 16, SB_TZ = 16;
-__global__ void __launch_bounds__(SB_TW* SB_TY* SB_TZ) k_sb_flood(const unsigned* __restrict__ mask, unsigned* reached,
-                                                                  const BitGrid g, int* flags, int r) {
+// sweep).  Only tiles with a face neighbour that the sweep before changed can change (all in the first sweep): tiles note a
+// change in stamp, as the number of the sweep modulo 251 plus one, so nothing has to be cleared between sweeps (a note 251
+// sweeps old reads as new, which costs a visit).  Sweep r sets flag r & 3 when it changed something, reads that of the sweep before
+// (nothing changed then: the fixed point is reached, exit) and clears the next one's.
+constexpr int SB_TW = 2, SB_TY = 16, SB_TZ = 32, SB_THREADS = SB_TW * SB_TY * SB_TZ / 2;
+__global__ void __launch_bounds__(SB_THREADS) k_sb_flood(const unsigned* __restrict__ mask, unsigned* reached,
+                                                                  const BitGrid g, int* flags, unsigned char* stamp,
+                                                                  long long sweep) {
     __shared__ unsigned t[SB_TZ + 2][SB_TY + 2][SB_TW + 2];
+    const int r = (int)(sweep & 3);
     if (blockIdx.x == 0 && threadIdx.x == 0) flags[(r + 1) & 3] = 0;
     if (((volatile int*)flags)[(r + 3) & 3] == 0) return;  // uniform over the grid: written by earlier launches only
     const int nbx = (g.W + SB_TW - 1) / SB_TW, nby = (g.n2 + SB_TY - 1) / SB_TY;
     const int bx = blockIdx.x % nbx, by = (blockIdx.x / nbx) % nby, bz = blockIdx.x / (nbx * nby);
+    if (sweep > 0) {
+        const int nbz = (g.n3 + SB_TZ - 1) / SB_TZ;
+        const unsigned char last = (unsigned char)((sweep - 1) % 251 + 1);
+        auto changed = [&](int dx, int dy, int dz) {
+            const int x = bx + dx, y = by + dy, z = bz + dz;
+            return x >= 0 && x < nbx && y >= 0 && y < nby && z >= 0 && z < nbz &&
+                   ((volatile unsigned char*)stamp)[((long long)z * nby + y) * nbx + x] == last;
+        };
+        // (a neighbour's note of this very sweep may hide that of the last one: the tile is then visited in the next)
+        bool any = false;
+        if (threadIdx.x < 6) {
+            const int s = threadIdx.x & 1 ? 1 : -1, a = threadIdx.x >> 1;
+            any = changed(a == 0 ? s : 0, a == 1 ? s : 0, a == 2 ? s : 0);
+        }
+        if (!__syncthreads_or(any)) return;
+    }
     const int x0 = bx * SB_TW - 1, y0 = by * SB_TY - 1, z0 = bz * SB_TZ - 1;
-    constexpr int CELLS = (SB_TZ + 2) * (SB_TY + 2) * (SB_TW + 2), THREADS = SB_TW * SB_TY * SB_TZ;
-    for (int q = threadIdx.x; q < CELLS; q += THREADS) {
+    constexpr int CELLS = (SB_TZ + 2) * (SB_TY + 2) * (SB_TW + 2), HALF = SB_TZ / 2;
+    for (int q = threadIdx.x; q < CELLS; q += SB_THREADS) {
         const int lx = q % (SB_TW + 2), ly = (q / (SB_TW + 2)) % (SB_TY + 2), lz = q / ((SB_TW + 2) * (SB_TY + 2));
         const int x = x0 + lx, y = y0 + ly, z = z0 + lz;
         const bool in = x >= 0 && x < g.W && y >= 0 && y < g.n2 && z >= 0 && z < g.n3;
         t[lz][ly][lx] = in ? ((volatile unsigned*)reached)[((long long)z * g.n2 + y) * g.W + x] : 0u;
     }
+    // a thread owns two words, HALF planes apart
     const int lx = threadIdx.x % SB_TW + 1, ly = (threadIdx.x / SB_TW) % SB_TY + 1, lz = threadIdx.x / (SB_TW * SB_TY) + 1;
     const int x = x0 + lx, y = y0 + ly, z = z0 + lz;
-    const bool in = x < g.W && y < g.n2 && z < g.n3;
-    const long long w = ((long long)z * g.n2 + y) * g.W + x;
-    const unsigned m = in ? mask[w] : 0u;
+    const bool in[2] = {x < g.W && y < g.n2 && z < g.n3, x < g.W && y < g.n2 && z + HALF < g.n3};
+    const long long w[2] = {((long long)z * g.n2 + y) * g.W + x, ((long long)(z + HALF) * g.n2 + y) * g.W + x};
+    const unsigned m[2] = {in[0] ? mask[w[0]] : 0u, in[1] ? mask[w[1]] : 0u};
     __syncthreads();
-    const unsigned first = t[lz][ly][lx];
-    unsigned own = first;
-    // every pass but the last reaches at least one more cell of the tile
-    for (int it = 0; it <= 32 * THREADS; ++it) {
-        const unsigned nb = (own << 1) | (own >> 1) | (t[lz][ly][lx - 1] >> 31) | (t[lz][ly][lx + 1] << 31) |
-                            t[lz][ly - 1][lx] | t[lz][ly + 1][lx] | t[lz - 1][ly][lx] | t[lz + 1][ly][lx] | own;
-        const unsigned f = own | fill_word(m, nb & m);
-        const int ch = f != own;
-        own = f;
+    const unsigned first[2] = {t[lz][ly][lx], t[lz + HALF][ly][lx]};
+    unsigned own[2] = {first[0], first[1]};
+    // Rounds of PASSES passes without a barrier: threads see each other's words in any order, but words only gain bits, so a
+    // round in which no word of the block changed ends at the fixed point.  Every round but the last reaches at least one
+    // more cell of the tile.
+    constexpr int PASSES = 6;
+    volatile unsigned(*v)[SB_TY + 2][SB_TW + 2] = t;
+    for (int it = 0; it <= 64 * SB_THREADS; ++it) {
+        int ch = 0;
+#pragma unroll 1
+        for (int q = 0; q < PASSES; ++q) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int k = lz + h * HALF;
+                const unsigned nb = (own[h] << 1) | (own[h] >> 1) | (v[k][ly][lx - 1] >> 31) | (v[k][ly][lx + 1] << 31) |
+                                    v[k][ly - 1][lx] | v[k][ly + 1][lx] | v[k - 1][ly][lx] | v[k + 1][ly][lx] | own[h];
+                const unsigned f = own[h] | fill_word(m[h], nb & m[h]);
+                if (f != own[h]) {
+                    v[k][ly][lx] = own[h] = f;
+                    ch = 1;
+                }
+            }
+        }
         if (!__syncthreads_or(ch)) break;
-        if (ch) t[lz][ly][lx] = f;
-        __syncthreads();
     }
-    if (in && own != first) {
-        reached[w] = own;
-        flags[r & 3] = 1;  // every writer stores the same value
-    }
+    for (int h = 0; h < 2; ++h)
+        if (in[h] && own[h] != first[h]) {
+            reached[w[h]] = own[h];
+            flags[r] = 1;  // every writer stores the same value, also in the note
+            stamp[blockIdx.x] = (unsigned char)(sweep % 251 + 1);
+        }
 }
 
 __global__ void __launch_bounds__(SF_THREADS) k_sb_apply(const float* __restrict__ prob, const double* seed,
                                                          const unsigned* __restrict__ reached,
                                                          const unsigned* __restrict__ water, const BitGrid g, double* out) {
     const int lane = threadIdx.x & 31;
-    const long long words = (long long)g.W * g.n2 * g.n3;
-    const long long warps = (long long)gridDim.x * (SF_THREADS / 32);
-    for (long long w0 = ((long long)blockIdx.x * (SF_THREADS / 32) + (threadIdx.x >> 5)) * WPI; w0 < words;
-         w0 += warps * WPI) {
+    const int rows = g.n2 * g.n3, step = gridDim.x * (SF_THREADS / 32);
+    for (int row = blockIdx.x * (SF_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += step)
+    for (int wx = 0; wx < g.W; wx += WPI) {
+        const long long w0 = (long long)row * g.W + wx;
         float p[WPI];
         double s[WPI];
         long long q[WPI];
         bool in[WPI], put[WPI];
 #pragma unroll
         for (int r = 0; r < WPI; ++r) {
-            const long long w = w0 + r;
-            const long long row = w / g.W;
-            const int x = (int)(w - row * g.W) * 32 + lane;
-            in[r] = w < words && x < g.n1;
-            put[r] = in[r] && ((reached[w] & water[w]) >> lane & 1u);
-            q[r] = row * g.n1 + x;
+            const int x = (wx + r) * 32 + lane;
+            in[r] = x < g.n1;
+            put[r] = in[r] && ((reached[w0 + r] & water[w0 + r]) >> lane & 1u);
+            q[r] = (long long)row * g.n1 + x;
             s[r] = in[r] ? seed[q[r]] : 0.0;
             p[r] = put[r] ? prob[q[r]] : 0.f;
         }
@@ -281,11 +313,12 @@ extern "C" pf_status pfnn_seed_connect(const float* prob, const double* phi_seed
         const long long words = (long long)g.W * n2 * n3;
         const int masks = erode ? 5 : 4;
         const long long tiles = ((g.W + SB_TW - 1) / SB_TW) * (long long)((n2 + SB_TY - 1) / SB_TY) * ((n3 + SB_TZ - 1) / SB_TZ);
-        if (4 * masks * words + 16 <= 16 * ((n + 15) / 16) + 4 && tiles < (1LL << 31)) {
+        if (4 * masks * words + 16 + tiles <= 16 * ((n + 15) / 16) + 4 && words < (1LL << 30)) {
             int* flags = reinterpret_cast<int*>(work);
             unsigned* ice = reinterpret_cast<unsigned*>(work + 16);
             unsigned *reached = ice + words, *spare = reached + words, *water = spare + words, *whole = water + words;
-            const int nbi = sf_blocks(words * 32 / WPI), nbw = sf_blocks(words);
+            unsigned char* stamp = work + 16 + 4 * masks * words;
+            const int nbi = sf_blocks((long long)n2 * n3 * 32), nbw = sf_blocks(words);
             k_sb_init<<<nbi, SF_THREADS, 0, s>>>(prob, phi_seed, G, zeta, g, ice, reached, water);
             pfgb::count_launch();
             if (erode && cudaMemcpyAsync(whole, ice, 4 * words, cudaMemcpyDeviceToDevice, s) != cudaSuccess) return PF_E_CUDA;
@@ -298,10 +331,12 @@ extern "C" pf_status pfnn_seed_connect(const float* prob, const double* phi_seed
             }
             long long done = 0;
             // every sweep that changes something reaches at least one more cell: at most n sweeps
-            if (cudaMemsetAsync(flags, 0xff, 4 * sizeof(int), s) != cudaSuccess) return PF_E_CUDA;
+            if (cudaMemsetAsync(flags, 0xff, 4 * sizeof(int), s) != cudaSuccess ||
+                cudaMemsetAsync(stamp, 0, tiles, s) != cudaSuccess)
+                return PF_E_CUDA;
             for (;;) {
                 for (int r = 0; r < SWEEPS_PER_CHECK; ++r)
-                    k_sb_flood<<<(unsigned)tiles, SB_TW * SB_TY * SB_TZ, 0, s>>>(ice, reached, g, flags, (int)((done + r) & 3));
+                    k_sb_flood<<<(unsigned)tiles, SB_THREADS, 0, s>>>(ice, reached, g, flags, stamp, done + r);
                 pfgb::count_launch(SWEEPS_PER_CHECK);
                 done += SWEEPS_PER_CHECK;
                 int h = 0;
