@@ -135,8 +135,11 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
                  : "memory");
 }
 
+// The .aligned instructions on TMEM need all 32 lanes together: the lanes meet first, whatever the caller did for some of
+// them only (cells outside the grid, waits that ended after different numbers of tries).
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];
+    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
         "%15}, [%16];"
@@ -276,16 +279,17 @@ k_conv_umma(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     for (int c0 = 0; c0 < p.cout; c0 += 16) {
         float o[16];
         tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, o);  // whole warp, always
-        if (!inside) continue;
-        if (p.bias) {
+        if (inside) {
+            if (p.bias) {
 #pragma unroll
-            for (int q = 0; q < 16; ++q) o[q] += p.bias[c0 + q];
-        }
-        if (p.relu) {
+                for (int q = 0; q < 16; ++q) o[q] += p.bias[c0 + q];
+            }
+            if (p.relu) {
 #pragma unroll
-            for (int q = 0; q < 16; ++q) o[q] = fmaxf(o[q], 0.f);
+                for (int q = 0; q < 16; ++q) o[q] = fmaxf(o[q], 0.f);
+            }
+            store_cell16(p.y, p.yf, v * p.ldy + p.yoff + c0, p.accumulate, o);
         }
-        store_cell16(p.y, p.yf, v * p.ldy + p.yoff + c0, p.accumulate, o);
     }
 
     // after a failed wait, the TMA loads still in flight must land before the block's shared memory
@@ -408,6 +412,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, lo
 // zero the accumulator columns [0, cols) of this warp's TMEM lane quadrant
 __device__ __forceinline__ void tmem_zero(uint32_t taddr, int cols) {
     const uint32_t z = 0u;
+    __syncwarp();  // as in tmem_ld16
     for (int c = 0; c < cols; c += 16)
         asm volatile(
             "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, "
@@ -600,14 +605,15 @@ k_conv_march(const __grid_constant__ CUtensorMap tmX, const MarchArgs p) {
                     const long long v = (((long long)br.n * p.D + z) * p.H + y) * p.W + x;
                     float o[16];
                     tmem_ld16(acc + (uint32_t)((br.planes - 1 - zo) * p.cout + c0), o);
-                    if (!inside) continue;
+                    if (inside) {
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) o[e] += bias[e];
-                    if (p.relu) {
+                        for (int e = 0; e < 16; ++e) o[e] += bias[e];
+                        if (p.relu) {
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) o[e] = fmaxf(o[e], 0.f);
+                            for (int e = 0; e < 16; ++e) o[e] = fmaxf(o[e], 0.f);
+                        }
+                        store_cell16(p.y, p.yf, v * p.ldy + p.yoff + c0, p.accumulate, o);
                     }
-                    store_cell16(p.y, p.yf, v * p.ldy + p.yoff + c0, p.accumulate, o);
                 }
             }
             tmem_zero(acc, br.planes * p.cout);
@@ -861,17 +867,18 @@ k_conv_wide(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     for (int c = 0; c < p.nc; c += 16) {
                         float r[16];
                         tmem_ld16(acc + (uint32_t)c, r);
-                        if (!inside) continue;
-                        const int ch = it.c0 + c;
-                        if (p.bias) {
+                        if (inside) {
+                            const int ch = it.c0 + c;
+                            if (p.bias) {
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) r[e] += __ldg(p.bias + ch + e);
-                        }
-                        if (p.relu) {
+                                for (int e = 0; e < 16; ++e) r[e] += __ldg(p.bias + ch + e);
+                            }
+                            if (p.relu) {
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) r[e] = fmaxf(r[e], 0.f);
+                                for (int e = 0; e < 16; ++e) r[e] = fmaxf(r[e], 0.f);
+                            }
+                            store_cell16(p.y, p.yf, v * p.ldy + p.yoff + ch, p.accumulate, r);
                         }
-                        store_cell16(p.y, p.yf, v * p.ldy + p.yoff + ch, p.accumulate, r);
                     }
                     tmem_zero(acc, p.nc);
                 }
@@ -1053,9 +1060,10 @@ k_wgrad_umma(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
         for (int c0 = 0; c0 < p.cout; c0 += 16) {
             float o[16];
             tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * p.cout + c0), o);  // whole warp, always
-            if (!live) continue;
+            if (live) {
 #pragma unroll
-            for (int k = 0; k < 16; ++k) atomicAdd(dst + (long long)(c0 + k) * p.cin, o[k]);
+                for (int k = 0; k < 16; ++k) atomicAdd(dst + (long long)(c0 + k) * p.cin, o[k]);
+            }
         }
     }
 
