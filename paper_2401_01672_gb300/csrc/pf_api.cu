@@ -512,6 +512,13 @@ static StageArgs<T> make_args(pf_grid* g) {
     return a;
 }
 
+// A launch takes at most 65535 tiles along y and chunks along z: longer grids take taller blocks and more planes.
+constexpr int GRID_YZ = 65535;
+static bool tiles_fit(const pf_grid* g, int by, int zc) {
+    const int h = tile_shape(g->n1, g->n2, by).h;
+    return ((long long)g->n2 + h - 1) / h <= GRID_YZ && ((long long)g->n3 + zc - 1) / zc <= GRID_YZ;
+}
+
 // Tiles of a grid that nobody set or tuned: blocks of 32 x 4 threads (never slower than 8 by more than 3 %, 16 always),
 // and planes per block by the planes of tiles each place on the chip gets, m = plane tiles / resident blocks: a large grid
 // amortises a block's prologue (3 planes loaded, one block's latency) over many planes, a small one needs every block it
@@ -520,10 +527,13 @@ static StageArgs<T> make_args(pf_grid* g) {
 // 8 % of the best of 24 shapes on nine grids of 32^3 to 256^3.  (32 planes of 32 x 8 threads everywhere: 302 us an attempt
 // at 32^3 in the binary64 micro model, now 23; 128^3 742 and 315 us.)
 static void default_tiles(const pf_grid* g, double plane_tiles, int* by, int* zc) {
+    const int longest = (int)(((long long)g->n3 + GRID_YZ - 1) / GRID_YZ);  // planes a chunk cannot do without
     *by = 4;
+    while (*by < 16 && !tiles_fit(g, *by, longest)) *by *= 2;
     const double m = plane_tiles / (152.0 * (is_f32(g) ? 7 : 6));
     const double z = (is_f32(g) ? 2.2 : 0.8) * std::sqrt(m);
     *zc = z < 1.5 ? 1 : (z > 24.0 ? 24 : (int)(z + 0.5));
+    if (*zc < longest) *zc = longest;
 }
 static double plane_tiles(const pf_grid* g, int by) {
     const TileShape ts = tile_shape(g->n1, g->n2, by);
@@ -1519,6 +1529,7 @@ pf_status pf_batch_create(int n, pf_grid* const* grids, pf_batch** out) {
         if (!grids[q]->tiles_set) {
             int by, zc;
             default_tiles(grids[q], total, &by, &zc);
+            if (by > b->by) b->by = by;
             if (zc != grids[q]->zc) free_graph(grids[q]);
             grids[q]->zc = zc;
         }
