@@ -1245,14 +1245,12 @@ pf_status conv_wide(const void* x, int ldx, int xoff, const void* w, int cin, in
     // multiplications and its reads from shared memory; half of the windows of three groups wrap around the ring
     const auto mma = [&](int m) { return std::max(m * a.nc / 2, 32 + m * a.nc / 4); };
     const long long full = (mma(3) + mma(1) + mma(2)) / 2;
+    // the tile planes of an item: one and two groups at each end, three between them (one plane: one group each time)
+    const long long ends = 2LL * (mma(1) + mma(2)), single = 3LL * mma(1);
     long long best = -1;
     for (int zc = 1; zc <= d; ++zc) {
         const long long tz = (d + zc - 1) / zc, items = (long long)a.tx * a.ty * tz * n * a.ncc;
-        long long clocks = 0;
-        for (int z = 0; z < zc + 2; ++z) {
-            const int m = std::min(2, z) - std::max(0, z - zc + 1) + 1;
-            clocks += m == 3 ? full : mma(m);
-        }
+        const long long clocks = zc == 1 ? single : ends + (zc - 2) * full;
         const long long cost = ((items + 151) / 152) * clocks * 2 * 9 * (cin / 16) + 4000;
         if (best < 0 || cost < best) {
             best = cost;
