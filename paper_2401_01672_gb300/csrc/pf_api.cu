@@ -518,26 +518,60 @@ static bool tiles_fit(const pf_grid* g, int by, int zc) {
     const int h = tile_shape(g->n1, g->n2, by).h;
     return ((long long)g->n2 + h - 1) / h <= GRID_YZ && ((long long)g->n3 + zc - 1) / zc <= GRID_YZ;
 }
+static double lateral_tiles(const pf_grid* g, int by) {
+    const TileShape ts = tile_shape(g->n1, g->n2, by);
+    return (double)((g->n1 + ts.w - 1) / ts.w) * ((g->n2 + ts.h - 1) / ts.h);
+}
 
-// Tiles of a grid that nobody set or tuned: blocks of 32 x 4 threads (never slower than 8 by more than 3 %, 16 always),
-// and planes per block by the planes of tiles each place on the chip gets, m = plane tiles / resident blocks: a large grid
+// The Temp model in binary64 is bound by the tanh of every cell that a block loads, its halo and its chunk's two extra planes
+// included, so both block heights and long chunks pay, as far as the blocks still spread over the chip: the fewest cells
+// loaded by a multiprocessor's share of the blocks and one more (the last ones do not end together; temperatures near the
+// melting point in one part of the grid make some blocks longer).  Measured at 22 grids of 16^3 to 192^3 and flat ones,
+// with temperatures near the melting point everywhere and in a front only: within 21 % of the best of 39 shapes, never more
+// than 2 % slower than 8 x 32.  128^3, near everywhere: 2.37 ms an attempt (3.65 with the rule below, 2.50 with 8 x 32).
+static const int kTempZC[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 24, 32};
+static bool temp_tiles(const pf_grid* g, double share, int only_by, int* by, int* zc) {
+    double best = INFINITY;
+    for (int b = 4; b <= 16; b *= 2) {
+        if (only_by && b != only_by) continue;
+        const TileShape ts = tile_shape(g->n1, g->n2, b);
+        for (int z : kTempZC) {
+            if ((z > 1 && z > 2 * g->n3) || !tiles_fit(g, b, z)) continue;
+            const double blocks = share * lateral_tiles(g, b) * ((g->n3 + z - 1) / z);
+            const int planes = std::min(z, g->n3);
+            const double cost = (std::ceil(blocks / 152.0) + 1.0) * ((planes + 3.0) * ts.w * ts.h + (planes + 2.0) * 2.0 * (ts.w + ts.h));
+            if (cost < best) {
+                best = cost;
+                *by = b;
+                *zc = z;
+            }
+        }
+    }
+    return best < INFINITY;
+}
+
+// Tiles of a grid that nobody set or tuned: blocks of 32 x 4 threads, and planes per block by the planes of tiles each place
+// on the chip gets, m = plane tiles / resident blocks (`share`: those of all instances of a batch over this grid's): a large grid
 // amortises a block's prologue (3 planes loaded, one block's latency) over many planes, a small one needs every block it
 // can get.  Measured best: binary64 1 plane at 32^3 and 64^3 (m = 2.2), 3 at 128^3 (m = 18), 5 to 12 at 256^3 (m = 144);
 // binary32 1 at 32^3, 3 at 64^3 (m = 1.9), 4 at 70^3, 10 at 128^3 (m = 15), 24 at 256^3; the formula stays within about
 // 8 % of the best of 24 shapes on nine grids of 32^3 to 256^3.  (32 planes of 32 x 8 threads everywhere: 302 us an attempt
 // at 32^3 in the binary64 micro model, now 23; 128^3 742 and 315 us.)
-static void default_tiles(const pf_grid* g, double plane_tiles, int* by, int* zc) {
+// One or two planes: a chunk is all of them once the lateral tiles fill half of the chip (300 x 300 x 2, binary64 micro 58 us, 70
+// with a plane each), and many tiles are blocks of 8 rows, whose halo is smaller (1000 x 1000 x 1, binary32 micro 69 us, 75
+// with 4 rows).  `only_by`: a block height that is given (0: none).
+static void default_tiles(const pf_grid* g, double share, int only_by, int* by, int* zc) {
+    if (g->model == PF_MODEL_TEMP && !is_f32(g) && temp_tiles(g, share, only_by, by, zc)) return;
     const int longest = (int)(((long long)g->n3 + GRID_YZ - 1) / GRID_YZ);  // planes a chunk cannot do without
     *by = 4;
-    while (*by < 16 && !tiles_fit(g, *by, longest)) *by *= 2;
-    const double m = plane_tiles / (152.0 * (is_f32(g) ? 7 : 6));
-    const double z = (is_f32(g) ? 2.2 : 0.8) * std::sqrt(m);
+    const double places = 152.0 * (is_f32(g) ? 7 : 6), lateral = share * lateral_tiles(g, 4);
+    const double z = (is_f32(g) ? 2.2 : 0.8) * std::sqrt(lateral * g->n3 / places);
     *zc = z < 1.5 ? 1 : (z > 24.0 ? 24 : (int)(z + 0.5));
+    if (g->n3 <= 2 && lateral > 0.5 * places) *zc = g->n3;
+    if (g->n3 <= 2 && lateral > 3.0 * places) *by = 8;
+    while (*by < 16 && !tiles_fit(g, *by, longest)) *by *= 2;
+    if (only_by) *by = only_by;
     if (*zc < longest) *zc = longest;
-}
-static double plane_tiles(const pf_grid* g, int by) {
-    const TileShape ts = tile_shape(g->n1, g->n2, by);
-    return (double)((g->n1 + ts.w - 1) / ts.w) * ((g->n2 + ts.h - 1) / ts.h) * g->n3;
 }
 
 static cudaError_t launch_stage(pf_grid* g, int stage, cudaStream_t s) {
@@ -672,7 +706,7 @@ static pf_status create_impl(int n1, int n2, int n3, double h, int model, int re
     c.theta_freeze = p->theta_freeze; c.theta_thaw = p->theta_thaw; c.t_freeze = p->t_freeze;
     fill_coefs(g->k64, *p, h);
     fill_coefs(g->k32, *p, h);
-    default_tiles(g, plane_tiles(g, 4), &g->by, &g->zc);
+    default_tiles(g, 1.0, 0, &g->by, &g->zc);
     auto alloc = [&](size_t bytes) -> void* {
         void* q = nullptr;
         if (cudaMalloc(&q, bytes) != cudaSuccess) return nullptr;
@@ -1524,13 +1558,17 @@ pf_status pf_batch_create(int n, pf_grid* const* grids, pf_batch** out) {
     b->by = grids[0]->by;
     // instances nobody set tiles for share the chip: their planes per block follow from the tiles of all
     double total = 0.0;
-    for (int q = 0; q < n; ++q) total += plane_tiles(grids[q], b->by);
+    for (int q = 0; q < n; ++q) total += lateral_tiles(grids[q], 4) * grids[q]->n3;
+    auto share = [&](const pf_grid* g) { return total / (lateral_tiles(g, 4) * g->n3); };
+    int by, zc;
+    if (!grids[0]->tiles_set) default_tiles(grids[0], share(grids[0]), 0, &b->by, &zc);
+    for (int q = 0; q < n; ++q)  // each can still be run by itself
+        while (!grids[q]->tiles_set && b->by < 16 && !tiles_fit(grids[q], b->by, grids[q]->n3)) b->by *= 2;
     for (int q = 0; q < n; ++q)
         if (!grids[q]->tiles_set) {
-            int by, zc;
-            default_tiles(grids[q], total, &by, &zc);
-            if (by > b->by) b->by = by;
-            if (zc != grids[q]->zc) free_graph(grids[q]);
+            default_tiles(grids[q], share(grids[q]), b->by, &by, &zc);
+            if (by != grids[q]->by || zc != grids[q]->zc) free_graph(grids[q]);
+            grids[q]->by = by;
             grids[q]->zc = zc;
         }
     b->stream = grids[0]->stream;
