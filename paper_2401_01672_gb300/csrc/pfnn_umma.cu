@@ -643,7 +643,7 @@ k_conv_march(const __grid_constant__ CUtensorMap tmX, const MarchArgs p) {
 // ---------------------------------------------------------------- wide layers: marching pairs of bricks, streamed weights
 // For larger cin x cout the weights do not fit shared memory beside the input (442 KB for 128 -> 64 channels).  Windows,
 // stacked taps dz and the order of the products are those of k_conv_march; the weights of (dy, dx, block of ck channels),
-// 3 nc rows (nc = up to 64 output channels; more are other work items), come through a ring of three stages for every tile
+// 3 nc rows (nc = 16, 32 or 64 output channels), come through a ring of three stages for every tile
 // plane, and two bricks side by side (16 x 16 columns, one tile of 18 x 18 cells) use each stage, so a stage feeds about 800
 // clocks of MMAs.  A work item marches along z over zc planes; the tile planes come through a ring of (plane, channel
 // block) slots, the accumulators of each brick lie in a ring of four planes (a window's column groups wrap around its end:
@@ -656,7 +656,7 @@ constexpr int WD_SLOTS = 4;      // most tile slots
 constexpr int WD_ACC = 4;        // accumulator planes per brick
 constexpr int WT_X = 2 * HB_X + 2;
 struct WideArgs {
-    int nc, ncc;                  // output channels of one work item, work items per brick pair
+    int nc;                       // output channels
     int ck, ncb;                  // channels per K block, K blocks
     int zc, slots;                // output planes per work item, tile slots
     int D, H, W, tx, ty, tz;
@@ -682,12 +682,10 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
 }
 
 struct WideItem {
-    int x0, y0, z0, n, c0, planes;
+    int x0, y0, z0, n, planes;
 };
 __device__ __forceinline__ WideItem wide_item(const WideArgs& p, long long q) {
     WideItem r;
-    r.c0 = (int)(q % p.ncc) * p.nc;
-    q /= p.ncc;
     r.x0 = (int)(q % p.tx) * (2 * HB_X);
     q /= p.tx;
     r.y0 = (int)(q % p.ty) * HB_Y;
@@ -762,7 +760,7 @@ k_conv_wide(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                         if (!ok || s_fail) { ok = false; break; }
                         mbar_expect_tx(rfull + 8u * rs, p.ring_tx);
                         if (l * p.ncb + cb != p.withhold) {
-                            tma_load_4d(ring0 + (uint32_t)rs * p.ring_bytes, &tmB, rfull + 8u * rs, cb * p.ck, it.c0, l, 0);
+                            tma_load_4d(ring0 + (uint32_t)rs * p.ring_bytes, &tmB, rfull + 8u * rs, cb * p.ck, 0, l, 0);
                             rpending |= bit;
                         } else {
                             rpending &= ~bit;
@@ -868,16 +866,15 @@ k_conv_wide(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                         float r[16];
                         tmem_ld16(acc + (uint32_t)c, r);
                         if (inside) {
-                            const int ch = it.c0 + c;
                             if (p.bias) {
 #pragma unroll
-                                for (int e = 0; e < 16; ++e) r[e] += __ldg(p.bias + ch + e);
+                                for (int e = 0; e < 16; ++e) r[e] += __ldg(p.bias + c + e);
                             }
                             if (p.relu) {
 #pragma unroll
                                 for (int e = 0; e < 16; ++e) r[e] = fmaxf(r[e], 0.f);
                             }
-                            store_cell16(p.y, p.yf, v * p.ldy + p.yoff + ch, p.accumulate, r);
+                            store_cell16(p.y, p.yf, v * p.ldy + p.yoff + c, p.accumulate, r);
                         }
                     }
                     tmem_zero(acc, p.nc);
@@ -1213,22 +1210,42 @@ pf_status conv_march(const void* x, int ldx, int xoff, const void* w, int cin, i
     return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
 }
 
-// The wide-layer kernel: more weights than fit shared memory, brick pairs that are mostly full, and enough 16 x 16 planes of
-// them for the chip (a work item needs two more tile planes than it has output planes).  Below that k_conv_umma, which
-// has 128 voxels per block, fills more SMs.
+// Brick of 128 cells of k_conv_umma: 32 x 4 x 1, 16 x 8 x 1 or 8 x 8 x 2 (x fastest), the widest that the grid fills.
+struct UmmaBricks {
+    int wb, hb, db;
+    long long tx, ty, tz;
+};
+UmmaBricks umma_bricks(int d, int h, int wd) {
+    UmmaBricks b;
+    b.wb = wd >= 32 ? 32 : (wd >= 16 ? 16 : 8);
+    b.hb = b.wb == 32 ? 4 : 8;
+    b.db = UM / (b.wb * b.hb);
+    b.tx = (wd + b.wb - 1) / b.wb;
+    b.ty = (h + b.hb - 1) / b.hb;
+    b.tz = (d + b.db - 1) / b.db;
+    return b;
+}
+
+// The wide-layer kernel: more weights than fit shared memory, in blocks of 32 or 64 input channels, all output channels in
+// one pass (of several 32- or 64-channel passes each reads the input again: 128 -> 128 channels on 64^3 276 us, k_conv_umma
+// 205; of 16-channel ones 64 -> 80 284 and 109), bricks of which no more hang over the grid than of k_conv_umma's (by less than 1.4: at
+// 1.6, 20 rows, 64 -> 64 157 and 136 us, at 1.33, 24 rows, 157 and 165), and enough 16 x 16 planes of them for the chip (a
+// work item needs two more tile planes than it has output planes: one plane 103 and 91 us, two 71 and 91).  64 -> 64
+// channels: 128 planes 23 and 19 us, 297 of 33^3 39 and 33, 360 of 40^3 34 and 48, 512 39 and 62, 1024 64 and 107.
 bool wide_shape(int cin, int cout, int n, int d, int h, int wd) {
-    const int nc = cout % 64 == 0 ? 64 : (cout % 32 == 0 ? 32 : 16), ck = cin % 64 == 0 ? 64 : (cin % 32 == 0 ? 32 : 16);
-    const long long planes = (long long)((wd + 15) / 16) * ((h + 15) / 16) * d * n * (cout / nc);
-    return cin * cout > 2048 && cin / ck <= 3 && (wd > 24 || (wd > 8 && wd <= 16)) && h >= HB_Y && planes >= 500;
+    if (cin % 32 || (cout != 16 && cout != 32 && cout != 64) || cin * cout <= 2048) return false;
+    const UmmaBricks b = umma_bricks(d, h, wd);
+    const long long planes = (long long)((wd + 15) / 16) * ((h + 15) / 16) * d * n;
+    return cin / (cin % 64 == 0 ? 64 : 32) <= 3 && d >= 2 && wd > HB_X && h >= HB_Y && planes >= 500 &&
+           256.0 * planes <= 1.4 * UM * (double)(b.tx * b.ty * b.tz * n);
 }
 
 pf_status conv_wide(const void* x, int ldx, int xoff, const void* w, int cin, int cout, const float* bias, int relu,
                     int flip, void* y_bf16, float* y_f32, int ldy, int yoff, int accumulate, int n, int d, int h, int wd,
                     cudaStream_t stream, PFN_cuTensorMapEncodeTiled_v12000 enc) {
     WideArgs a{};
-    a.nc = cout % 64 == 0 ? 64 : (cout % 32 == 0 ? 32 : 16);
-    a.ncc = cout / a.nc;
-    a.ck = cin % 64 == 0 ? 64 : (cin % 32 == 0 ? 32 : 16);
+    a.nc = cout;
+    a.ck = cin % 64 == 0 ? 64 : 32;
     a.ncb = cin / a.ck;
     a.D = d;
     a.H = h;
@@ -1249,7 +1266,7 @@ pf_status conv_wide(const void* x, int ldx, int xoff, const void* w, int cin, in
     const long long ends = 2LL * (mma(1) + mma(2)), single = 3LL * mma(1);
     long long best = -1;
     for (int zc = 1; zc <= d; ++zc) {
-        const long long tz = (d + zc - 1) / zc, items = (long long)a.tx * a.ty * tz * n * a.ncc;
+        const long long tz = (d + zc - 1) / zc, items = (long long)a.tx * a.ty * tz * n;
         const long long clocks = zc == 1 ? single : ends + (zc - 2) * full;
         const long long cost = ((items + 151) / 152) * clocks * 2 * 9 * (cin / 16) + 4000;
         if (best < 0 || cost < best) {
@@ -1304,16 +1321,14 @@ pf_status conv_wide(const void* x, int ldx, int xoff, const void* w, int cin, in
     static std::once_flag attr_once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(attr_once, [] {
-        for (auto f : {k_conv_wide<16, false>, k_conv_wide<32, false>, k_conv_wide<64, false>, k_conv_wide<16, true>,
-                       k_conv_wide<32, true>, k_conv_wide<64, true>}) {
+        for (auto f : {k_conv_wide<32, false>, k_conv_wide<64, false>, k_conv_wide<32, true>, k_conv_wide<64, true>}) {
             const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 216 * 1024);
             if (e != cudaSuccess) attr_err = e;
         }
     });
     if (attr_err != cudaSuccess || smem > 216u * 1024u) return PF_E_CUDA;
-    auto k = a.ck == 16 ? (flip ? k_conv_wide<16, true> : k_conv_wide<16, false>)
-             : a.ck == 32 ? (flip ? k_conv_wide<32, true> : k_conv_wide<32, false>)
-                          : (flip ? k_conv_wide<64, true> : k_conv_wide<64, false>);
+    auto k = a.ck == 32 ? (flip ? k_conv_wide<32, true> : k_conv_wide<32, false>)
+                        : (flip ? k_conv_wide<64, true> : k_conv_wide<64, false>);
     k<<<(unsigned)std::min<long long>(a.items, 152), MR_THR, smem, stream>>>(mA, mB, a);
     pfgb::count_launch();
     return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
@@ -1446,16 +1461,16 @@ pf_status pfnn_conv3d(const void* x, int ldx, int xoff, const void* w, int cin, 
     a.cout = cout;
     a.ck = cin % 64 == 0 ? 64 : (cin % 32 == 0 ? 32 : 16);
     a.nkb = cin / a.ck;
-    // brick of 128 cells: 32 x 4 x 1, 16 x 8 x 1 or 8 x 8 x 2 (x fastest), the widest that the grid fills
-    a.wb = wd >= 32 ? 32 : (wd >= 16 ? 16 : 8);
-    a.hb = a.wb == 32 ? 4 : 8;
-    a.db = UM / (a.wb * a.hb);
+    const UmmaBricks bricks = umma_bricks(d, h, wd);
+    a.wb = bricks.wb;
+    a.hb = bricks.hb;
+    a.db = bricks.db;
     a.D = d;
     a.H = h;
     a.W = wd;
-    a.tx = (wd + a.wb - 1) / a.wb;
-    a.ty = (h + a.hb - 1) / a.hb;
-    a.tz = (d + a.db - 1) / a.db;
+    a.tx = (int)bricks.tx;
+    a.ty = (int)bricks.ty;
+    a.tz = (int)bricks.tz;
     a.flip = flip;
     a.relu = relu;
     a.withhold = g_test_withhold;
