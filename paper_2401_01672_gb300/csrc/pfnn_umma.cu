@@ -918,16 +918,17 @@ k_conv_wide(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 //   outside the grid, and keeps three planes of X, so every value is loaded once (and its halo).
 //   A (M) = X: core matrices along M are 160 bytes apart, which walks the chunks of a row of the tile and
 //   then the next row, so for 16 or 32 channels the three taps dy = -1, 0, +1 lie along M by themselves
-//   ("stacked": 6 of 8 or 12 of 16 core matrices used); 64 and 128 channels fill M = 64 or 128 with one tap.
+//   ("stacked": 6 of 8 or 12 of 16 core matrices used); 128 channels fill M = 128 with one tap.
 //   B (N) = dY, N = cout.  K = 16 voxels: two rows of 8 cells, 8 MMAs per tap and plane.  The taps dx and
 //   dz are other start addresses (16 bytes further, another plane).
 //   Accumulators: cout TMEM columns per tap (per three taps when stacked); where the 27 taps need more than
-//   512 columns they are divided over blocks by dz, then by dy (rule in wgrad_plan).
+//   512 columns they are divided over blocks by dz (rule in wgrad_plan).  Taps dz whose planes all lie outside the grid
+//   for a block (one-plane grids: two of three) are left out.
 // Shared-memory reads bound it for 16 and 32 channels (2.5 to 5 KB per MMA of N = 16 or 32).
 struct WgArgs {
     int cin, cout;
-    int cb, nchunk;               // input channels of a block (16, 32, 64 or 128), cb / 8
-    int stacked, ndz, ndy;        // taps dy along M; dz and (unstacked) dy accumulated by one block
+    int cb, nchunk;               // input channels of a block (16, 32 or 128; the last one's may exceed cin), cb / 8
+    int stacked, ndz;             // taps dy along M; taps dz accumulated by one block
     int D, H, W, tx, ty;
     int zc, nzc;                  // planes per block, blocks along z
     int slots;
@@ -935,7 +936,7 @@ struct WgArgs {
     unsigned x_bytes, slot_bytes; // their places in a slot
     unsigned idesc;
     unsigned long long a_hi, b_hi;  // descriptors without the start address
-    int m64;                      // MMA M = 64 (else 128)
+    int m64;                      // MMA M = 64 (16 channels; else 128)
     int tmem_cols;
     long long tries;
     float* dw;
@@ -964,10 +965,12 @@ k_wgrad_umma(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
     const int z0 = (b % p.nzc) * p.zc, bn = b / p.nzc;
     const int nsteps = min(p.zc, p.D - z0);
     // tap group and channel block
-    const int gdy = p.stacked ? 1 : 3 / p.ndy, ngrp = (3 / p.ndz) * gdy;
-    const int grp = blockIdx.y % ngrp, cb = blockIdx.y / ngrp;
-    const int dz0 = p.ndz == 3 ? 0 : grp / gdy, dy0 = p.ndy == 3 ? 0 : grp % gdy;
-    const int ndyu = p.stacked ? 1 : p.ndy;
+    const int ngrp = 3 / p.ndz, cb = blockIdx.y / ngrp;
+    const int dz0 = p.ndz == 3 ? 0 : blockIdx.y % ngrp;
+    const int ndyu = p.stacked ? 1 : 3;
+    // the X planes of tap dz that the block multiplies, z0 + dz - 1 .. z0 + nsteps + dz - 2, meet the grid
+    auto used = [&](int dz) { return z0 + nsteps + dz - 2 >= 0 && z0 + dz - 1 < p.D; };
+    if (p.ndz == 1 && !used(dz0)) return;
     const int nacc = p.ndz * ndyu * 3;
 
     if (threadIdx.x == 0) {
@@ -1024,7 +1027,7 @@ k_wgrad_umma(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
             for (int dz = 0; dz < p.ndz; ++dz) {
                 const int zx = z0 + k + dz + xoff;
                 if (zx < 0 || zx >= p.D) continue;  // the zero padding: nothing to add
-                uint32_t xl = alo + ((sm0 + (uint32_t)((k + dz) % S) * p.slot_bytes) >> 4) + (uint32_t)dy0 * yrow;
+                uint32_t xl = alo + ((sm0 + (uint32_t)((k + dz) % S) * p.slot_bytes) >> 4);
                 uint32_t dt = tmem + (uint32_t)(dz * ndyu * 3) * p.cout;
                 for (int dy = 0; dy < ndyu; ++dy, xl += yrow)
 #pragma unroll
@@ -1049,10 +1052,11 @@ k_wgrad_umma(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
     const int core = r >> 3;
     const int dys = p.stacked ? core / p.nchunk : 0;
     const int ci = cb * p.cb + (p.stacked ? core % p.nchunk : core) * 8 + (r & 7);
-    const bool live = ready && !(p.m64 && lane >= 16) && dys < 3;
+    const bool live = ready && !(p.m64 && lane >= 16) && dys < 3 && ci < p.cin;
     for (int acc = 0; acc < nacc; ++acc) {
         const int dx = acc % 3, q = acc / 3;
-        const int dy = p.stacked ? dys : dy0 + q % ndyu, dz = dz0 + q / ndyu;
+        const int dy = p.stacked ? dys : q % ndyu, dz = dz0 + q / ndyu;
+        if (!used(dz)) continue;  // (the same for the whole block)
         float* dst = p.dw + ((long long)((dz * 3 + dy) * 3 + dx) * p.cout) * p.cin + ci;
         for (int c0 = 0; c0 < p.cout; c0 += 16) {
             float o[16];
@@ -1334,18 +1338,20 @@ pf_status conv_wide(const void* x, int ldx, int xoff, const void* w, int cin, in
     return cudaGetLastError() == cudaSuccess ? PF_OK : PF_E_CUDA;
 }
 
-// Division of a weight gradient's taps and channels over blocks.  cb: the largest of 128, 64, 32, 16 that
-// divides cin.  Stacked (dy along M) for 16 and 32 channels.  A block takes every dz (each X plane loaded
-// once) while its accumulators fit 512 TMEM columns, else one dz (dY loaded three times), else one (dz, dy).
+// Division of a weight gradient's taps and channels over blocks.  Blocks of 32 input channels with dy along M (12 of 16 core
+// matrices used); a last block of 16 reads zeros beyond.  (64 channels unstacked fill M = 64, at half the rate, in nine blocks for
+// 64 output channels: 64 -> 64 channels on 4 x 64^3 voxels 689 us, now 360; 192 -> 128 on 2 x 33^3 392 and 215; 128 -> 128 on
+// 4 x 64^3 1352 and 1083; 48 -> 32 on 50^3 in blocks of 16 105 and 73.)  128 channels unstacked with up to 32 output channels, whose
+// taps dy share a block (128 -> 32 on 4 x 64^3 468 us, stacked 640).  A block takes every dz (each X plane loaded once) while
+// its accumulators fit 512 TMEM columns, else one dz (dY loaded three times).
 void wgrad_plan(WgArgs& a) {
-    a.cb = a.cin % 128 == 0 ? 128 : (a.cin % 64 == 0 ? 64 : (a.cin % 32 == 0 ? 32 : 16));
+    a.stacked = !(a.cin % 128 == 0 && a.cout <= 32);
+    a.cb = !a.stacked ? 128 : (a.cin == 16 ? 16 : 32);
     a.nchunk = a.cb / 8;
-    a.stacked = a.cb <= 32;
-    a.m64 = a.cb == 16 || a.cb == 64;
+    a.m64 = a.cb == 16;
     const int per_dz = (a.stacked ? 3 : 9) * a.cout;
     a.ndz = 3 * per_dz <= 512 ? 3 : 1;
-    a.ndy = a.stacked || per_dz <= 512 ? 3 : 1;
-    const int cols = a.ndz * (a.stacked ? 1 : a.ndy) * 3 * a.cout;
+    const int cols = a.ndz * per_dz;
     a.tmem_cols = cols <= 64 ? 64 : (cols <= 128 ? 128 : (cols <= 256 ? 256 : 512));
 }
 
@@ -1370,8 +1376,9 @@ pf_status wgrad(const void* dy, int lddy, int dyoff, int cout, const void* x, in
     a.slot_bytes = (a.x_bytes + a.dy_tx + 127u) & ~127u;
     // the unused core matrices of a stacked A operand reach one row past a plane: at least 4 KB follow the slots
     const unsigned slack = 4096;
+    // (with up to 256 TMEM columns the slots of two blocks share the 228 KB of a multiprocessor)
     const int want = a.ndz == 3 ? 6 : 4;
-    int slots = (int)((200u * 1024u - slack) / a.slot_bytes);
+    int slots = (int)(((a.ndz == 1 && a.tmem_cols <= 256 ? 108u : 200u) * 1024u - slack) / a.slot_bytes);
     a.slots = slots < want ? slots : want;
     const size_t smem = 1024 + (size_t)a.slots * a.slot_bytes + slack;
     // MN-major, no swizzle (bits 15, 16 of the instruction descriptor = 1): leading offset = stride between
@@ -1380,17 +1387,18 @@ pf_status wgrad(const void* dy, int lddy, int dyoff, int cout, const void* x, in
               ((unsigned)((a.m64 ? 64 : 128) >> 4) << 24);
     a.a_hi = desc_plain(0, (unsigned)a.nchunk * WX_ROW, WX_ROW);
     a.b_hi = desc_plain(0, 128u, 16u * 128u);
-    const int groups = (3 / a.ndz) * (a.stacked ? 1 : 3 / a.ndy) * (cin / a.cb);
+    const int groups = (3 / a.ndz) * ((cin + a.cb - 1) / a.cb);
     // about one wave: resident blocks by shared memory (228 KB per SM) and TMEM columns (512)
     int occ = (int)(228u * 1024u / (smem + 2048));
     if (occ > 512 / a.tmem_cols) occ = 512 / a.tmem_cols;
     if (occ < 1) occ = 1;
-    // z chunks: the fewest waves x (planes + about four for the prologue, the extra X planes and the epilogue)
+    // z chunks: the fewest (waves + blocks a multiprocessor takes, which share its loads and atomics) x (planes + about four for
+    // the prologue, the extra X planes and the epilogue)
     const long long columns = (long long)a.tx * a.ty * n * groups, cap = 152LL * occ;
     long long best = -1;
-    for (int nz = 1; nz <= d && nz <= 64; ++nz) {
+    for (int nz = 1; nz <= d; nz += 1 + nz / 64) {
         const int zc = (d + nz - 1) / nz, chunks = (d + zc - 1) / zc;
-        const long long cost = ((columns * chunks + cap - 1) / cap) * (zc + 4);
+        const long long blocks = columns * chunks, cost = ((blocks + cap - 1) / cap + (blocks + 151) / 152) * (zc + 4);
         if (best < 0 || cost < best) {
             best = cost;
             a.zc = zc;
