@@ -929,7 +929,8 @@ struct WgArgs {
     int cin, cout;
     int cb, nchunk;               // input channels of a block (16, 32 or 128; the last one's may exceed cin), cb / 8
     int stacked, ndz;             // taps dy along M; taps dz accumulated by one block
-    int D, H, W, tx, ty;
+    int D, H, W, tx, ty;          // the grid's axes as the kernel takes them (wgrad_axes)
+    int tapx, tapy, tapz;         // a step's distance in the tap index along each
     int zc, nzc;                  // planes per block, blocks along z
     int slots;
     unsigned x_tx, dy_tx;         // bytes of the two boxes
@@ -1057,7 +1058,7 @@ k_wgrad_umma(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
         const int dx = acc % 3, q = acc / 3;
         const int dy = p.stacked ? dys : q % ndyu, dz = dz0 + q / ndyu;
         if (!used(dz)) continue;  // (the same for the whole block)
-        float* dst = p.dw + ((long long)((dz * 3 + dy) * 3 + dx) * p.cout) * p.cin + ci;
+        float* dst = p.dw + ((long long)(dz * p.tapz + dy * p.tapy + dx * p.tapx) * p.cout) * p.cin + ci;
         for (int c0 = 0; c0 < p.cout; c0 += 16) {
             float o[16];
             tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * p.cout + c0), o);  // whole warp, always
@@ -1355,6 +1356,31 @@ void wgrad_plan(WgArgs& a) {
     a.tmem_cols = cols <= 64 ? 64 : (cols <= 128 ? 128 : (cols <= 256 ? 256 : 512));
 }
 
+// The grid's axes in the order of the kernel's x (tiles of 8 cells), y (16) and z (marched along).  Neither operand is read along
+// rows (a cell's 8 channels are a 16-byte piece), so any order loads as fast, and grids a few cells wide fill tiles laid
+// along their long axes: taken where it leaves less than three quarters of the tile planes (128 -> 128 channels on 2000 x 2 x 2
+// voxels 94 us, 244 in their own order).  Samples follow one another along the grid's z, so with several of them only x and y change places.
+struct WgAxis {
+    int n, tap;
+    long long stride;  // voxels
+};
+struct WgAxes {
+    WgAxis a[3];
+};
+WgAxes wgrad_axes(int n, int d, int h, int wd) {
+    const WgAxis X{wd, 1, 1}, Y{h, 3, wd}, Z{d, 9, (long long)wd * h};
+    const auto planes = [](const WgAxes& q) {
+        return (double)((q.a[0].n + 7) / 8) * ((q.a[1].n + 15) / 16) * (q.a[2].n + 2.0);
+    };
+    const WgAxes own{{X, Y, Z}};
+    WgAxes best = own;
+    for (const WgAxes& q : {WgAxes{{Y, X, Z}}, WgAxes{{X, Z, Y}}, WgAxes{{Z, X, Y}}, WgAxes{{Y, Z, X}}, WgAxes{{Z, Y, X}}}) {
+        if (n > 1 && q.a[2].tap != 9) continue;
+        if (planes(q) < planes(best)) best = q;
+    }
+    return planes(best) < 0.75 * planes(own) ? best : own;
+}
+
 pf_status wgrad(const void* dy, int lddy, int dyoff, int cout, const void* x, int ldx, int xoff, int cin, float* dw, int n,
                 int d, int h, int wd, cudaStream_t st) {
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
@@ -1362,14 +1388,19 @@ pf_status wgrad(const void* dy, int lddy, int dyoff, int cout, const void* x, in
     WgArgs a{};
     a.cin = cin;
     a.cout = cout;
-    a.D = d;
-    a.H = h;
-    a.W = wd;
+    const WgAxes axes = wgrad_axes(n, d, h, wd);
+    const WgAxis &ax = axes.a[0], &ay = axes.a[1], &az = axes.a[2];
+    a.W = ax.n;
+    a.H = ay.n;
+    a.D = az.n;
+    a.tapx = ax.tap;
+    a.tapy = ay.tap;
+    a.tapz = az.tap;
     a.tries = WAIT_TRIES;
     a.dw = dw;
     wgrad_plan(a);
-    a.tx = (wd + 7) / 8;
-    a.ty = (h + 15) / 16;
+    a.tx = (a.W + 7) / 8;
+    a.ty = (a.H + 15) / 16;
     a.x_tx = 18u * (unsigned)a.nchunk * WX_ROW;
     a.dy_tx = 16u * 8u * 2u * (unsigned)cout;
     a.x_bytes = (a.x_tx + 127u) & ~127u;
@@ -1396,8 +1427,8 @@ pf_status wgrad(const void* dy, int lddy, int dyoff, int cout, const void* x, in
     // the prologue, the extra X planes and the epilogue)
     const long long columns = (long long)a.tx * a.ty * n * groups, cap = 152LL * occ;
     long long best = -1;
-    for (int nz = 1; nz <= d; nz += 1 + nz / 64) {
-        const int zc = (d + nz - 1) / nz, chunks = (d + zc - 1) / zc;
+    for (int nz = 1; nz <= a.D; nz += 1 + nz / 64) {
+        const int zc = (a.D + nz - 1) / nz, chunks = (a.D + zc - 1) / zc;
         const long long blocks = columns * chunks, cost = ((blocks + cap - 1) / cap + (blocks + 151) / 152) * (zc + 4);
         if (best < 0 || cost < best) {
             best = cost;
@@ -1409,8 +1440,8 @@ pf_status wgrad(const void* dy, int lddy, int dyoff, int cout, const void* x, in
     const cuuint32_t es[5] = {1, 1, 1, 1, 1};
     {
         const cuuint64_t row = (cuuint64_t)ldx * 2;
-        const cuuint64_t dims[5] = {8, (cuuint64_t)wd, (cuuint64_t)(cin / 8), (cuuint64_t)h, (cuuint64_t)n * d};
-        const cuuint64_t strides[4] = {row, 16, row * wd, row * wd * h};
+        const cuuint64_t dims[5] = {8, (cuuint64_t)a.W, (cuuint64_t)(cin / 8), (cuuint64_t)a.H, (cuuint64_t)n * a.D};
+        const cuuint64_t strides[4] = {row * ax.stride, 16, row * ay.stride, row * az.stride};
         const cuuint32_t box[5] = {8, 10, (cuuint32_t)a.nchunk, 18, 1};
         if (enc(&mX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)((const bf16*)x + xoff), dims, strides, box, es,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -1419,8 +1450,8 @@ pf_status wgrad(const void* dy, int lddy, int dyoff, int cout, const void* x, in
     }
     {
         const cuuint64_t row = (cuuint64_t)lddy * 2;
-        const cuuint64_t dims[5] = {8, (cuuint64_t)wd, (cuuint64_t)h, (cuuint64_t)(cout / 8), (cuuint64_t)n * d};
-        const cuuint64_t strides[4] = {row, row * wd, 16, row * wd * h};
+        const cuuint64_t dims[5] = {8, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)(cout / 8), (cuuint64_t)n * a.D};
+        const cuuint64_t strides[4] = {row * ax.stride, row * ay.stride, 16, row * az.stride};
         const cuuint32_t box[5] = {8, 8, 16, (cuuint32_t)(cout / 8), 1};
         if (enc(&mY, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)((const bf16*)dy + dyoff), dims, strides, box, es,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
