@@ -1289,19 +1289,15 @@ pf_status pf_get_tiles(pf_grid* g, int* by, int* zc) {
 
 static const int kTuneBY[3] = {4, 8, 16};
 // z chunks: powers of two plus the values between them that let small grids fill the SMs in about one
-// wave of blocks (a 50 x 50 x 100 grid in 32 x 4 columns: zc = 5 gives 520 blocks, zc = 4 gives 650)
-constexpr int NZC = 12;
-static const int kTuneZC[NZC] = {2, 3, 4, 5, 6, 8, 10, 12, 16, 24, 32, 64};
+// wave of blocks (a 50 x 50 x 100 grid in 25 x 5 columns: zc = 5 gives 400 blocks, zc = 4 gives 500)
+constexpr int NZC = 13;
+static const int kTuneZC[NZC] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 24, 32, 64};
 
-// Time the plain right-hand side (the stage kernels' common body) for every (by, zc) candidate on the
-// grid itself; ms[b][z] = best of 3 launches (infinity for skipped candidates).
-// Device time of one Merson attempt's five stage kernels for every tile shape (best of three after
-// a warm-up).  The controller is not launched: the state, the time and the step counters stay as
-// they are (stage 5 writes only the spare state buffer), and the control block is restored after.
-static pf_status tune_table(pf_grid* g, double ms[3][NZC]) {
+// The control block as the tuners' launches need it (a forced step of the current size, on every stage), and back.
+static pf_status tune_begin(pf_grid* g, Ctrl* saved) {
     pf_status s = sync_ctrl_to_host(g);
     if (s != PF_OK) return s;
-    const Ctrl saved = *g->hctrl;
+    *saved = *g->hctrl;
     Ctrl* c = g->hctrl;
     c->dt_step = c->dt;
     prepare_step(c);
@@ -1309,42 +1305,73 @@ static pf_status tune_table(pf_grid* g, double ms[3][NZC]) {
     c->status = 0;
     c->fixed = 1;
     c->single = 1;
-    s = push_ctrl(g);
+    return push_ctrl(g);
+}
+static pf_status tune_end(pf_grid* g, const Ctrl& saved) {
+    *g->hctrl = saved;
+    const pf_status s = push_ctrl(g);
+    if (s != PF_OK) return s;
+    PF_CUDA(g, cudaStreamSynchronize(g->stream));
+    return PF_OK;
+}
+
+// Device time of one Merson attempt's five stage kernels for every tile shape that a launch can cover (best of three after
+// a warm-up; infinity for the others).  The controller is not launched: the state, the time and the step counters stay as
+// they are (stage 5 writes only the spare state buffer), and the control block is restored after.  With `by` and `zc`, they
+// and `best` return the fastest shape, which is the grid's present one unless the other is faster in four more attempts
+// of each in turn: the least of 39 short times is a lucky one.
+static pf_status tune_table(pf_grid* g, double ms[3][NZC], int* by = nullptr, int* zc = nullptr, double* best = nullptr) {
+    Ctrl saved;
+    pf_status s = tune_begin(g, &saved);
     if (s != PF_OK) return s;
     cudaEvent_t e0, e1;
     PF_CUDA(g, cudaEventCreate(&e0));
     PF_CUDA(g, cudaEventCreate(&e1));
     cudaError_t e = cudaSuccess;
     const int by0 = g->by, zc0 = g->zc;
+    auto attempt = [&](int b, int z) {
+        g->by = b;
+        g->zc = z;
+        e = cudaEventRecord(e0, g->stream);
+        for (int st = 1; st <= 5 && e == cudaSuccess; ++st) e = launch_stage(g, st, g->stream);
+        if (e == cudaSuccess) e = cudaEventRecord(e1, g->stream);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        float t = 0.f;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
+        return (double)t;
+    };
+    int wb = by0, wz = zc0;
+    double w = INFINITY;
     for (int b = 0; b < 3; ++b)
         for (int z = 0; z < NZC; ++z) {
             ms[b][z] = INFINITY;
             if (e != cudaSuccess) continue;
-            if (kTuneZC[z] > 2 * g->n3 && z > 0) continue;
-            g->by = kTuneBY[b];
-            g->zc = kTuneZC[z];
-            double best = INFINITY;
+            if ((kTuneZC[z] > 2 * g->n3 && z > 0) || !tiles_fit(g, kTuneBY[b], kTuneZC[z])) continue;
+            double least = INFINITY;
             for (int r = 0; r < 4 && e == cudaSuccess; ++r) {
-                e = cudaEventRecord(e0, g->stream);
-                for (int st = 1; st <= 5 && e == cudaSuccess; ++st) e = launch_stage(g, st, g->stream);
-                if (e == cudaSuccess) e = cudaEventRecord(e1, g->stream);
-                if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-                float t = 0.f;
-                if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
-                if (r > 0 && t < best) best = t;  // first launch is a warm-up
+                const double t = attempt(kTuneBY[b], kTuneZC[z]);
+                if (r > 0 && t < least) least = t;  // first launch is a warm-up
             }
-            ms[b][z] = best;
+            ms[b][z] = least;
+            if (least < w) { w = least; wb = kTuneBY[b]; wz = kTuneZC[z]; }
         }
+    if (by && e == cudaSuccess) {
+        double t0 = INFINITY, t1 = INFINITY;
+        for (int r = 0; r < 5 && e == cudaSuccess; ++r) {
+            const double a = tiles_fit(g, by0, zc0) ? attempt(by0, zc0) : INFINITY, b = e == cudaSuccess ? attempt(wb, wz) : 0.0;
+            if (r > 0) { t0 = fmin(t0, a); t1 = fmin(t1, b); }
+        }
+        const bool other = t1 < t0;
+        *by = other ? wb : by0;
+        *zc = other ? wz : zc0;
+        *best = other ? t1 : t0;
+    }
     g->by = by0;
     g->zc = zc0;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (e != cudaSuccess) return fail(g, PF_E_CUDA, std::string("autotune: ") + cudaGetErrorString(e));
-    *g->hctrl = saved;
-    s = push_ctrl(g);
-    if (s != PF_OK) return s;
-    PF_CUDA(g, cudaStreamSynchronize(g->stream));
-    return PF_OK;
+    return tune_end(g, saved);
 }
 
 static std::string tune_key(const pf_grid* g) {
@@ -1383,11 +1410,8 @@ pf_status pf_autotune(pf_grid* g, const char* cache_path, int* by_out, int* zc_o
     const std::string key = tune_key(g);
     if (!cache_lookup(cache_path, key, &by, &zc, &best)) {
         double ms[3][NZC];
-        pf_status s = tune_table(g, ms);
+        pf_status s = tune_table(g, ms, &by, &zc, &best);
         if (s != PF_OK) return s;
-        for (int b = 0; b < 3; ++b)
-            for (int z = 0; z < NZC; ++z)
-                if (ms[b][z] < best) { best = ms[b][z]; by = kTuneBY[b]; zc = kTuneZC[z]; }
         cache_store(cache_path, key, by, zc, best);
     }
     pf_status s = set_tiles_impl(g, by, zc);
