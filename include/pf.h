@@ -209,7 +209,8 @@ typedef struct pf_batch_result {
 pf_status pf_batch_create(int n, pf_grid* const* grids, pf_batch** out);
 pf_status pf_batch_destroy(pf_batch* b);
 pf_grid* pf_batch_grid(pf_batch* b, int i);
-/* One block height for all instances (minimising the summed best times), then the best zc per instance. */
+/* One block height and chunk for all instances: the fastest of the shapes of pf_autotune on the batch's own kernels with all instances
+ * at once, or the present tiles if none is faster.  With a cache_path each instance's best tiles by itself are appended for pf_autotune. */
 pf_status pf_batch_autotune(pf_batch* b, const char* cache_path);
 pf_status pf_batch_run_to(pf_batch* b, const double* t_end, const double* eq_window, double eq_rel_tol,
                           const double* eq_rate, double tol, long long max_steps, pf_batch_result* res);

@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <algorithm>
 #include <array>
 #include <vector>
 
@@ -1434,6 +1435,7 @@ struct pf_batch {
     std::vector<StageArgs<double>> args64;
     Ctrl** d_ctrls = nullptr;
     int4* d_tiles = nullptr;
+    std::vector<int4> tiles;                // what d_tiles holds
     BatchPlan* d_plan = nullptr;
     cudaGraphExec_t exec = nullptr;
     long long iters = 0;
@@ -1459,15 +1461,15 @@ static void batch_free_graph(pf_batch* b) {
 
 // per-instance stage arguments and tile lattices on the device
 static pf_status batch_upload(pf_batch* b) {
-    std::vector<int4> tiles(b->n);
+    b->tiles.resize(b->n);
     for (int q = 0; q < b->n; ++q) {
         pf_grid* g = b->g[q];
         g->by = b->by;
         const TileShape ts = tile_shape(g->n1, g->n2, b->by);
         const int nbx = (g->n1 + ts.w - 1) / ts.w, nby = (g->n2 + ts.h - 1) / ts.h, nbz = (g->n3 + g->zc - 1) / g->zc;
-        tiles[q] = make_int4(nbx, nby, nbz, nbx * nby * nbz);
+        b->tiles[q] = make_int4(nbx, nby, nbz, nbx * nby * nbz);
     }
-    PF_BCUDA(b, cudaMemcpy(b->d_tiles, tiles.data(), sizeof(int4) * b->n, cudaMemcpyHostToDevice));
+    PF_BCUDA(b, cudaMemcpy(b->d_tiles, b->tiles.data(), sizeof(int4) * b->n, cudaMemcpyHostToDevice));
     if (b->prec == PF_PREC_FP32_FIELDS) {
         b->args32.resize(b->n);
         for (int q = 0; q < b->n; ++q) b->args32[q] = make_args<float>(b->g[q]);
@@ -1480,7 +1482,8 @@ static pf_status batch_upload(pf_batch* b) {
     return PF_OK;
 }
 
-static cudaError_t batch_enqueue_step(pf_batch* b, cudaStream_t s, int sms, cudaGraphConditionalHandle h) {
+// the five stage kernels over the listed instances' tiles
+static cudaError_t batch_enqueue_stages(pf_batch* b, cudaStream_t s, int sms) {
     cudaError_t e = cudaSuccess;
     for (int st = 1; st <= 5 && e == cudaSuccess; ++st) {
         if (b->prec == PF_PREC_FP32_FIELDS)
@@ -1490,6 +1493,18 @@ static cudaError_t batch_enqueue_step(pf_batch* b, cudaStream_t s, int sms, cuda
             e = launch_batch_stage_f64(b->model, b->rx, st, {b->args64.data(), (const StageArgs<double>*)b->d_args, b->n},
                                        b->d_plan, b->d_tiles, b->by, sms, s);
     }
+    return e;
+}
+
+static int multiprocessors() {
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
+static cudaError_t batch_enqueue_step(pf_batch* b, cudaStream_t s, int sms, cudaGraphConditionalHandle h) {
+    const cudaError_t e = batch_enqueue_stages(b, s, sms);
     if (e != cudaSuccess) return e;
     k_batch_controller<<<(b->n + BC_WARPS - 1) / BC_WARPS, 32 * BC_WARPS, 0, s>>>(b->d_ctrls, b->d_plan);
     k_batch_plan<<<1, BATCH_MAX, 0, s>>>(b->d_ctrls, b->d_tiles, b->n, b->d_plan, h);
@@ -1505,9 +1520,7 @@ static pf_status batch_build_graph(pf_batch* b) {
     PF_BCUDA(b, cudaGraphCreate(&graph, 0));
     cudaGraphConditionalHandle h;
     cudaError_t e = cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault);
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = multiprocessors();
     if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(b->cap, graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         k_batch_plan<<<1, BATCH_MAX, 0, b->cap>>>(b->d_ctrls, b->d_tiles, b->n, b->d_plan, h);
@@ -1630,32 +1643,136 @@ pf_status pf_batch_create(int n, pf_grid* const* grids, pf_batch** out) {
 
 pf_grid* pf_batch_grid(pf_batch* b, int i) { return (b && i >= 0 && i < b->n) ? b->g[i] : nullptr; }
 
+// Attempts of all instances with the batch's present tiles, in ms: `runs` graph launches of the five stage kernels after a
+// warm-up, the least.  The control blocks are prepared (tune_begin); nothing but scratch and spare buffers changes.
+static pf_status batch_attempt_ms(pf_batch* b, int runs, double* ms) {
+    BatchPlan plan = {};
+    plan.nactive = b->n;
+    for (int q = 0; q < b->n; ++q) {
+        plan.inst[q] = q;
+        plan.tile_start[q] = plan.ntiles;
+        plan.ntiles += b->tiles[q].w;
+    }
+    plan.tile_start[b->n] = plan.ntiles;
+    PF_BCUDA(b, cudaMemcpy(b->d_plan, &plan, sizeof(plan), cudaMemcpyHostToDevice));
+    const long long before = pfgb::g_launches.load();
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        cudaError_t e1 = cudaMemsetAsync(b->d_plan->next, 0, sizeof(plan.next), b->cap);
+        if (e1 == cudaSuccess) e1 = batch_enqueue_stages(b, b->cap, multiprocessors());
+        const cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);
+        e = e1 != cudaSuccess ? e1 : e2;
+    }
+    pfgb::g_launches.store(before);  // recorded, not executed
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
+    if (graph) cudaGraphDestroy(graph);
+    cudaEvent_t t0 = nullptr, t1 = nullptr;
+    if (e == cudaSuccess) e = cudaEventCreate(&t0);
+    if (e == cudaSuccess) e = cudaEventCreate(&t1);
+    *ms = INFINITY;
+    for (int r = 0; r <= runs && e == cudaSuccess; ++r) {
+        e = cudaEventRecord(t0, b->stream);
+        if (e == cudaSuccess) e = cudaGraphLaunch(exec, b->stream);
+        if (e == cudaSuccess) e = cudaEventRecord(t1, b->stream);
+        if (e == cudaSuccess) e = cudaEventSynchronize(t1);
+        float t = 0.f;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&t, t0, t1);
+        if (e == cudaSuccess) count_launch(5);
+        if (r > 0) *ms = fmin(*ms, t);
+    }
+    if (t0) cudaEventDestroy(t0);
+    if (t1) cudaEventDestroy(t1);
+    if (exec) cudaGraphExecDestroy(exec);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return bfail(b, PF_E_CUDA, std::string("batch autotune: ") + cudaGetErrorString(e));
+    }
+    return PF_OK;
+}
+
+// Tiles of all instances: blocks of `by` rows and, per instance, zc planes.
+struct BatchShape {
+    int by;
+    std::vector<int> zc;
+};
+static pf_status batch_set_shape(pf_batch* b, const BatchShape& t) {
+    b->by = t.by;
+    for (int q = 0; q < b->n; ++q) b->g[q]->zc = t.zc[q];
+    return batch_upload(b);
+}
+
+// Every block height with every chunk common to the instances, and the present tiles, on the batch's own kernels and all
+// instances at once: they share the chip, so an instance's best tiles by itself (which the tuner took before) leave it
+// too many short blocks (8 x 64^3 binary32 full model: by themselves 248 us an attempt, untuned 205).
+static pf_status batch_tune(pf_batch* b) {
+    BatchShape present{b->by, {}}, best;
+    int deepest = 1;
+    for (pf_grid* g : b->g) {
+        present.zc.push_back(g->zc);
+        deepest = std::max(deepest, g->n3);
+    }
+    best = present;
+    double least = INFINITY, ms = 0.0;
+    pf_status s = PF_OK;
+    for (int by : kTuneBY)
+        for (int zc : kTuneZC) {
+            if (s != PF_OK || (zc > 2 * deepest && zc > 1)) continue;
+            // (each instance can still be run by itself)
+            if (!std::all_of(b->g.begin(), b->g.end(), [&](pf_grid* g) { return tiles_fit(g, by, zc); })) continue;
+            const BatchShape t{by, std::vector<int>(b->n, zc)};
+            s = batch_set_shape(b, t);
+            if (s == PF_OK) s = batch_attempt_ms(b, 3, &ms);
+            if (s == PF_OK && ms < least) {
+                least = ms;
+                best = t;
+            }
+        }
+    // the present tiles unless the others are faster in turn, twice four attempts each
+    double old_ms = INFINITY, new_ms = INFINITY;
+    for (int r = 0; r < 2 && s == PF_OK; ++r) {
+        s = batch_set_shape(b, present);
+        if (s == PF_OK) s = batch_attempt_ms(b, 4, &ms);
+        old_ms = fmin(old_ms, ms);
+        if (s == PF_OK) s = batch_set_shape(b, best);
+        if (s == PF_OK) s = batch_attempt_ms(b, 4, &ms);
+        new_ms = fmin(new_ms, ms);
+    }
+    const pf_status s2 = batch_set_shape(b, s == PF_OK && new_ms < old_ms ? best : present);
+    return s != PF_OK ? s : s2;
+}
+
 pf_status pf_batch_autotune(pf_batch* b, const char* cache_path) {
     if (!b) return bfail(nullptr, PF_E_INVALID, "batch is NULL");
-    // a common block height for the batched kernels, then the best z chunk per instance
-    std::vector<std::array<std::array<double, NZC>, 3>> t(b->n);
-    double sum[3] = {0, 0, 0};
-    for (int q = 0; q < b->n; ++q) {
-        double ms[3][NZC];
-        pf_status s = tune_table(b->g[q], ms);
+    for (int q = 0; cache_path && q < b->n; ++q) {  // for pf_autotune: each instance's best tiles by itself
+        double ms[3][NZC], least = INFINITY;
+        int by = 0, zc = 0;
+        const pf_status s = tune_table(b->g[q], ms, &by, &zc, &least);
         if (s != PF_OK) return bfail(b, s, b->g[q]->err);
-        for (int bb = 0; bb < 3; ++bb) {
-            double m = INFINITY;
-            for (int z = 0; z < NZC; ++z) { t[q][bb][z] = ms[bb][z]; m = fmin(m, ms[bb][z]); }
-            sum[bb] += m;
+        cache_store(cache_path, tune_key(b->g[q]), by, zc, least);
+    }
+    std::vector<Ctrl> saved(b->n);
+    pf_status s = PF_OK;
+    int prepared = 0;
+    for (; prepared < b->n && s == PF_OK; ++prepared) {
+        s = tune_begin(b->g[prepared], &saved[prepared]);
+        if (s != PF_OK) {
+            bfail(b, s, b->g[prepared]->err);
+            break;
         }
+        cudaStreamSynchronize(b->g[prepared]->stream);
     }
-    int bb = 0;
-    for (int k = 1; k < 3; ++k) if (sum[k] < sum[bb]) bb = k;
-    b->by = kTuneBY[bb];
-    for (int q = 0; q < b->n; ++q) {
-        int z = 0;
-        for (int k = 1; k < NZC; ++k) if (t[q][bb][k] < t[q][bb][z]) z = k;
-        set_tiles_impl(b->g[q], b->by, kTuneZC[z]);
-        cache_store(cache_path, tune_key(b->g[q]), b->by, kTuneZC[z], t[q][bb][z]);
-    }
+    if (s == PF_OK) s = batch_tune(b);
     batch_free_graph(b);
-    return batch_upload(b);
+    for (int q = 0; q < prepared; ++q) {
+        pf_grid* g = b->g[q];
+        const pf_status s2 = tune_end(g, saved[q]);
+        if (s == PF_OK && s2 != PF_OK) s = bfail(b, s2, g->err);
+        free_graph(g);
+        g->tiles_set = true;
+    }
+    return s;
 }
 
 pf_status pf_batch_run_to(pf_batch* b, const double* t_end, const double* eq_window, double eq_rel_tol,
