@@ -569,7 +569,7 @@ static void default_tiles(const pf_grid* g, double share, int only_by, int* by, 
     const double z = (is_f32(g) ? 2.2 : 0.8) * std::sqrt(lateral * g->n3 / places);
     *zc = z < 1.5 ? 1 : (z > 24.0 ? 24 : (int)(z + 0.5));
     if (g->n3 <= 2 && lateral > 0.5 * places) *zc = g->n3;
-    if (g->n3 <= 2 && lateral > 3.0 * places) *by = 8;
+    if (g->n3 <= 2 && lateral > 2.0 * places) *by = 8;
     while (*by < 16 && !tiles_fit(g, *by, longest)) *by *= 2;
     if (only_by) *by = only_by;
     if (*zc < longest) *zc = longest;

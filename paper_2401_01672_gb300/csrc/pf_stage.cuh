@@ -963,10 +963,10 @@ stage_kernel_r128(const StageArgs<T> a) {
     stage_tile<MODEL, RX, T, TIN, STAGE, BY, true>(a, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
-// Batched persistent form: as many blocks as fit the chip take the tiles of the instances listed in the plan (instances
+// Batched persistent form: as many blocks as fit the chip, or somewhat more (batch_launch), take the tiles of the instances listed in the plan (instances
 // that are finished are not listed), the first one each by number, then the next from a counter that k_batch_plan zeroes;
 // a block asks for its next tile before it starts one, so the answer is there when it needs it.  (With a stride of the
-// grid, and a third more blocks than fit, one 128^3 instance in binary64 took 9.1 ms for 24 attempts; see batch_one.)
+// grid, and a third more blocks than fit, one 128^3 instance in binary64 took 9.1 ms for 24 attempts, now 7.2.)
 // `args`: the instances' stage arguments, in the kernel's parameters (constant bank, as for a single grid) where they
 // fit, else in global memory, where every use of a pointer or coefficient is a load or a register (12 binary32 instances, 16 attempts: 24.0 and 20.4 ms).
 template <int MODEL, int RX, typename T, typename TIN, int STAGE, int BY, typename ARGS>
@@ -1046,34 +1046,47 @@ cudaError_t launch_by(int stage, const StageArgs<T>& a, cudaStream_t s) {
     return e;
 }
 
-// one block for every place on the chip (occupancy of this kernel); `sms` multiprocessors
+// One block for every place on the chip (occupancy of this kernel; `sms` multiprocessors), or, with up to `most` times as many
+// tiles, one for every tile: resident blocks that end together take the tiles left over on the same few multiprocessors,
+// where blocks that the hardware places spread over all (4 x 64^3 in 32 x 4 x 9 tiles, 1.12 tiles a place: binary64 full 1309 us an
+// attempt and 733, binary32 full 144 and 126, binary64 Temp 2677 and 1530).  With more tiles a block saves the launch of the
+// next ones: binary32 full 134 and 138 us at 2.2 to 2.7 tiles a place, 962 and 1013 at 20; in binary64, whose tiles are
+// longer, that pays from about 4 (64^3 Temp 1669 and 1508 us at 2.25; flat grids 462 and 442 at 2.5).
 template <typename ARGS>
 void batch_launch(void (*k)(ARGS, BatchPlan*, const int4*), const ARGS& args, int threads_y, BatchPlan* plan, const int4* tg,
-                  int sms, cudaStream_t s) {
+                  int sms, cudaStream_t s, long long tiles, int most) {
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, TX * threads_y, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
-    k<<<sms * per_sm, dim3(TX, threads_y), 0, s>>>(args, plan, tg);
+    const long long places = (long long)sms * per_sm;
+    const long long grid = tiles > places && tiles <= most * places ? tiles : places;
+    k<<<(unsigned)grid, dim3(TX, threads_y), 0, s>>>(args, plan, tg);
 }
 template <typename T, int MODEL, int RX, int STAGE, int BY>
 void batch_one(const BatchArgs<T>& args, BatchPlan* plan, const int4* tg, int sms, cudaStream_t s) {
     using TIN = typename std::conditional<STAGE == 1 && !(std::is_same<T, float>::value && MODEL == M_FULL), double,
                                           T>::type;
     constexpr bool BOUND = std::is_same<T, double>::value;
+    constexpr int MOST = BOUND && BY <= 8 ? 4 : 2;
+    long long tiles = 0;
+    for (int q = 0; q < args.n; ++q) {
+        const StageArgs<T>& a = args.host[q];
+        tiles += (long long)((a.cf.n1 + a.tw - 1) / a.tw) * ((a.cf.n2 + a.th - 1) / a.th) * ((a.cf.n3 + a.zc - 1) / a.zc);
+    }
     if (args.n <= BATCH_PARAMS) {
         BatchParams<T> p;
         for (int q = 0; q < args.n; ++q) p.a[q] = args.host[q];
         for (int q = args.n; q < BATCH_PARAMS; ++q) p.a[q] = args.host[0];
         using P = BatchParams<T>;
         if constexpr (BOUND)
-            batch_launch<P>(batch_param_kernel_r128<MODEL, RX, T, TIN, STAGE, BY>, p, BY, plan, tg, sms, s);
+            batch_launch<P>(batch_param_kernel_r128<MODEL, RX, T, TIN, STAGE, BY>, p, BY, plan, tg, sms, s, tiles, MOST);
         else
-            batch_launch<P>(batch_param_kernel<MODEL, RX, T, TIN, STAGE, BY>, p, BY, plan, tg, sms, s);
+            batch_launch<P>(batch_param_kernel<MODEL, RX, T, TIN, STAGE, BY>, p, BY, plan, tg, sms, s, tiles, MOST);
     } else {
         using P = const StageArgs<T>*;
         if constexpr (BOUND)
-            batch_launch<P>(batch_stage_kernel_r128<MODEL, RX, T, TIN, STAGE, BY>, args.device, BY, plan, tg, sms, s);
+            batch_launch<P>(batch_stage_kernel_r128<MODEL, RX, T, TIN, STAGE, BY>, args.device, BY, plan, tg, sms, s, tiles, MOST);
         else
-            batch_launch<P>(batch_stage_kernel<MODEL, RX, T, TIN, STAGE, BY>, args.device, BY, plan, tg, sms, s);
+            batch_launch<P>(batch_stage_kernel<MODEL, RX, T, TIN, STAGE, BY>, args.device, BY, plan, tg, sms, s, tiles, MOST);
     }
 }
 

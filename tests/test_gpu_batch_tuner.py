@@ -11,7 +11,7 @@ from test_gpu_tiles import pf, state  # noqa: F401  (pf is a fixture)
 pytestmark = pytest.mark.gpu
 
 
-def batch(pf, shapes, model, prec, stream):  # noqa: F811
+def batch(pf, shapes, model, prec, stream, tiles=None):  # noqa: F811
     grids, init = [], []
     for q, shape in enumerate(shapes):
         th, ph, G = I.random_fields(shape, q)
@@ -19,6 +19,8 @@ def batch(pf, shapes, model, prec, stream):  # noqa: F811
                              theta_freeze=-5.0, theta_thaw=2.0, theta_micro=-0.5)
         g = pf.Grid(shape, 3e-4, model, I.REACT_SIGMAP1P, prec, p, stream=stream)
         g.set_glass(G)
+        if tiles:
+            g.set_tiles(*tiles)
         init.append((None if model == I.MODEL_MICRO else th, None if model == I.MODEL_TEMP else ph))
         g.set_state(*init[-1], 0.0, 1e-5)
         grids.append(g)
