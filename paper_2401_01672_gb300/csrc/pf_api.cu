@@ -527,9 +527,10 @@ static double lateral_tiles(const pf_grid* g, int by) {
 // The Temp model in binary64 is bound by the tanh of every cell that a block loads, its halo and its chunk's two extra planes
 // included, so both block heights and long chunks pay, as far as the blocks still spread over the chip: the fewest cells
 // loaded by a multiprocessor's share of the blocks and one more (the last ones do not end together; temperatures near the
-// melting point in one part of the grid make some blocks longer).  Measured at 22 grids of 16^3 to 192^3 and flat ones,
-// with temperatures near the melting point everywhere and in a front only: within 21 % of the best of 39 shapes, never more
-// than 2 % slower than 8 x 32.  128^3, near everywhere: 2.37 ms an attempt (3.65 with the rule below, 2.50 with 8 x 32).
+// melting point in one part of the grid make some blocks longer), a quarter more again where they do not all fit at once and the
+// last ones start late.  Measured at 36 grids of 16^3 to 256^3, slabs and flat ones, with temperatures near the melting point
+// everywhere and in a front only: within 29 % of the best of 39 shapes, 5 % on average, never more than 2 % slower than 8 x 32.
+// 128^3, near everywhere: 2.37 ms an attempt (3.65 with the rule below, 2.50 with 8 x 32).
 static const int kTempZC[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 24, 32};
 static bool temp_tiles(const pf_grid* g, double share, int only_by, int* by, int* zc) {
     double best = INFINITY;
@@ -540,7 +541,8 @@ static bool temp_tiles(const pf_grid* g, double share, int only_by, int* by, int
             if ((z > 1 && z > 2 * g->n3) || !tiles_fit(g, b, z)) continue;
             const double blocks = share * lateral_tiles(g, b) * ((g->n3 + z - 1) / z);
             const int planes = std::min(z, g->n3);
-            const double cost = (std::ceil(blocks / 152.0) + 1.0) * ((planes + 3.0) * ts.w * ts.h + (planes + 2.0) * 2.0 * (ts.w + ts.h));
+            const double spare = blocks > 152.0 * (b <= 8 ? 24 / b : 1) ? 1.25 : 1.0;  // (f64_min_blocks)
+            const double cost = (std::ceil(blocks / 152.0) + spare) * ((planes + 3.0) * ts.w * ts.h + (planes + 2.0) * 2.0 * (ts.w + ts.h));
             if (cost < best) {
                 best = cost;
                 *by = b;

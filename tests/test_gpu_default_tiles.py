@@ -23,7 +23,7 @@ def attempt(g):
 
 @pytest.mark.parametrize("model,prec,shape", [
     (I.MODEL_TEMP, I.PREC_FP64, (128, 128, 128)), (I.MODEL_TEMP, I.PREC_FP64, (160, 160, 160)),
-    (I.MODEL_TEMP, I.PREC_FP64, (300, 300, 4)), (I.MODEL_TEMP, I.PREC_FP64, (17, 2000, 5)),
+    (I.MODEL_TEMP, I.PREC_FP64, (128, 128, 64)), (I.MODEL_TEMP, I.PREC_FP64, (300, 300, 4)), (I.MODEL_TEMP, I.PREC_FP64, (17, 2000, 5)),
     (I.MODEL_TEMP, I.PREC_FP64, (50, 50, 100)), (I.MODEL_TEMP, I.PREC_FP32, (100, 100, 100)),
     (I.MODEL_MICRO, I.PREC_FP64, (300, 300, 2)), (I.MODEL_MICRO, I.PREC_FP32, (1000, 1000, 1)),
     (I.MODEL_FULL, I.PREC_FP64, (700, 700, 2)), (I.MODEL_MICRO, I.PREC_FP64, (64, 64, 64))])
