@@ -1354,6 +1354,7 @@ static pf_status tune_table(pf_grid* g, double ms[3][NZC], int* by = nullptr, in
             for (int r = 0; r < 4 && e == cudaSuccess; ++r) {
                 const double t = attempt(kTuneBY[b], kTuneZC[z]);
                 if (r > 0 && t < least) least = t;  // first launch is a warm-up
+                if (t > (r ? 1.5 : 3.0) * w) break;  // clearly slower than the best so far
             }
             ms[b][z] = least;
             if (least < w) { w = least; wb = kTuneBY[b]; wz = kTuneZC[z]; }
@@ -1646,8 +1647,9 @@ pf_status pf_batch_create(int n, pf_grid* const* grids, pf_batch** out) {
 pf_grid* pf_batch_grid(pf_batch* b, int i) { return (b && i >= 0 && i < b->n) ? b->g[i] : nullptr; }
 
 // Attempts of all instances with the batch's present tiles, in ms: `runs` graph launches of the five stage kernels after a
-// warm-up, the least.  The control blocks are prepared (tune_begin); nothing but scratch and spare buffers changes.
-static pf_status batch_attempt_ms(pf_batch* b, int runs, double* ms) {
+// warm-up, the least, fewer once one takes 1.5 times `limit` (the warm-up three times).  The control blocks are prepared
+// (tune_begin); nothing but scratch and spare buffers changes.
+static pf_status batch_attempt_ms(pf_batch* b, int runs, double limit, double* ms) {
     BatchPlan plan = {};
     plan.nactive = b->n;
     for (int q = 0; q < b->n; ++q) {
@@ -1683,6 +1685,7 @@ static pf_status batch_attempt_ms(pf_batch* b, int runs, double* ms) {
         if (e == cudaSuccess) e = cudaEventElapsedTime(&t, t0, t1);
         if (e == cudaSuccess) count_launch(5);
         if (r > 0) *ms = fmin(*ms, t);
+        if (t > (r ? 1.5 : 3.0) * limit) break;
     }
     if (t0) cudaEventDestroy(t0);
     if (t1) cudaEventDestroy(t1);
@@ -1725,7 +1728,7 @@ static pf_status batch_tune(pf_batch* b) {
             if (!std::all_of(b->g.begin(), b->g.end(), [&](pf_grid* g) { return tiles_fit(g, by, zc); })) continue;
             const BatchShape t{by, std::vector<int>(b->n, zc)};
             s = batch_set_shape(b, t);
-            if (s == PF_OK) s = batch_attempt_ms(b, 3, &ms);
+            if (s == PF_OK) s = batch_attempt_ms(b, 3, least, &ms);
             if (s == PF_OK && ms < least) {
                 least = ms;
                 best = t;
@@ -1735,10 +1738,10 @@ static pf_status batch_tune(pf_batch* b) {
     double old_ms = INFINITY, new_ms = INFINITY;
     for (int r = 0; r < 2 && s == PF_OK; ++r) {
         s = batch_set_shape(b, present);
-        if (s == PF_OK) s = batch_attempt_ms(b, 4, &ms);
+        if (s == PF_OK) s = batch_attempt_ms(b, 4, INFINITY, &ms);
         old_ms = fmin(old_ms, ms);
         if (s == PF_OK) s = batch_set_shape(b, best);
-        if (s == PF_OK) s = batch_attempt_ms(b, 4, &ms);
+        if (s == PF_OK) s = batch_attempt_ms(b, 4, INFINITY, &ms);
         new_ms = fmin(new_ms, ms);
     }
     const pf_status s2 = batch_set_shape(b, s == PF_OK && new_ms < old_ms ? best : present);
