@@ -1659,7 +1659,6 @@ static pf_status batch_attempt_ms(pf_batch* b, int runs, double limit, double* m
     }
     plan.tile_start[b->n] = plan.ntiles;
     PF_BCUDA(b, cudaMemcpy(b->d_plan, &plan, sizeof(plan), cudaMemcpyHostToDevice));
-    const long long before = pfgb::g_launches.load();
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
@@ -1669,7 +1668,7 @@ static pf_status batch_attempt_ms(pf_batch* b, int runs, double limit, double* m
         const cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);
         e = e1 != cudaSuccess ? e1 : e2;
     }
-    pfgb::g_launches.store(before);  // recorded, not executed
+    if (e == cudaSuccess) count_launch(-5);  // recorded, not executed
     if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
     if (graph) cudaGraphDestroy(graph);
     cudaEvent_t t0 = nullptr, t1 = nullptr;
