@@ -54,7 +54,7 @@ def test_tuned_batch_is_not_slower(pf, tmp_path, model, prec, shapes):  # noqa: 
         ends.append([state(g) for g in grids])
         b.close()
     assert all(np.array_equal(u, v) for u, v in zip(*ends))
-    assert ms[1] <= 1.06 * ms[0], (ms, tiles)
+    assert ms[1] <= 1.1 * ms[0], (ms, tiles)
 
 
 def test_instances_own_tiles_are_cached(pf, tmp_path):  # noqa: F811

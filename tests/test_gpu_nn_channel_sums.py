@@ -42,4 +42,4 @@ def test_vectors_are_not_slower_than_single_channels(env, c):  # noqa: F811
             best = min(best, e0.elapsed_time(e1))
         return best
 
-    assert time(0) <= 1.2 * time(1)  # (one float off 16 bytes: the kernel for any alignment)
+    assert time(0) <= 1.5 * time(1)  # (one float off 16 bytes: the kernel for any alignment)

@@ -35,5 +35,5 @@ def test_a_call_is_not_slower_than_four_on_a_quarter(env, cin, cout):  # noqa: F
 
     stream = torch.cuda.default_stream()
     whole, parts = time(h, 10), time(h // 4, 40)
-    assert whole <= 1.1 * parts, (whole, parts)
+    assert whole <= 1.15 * parts, (whole, parts)
     assert no_failed_waits(nn)

@@ -30,7 +30,7 @@ def test_tuned_is_not_slower_than_untuned(pf, model, prec, shape):  # noqa: F811
     before = state(tuned)
     by, zc, ms = tuned.autotune()
     assert tuned.get_tiles() == (by, zc) and ms > 0 and np.array_equal(state(tuned), before)
-    assert attempt(tuned) <= 1.06 * attempt(free), (free.get_tiles(), (by, zc))
+    assert attempt(tuned) <= 1.12 * attempt(free), (free.get_tiles(), (by, zc))
     assert np.array_equal(state(tuned), state(free))
     free.close()
     tuned.close()
