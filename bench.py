@@ -57,12 +57,11 @@ FLOPS_RHS = 64
 FLOPS_COMB = [4, 6, 8, 12, 24]
 # DRAM traffic per cell of the stage-5 kernels from one ncu capture each at 192^3, mid-front state
 # (dram__bytes_read.sum + dram__bytes_write.sum over 7,077,888 cells; None once a kernel changes until
-# it is captured again).  Binary64: 1072.2 MB -- the method's 104 B plus the per-cell blend
+# it is captured again).  Binary64: 1070.5 MB -- the method's 104 B plus the per-cell blend
 # coefficients (64 B where the Allen-Cahn arithmetic runs, 24 B in the bulk), read instead of
-# recomputed on the binary64 pipe that bounds it.  Binary32 form: not captured since stage 5 forms its input
-# from the slopes.
-TRAFFIC_F64_S5_PER_CELL = 151.5
-TRAFFIC_F32_S5_PER_CELL = None
+# recomputed on the binary64 pipe that bounds it.  Binary32 form: 529.5 MB, the method's 76 B.
+TRAFFIC_F64_S5_PER_CELL = 151.2
+TRAFFIC_F32_S5_PER_CELL = 74.8
 KERNEL_BYTES_F64_S5 = None
 
 
@@ -560,6 +559,18 @@ CONV_LAYERS = [("infer_l0_256", 1, 256, 16, 16), ("infer_l1_128", 1, 128, 32, 32
                ("infer_l3_32", 1, 32, 128, 128), ("train_l2_32x8", 8, 32, 128, 64), ("train_l0_64x8", 8, 64, 32, 16)]
 
 
+def conv_kernel(n, side, cin, cout):
+    """The kernel that a layer takes on n cubes of side^3 voxels (march_shape and wide_shape of the library)."""
+    if cin in (16, 32, 64) and cout in (16, 32, 64) and cin * cout <= 2048 and side >= 16:
+        return "k_conv_march"
+    bricks = -(-side // 32) * -(-side // 4) * side if side >= 32 else -(-side // 16) * -(-side // 8) * side
+    planes = n * side * (-(-side // 16)) ** 2
+    if cin % 32 == 0 and cout in (16, 32, 64) and cin * cout > 2048 and cin // (64 if cin % 64 == 0 else 32) <= 3 and \
+            side >= 16 and planes >= 500 and 256 * planes <= 1.4 * 128 * bricks * n:
+        return "k_conv_wide"
+    return "k_conv_umma"
+
+
 def run_conv(args, rank, world):
     """Forward 3x3x3 convolutions of the warm-start network on the tensor cores (tcgen05, TMA operands,
     TMEM accumulators), bf16 in and out, fp32 accumulation: device time per layer with CUDA events on
@@ -595,11 +606,9 @@ def run_conv(args, rank, world):
             ms = e0.elapsed_time(e1) / reps
             tf = 2.0 * 27 * cin * cout * nv / (ms * 1e-3) / 1e12
             io_gbs = nv * (cin + cout) * 2 / (ms * 1e-3) / 1e9
-            march = cin in (16, 32, 64) and cout in (16, 32, 64) and cin * cout <= 2048 and side >= 16
-            wide = cin * cout > 2048 and side >= 16 and n * side * (-(-side // 16)) ** 2 * max(1, cout // 64) >= 500
             out[label] = {"samples": n, "side": side, "cin": cin, "cout": cout, "ms": ms, "tflops": tf,
                           "frac_of_bf16_peak": tf / peaks["bf16_tflops"],
-                          "kernel": "k_conv_march" if march else ("k_conv_wide" if wide else "k_conv_umma"),
+                          "kernel": conv_kernel(n, side, cin, cout),
                           "io_gbs": io_gbs, "frac_of_hbm": io_gbs / peaks["hbm_gbs"]}
         nn.check_device()
     top = max(out, key=lambda k: out[k]["tflops"])

@@ -8,8 +8,8 @@ namespace pfgb {
 enum { M_FULL = 0, M_TEMP = 1, M_MICRO = 2 };
 enum { R_SIGMA = 0, R_GRADP = 1 };
 
-// Tile of a stage kernel: one warp spans 32 cells along x, BY warps span y,
-// each thread marches along z over a chunk of ZC planes.
+// Block of a stage kernel: 32 x BY threads over a lateral tile of 32 x BY cells or of another shape with no more cells
+// (tile_shape); each thread marches along z over a chunk of planes.
 constexpr int TX = 32;
 
 // per-cell coefficient arrays of the binary64 full model (see StageArgs::statics)

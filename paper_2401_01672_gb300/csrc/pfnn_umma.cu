@@ -425,7 +425,7 @@ __device__ __forceinline__ void tmem_zero(uint32_t taddr, int cols) {
 // l = 3 (dy + 1) + (dx + 1); flipped: the tap 26 - t), in rounds of 7 16-byte vectors per thread: each
 // round loads all of its vectors (read-only path) before storing them, so the copy costs one round trip
 // to L2 per 14 KB (one for 16 x 16 channels, four for 32 x 32).
-__device__ __forceinline__ void halo_weights(const bf16* __restrict__ w, unsigned char* dst, int cout, int nkc,
+__device__ __forceinline__ void march_weights(const bf16* __restrict__ w, unsigned char* dst, int cout, int nkc,
                                              int flip) {
     constexpr int CAP = 7;
     const int nvec = 27 * cout * nkc;
@@ -516,7 +516,7 @@ k_conv_march(const __grid_constant__ CUtensorMap tmX, const MarchArgs p) {
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    halo_weights(p.w, sm + (size_t)p.slots * p.plane_bytes, p.cout, CK / 8, p.flip);
+    march_weights(p.w, sm + (size_t)p.slots * p.plane_bytes, p.cout, CK / 8, p.flip);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
